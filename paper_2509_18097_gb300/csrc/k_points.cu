@@ -40,7 +40,7 @@ __global__ void k_plan(Plan* P) {
     cnt[ST_NNQ][j] = J->Q + nrs * J->M;
     cnt[ST_E][j] = J->E;
     cnt[ST_MOVCH][j] = (2 * G * G * G + SCAN_CHUNK - 1) / SCAN_CHUNK;
-    int a = 0, t = 0, p3 = 0, cols = 0, ad = 0;
+    int a = 0, t = 0, xt = 0, p3 = 0, cols = 0, ad = 0;
     int aw = 0;
     // the levels' loads are independent: issue them level-parallel (a dependent chain of
     // global loads per level would put a dozen memory latencies on the step's critical path)
@@ -66,8 +66,10 @@ __global__ void k_plan(Plan* P) {
       lv.adj_lg = lg;
       if (lg == 6) a += na;
       else aw += (na + (32 >> lg) - 1) >> (5 - lg);
-      if (tile_level(J->lev[l].n)) t += J->lev[l].tiles;
-      else {
+      if (tile_level(J->lev[l].n)) {
+        t += J->C * yz_tiles(J->lev[l].n);
+        xt += J->C / 3 * x_tiles(J->lev[l].n);
+      } else {
         p3 += J->lev[l].n;
         cols += J->C * ((J->lev[l].n * J->lev[l].n + 63) / 64);  // blocks of 64 columns (two threads each)
         ad += (J->lev[l].n3 + 3) >> 2;
@@ -75,6 +77,7 @@ __global__ void k_plan(Plan* P) {
     }
     cnt[ST_ADJ][j] = a + ((aw + 7) >> 3);
     cnt[ST_TILE][j] = t;
+    cnt[ST_XTILE][j] = xt;
     cnt[ST_PLANE][j] = J->C * p3;
     cnt[ST_COL][j] = cols;
     cnt[ST_ADAM][j] = ad;

@@ -723,9 +723,9 @@ __global__ void __launch_bounds__(256) k_adam(const Plan* __restrict__ P) {
 __global__ void k_zmask(Job* __restrict__ Jp, int l) {
   const Level& lv = Jp->lev[l];
   const int na = *lv.n_active;
-  const int sh = 2 * lv.lg;
+  const int n2 = lv.n * lv.n;
   for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < na; i += gridDim.x * blockDim.x)
-    lv.zmask[lv.act_v[i] >> sh] = 1;
+    lv.zmask[lv.act_v[i] / n2] = 1;
 }
 
 void launch_zmask(Job* J, const Job& hJ, cudaStream_t s) {

@@ -1,5 +1,7 @@
 // Host-side launchers of the libpdg kernels (each defined next to its kernels).
 #pragma once
+#include <algorithm>
+
 #include "pdg_internal.cuh"
 
 namespace pdg {
@@ -15,7 +17,10 @@ void launch_nn_hard(const Plan* P, int grid, cudaStream_t s, bool count);
 void launch_iso_edges(const Plan* P, int grid, cudaStream_t s);
 void launch_assemble(const Plan* P, int grid, cudaStream_t s);
 void launch_adjoint(const Plan* P, int grid, cudaStream_t s);
-void launch_sobolev_tiles(const Plan* P, int sms, int nlo, int nhi, int nsmem, cudaStream_t s);
+// line path (256 and sizes with a factor 3); nmax: the largest level it takes in the plan
+enum YzPass { YZ_FWD = 0, YZ_Z, YZ_INV };
+void launch_sobolev_x(const Plan* P, int sms, int nmax, bool fwd, cudaStream_t s);
+void launch_sobolev_yz(const Plan* P, int sms, int nmax, int pass, cudaStream_t s);
 void launch_sobolev_plane(const Plan* P, int grid, int nmax, cudaStream_t s, int part = -1);
 void launch_loss(const Plan* P, int grid, cudaStream_t s);
 
@@ -39,8 +44,8 @@ struct ScanSeg {
 void launch_scan_segments(const ScanSeg* hsegs, int nseg, ScanSeg* dsegs_scratch, int* dpre_scratch,
                           cudaStream_t s);
 
-int sobolev_smem_bytes(int n);
-void sobolev_configure();
+void sobolev_x_configure();
+void sobolev_yz_configure();
 void sobolev_plane_configure();
 int plane_smem_bytes(int n);
 int plane_smem_max(int nmax);

@@ -13,9 +13,6 @@ constexpr int MAXJ = 256;            // jobs (contexts) per batch
 constexpr int MAXL = PDG_MAX_LEVELS; // grid levels
 constexpr int SCAN_CHUNK = 4096;     // elements per scan chunk (1024 threads x 4)
 constexpr int SCAN_THREADS = 1024;
-constexpr int TILE_LINES = 32;       // lines per Sobolev tile (per channel)
-constexpr int SOB_WARPS = 8;
-constexpr int SOB_THREADS = SOB_WARPS * 32;
 constexpr int NN_RMAX = 8;           // ring radius after which a query is searched exhaustively
 constexpr int NN_RTHREAD = 2;        // rings searched by the one-thread-per-query pass
 constexpr int LOSS_CHUNK = 2048;     // elements per loss-reduction chunk
@@ -42,7 +39,6 @@ struct Level {
   int n;       // vertices per axis (1 or a power of two)
   int lg;      // log2(n)
   int n3;      // n^3
-  int tiles;   // tile-path Sobolev tiles: 3 channels x ceil(n^2 / 32) lines of 32
   float sc_hi[3], sc_lo[3];  // (n - 1) / (hi - lo) per axis as a float pair (hi + lo)
   float lr;    // learning rate of the level (already x0.1 without preconditioning)
   float lam;   // lambda of the level
@@ -57,6 +53,7 @@ struct Level {
   int* piv_slow;  // device flag: some pivot past the first 16 differs from the limit (no register path)
   float* mu;      // [n] eigenvalues 4 sin^2(pi k / 2n) of the 1-D path Laplacian
   float2* tw;     // [n] FFT twiddles exp(-2 pi i k / n)
+  float2* twm;    // [n] line path: twm[k N1 + t] = exp(-2 pi i t k / n) (N1 = line_n1(n))
   float2* tw4;    // [n] DCT twiddles exp(-i pi k / 2n)
   // point -> vertex interpolation lists, built once per frame (x is fixed in a frame)
   int* cnt;       // [n3] per-vertex entry counts (zero between builds)
@@ -120,12 +117,14 @@ struct Job {
   unsigned long long* counters;  // [4] of the last step: NN candidates evaluated (counted only
                                  // when count_nn), NN queries decided by an exact tie,
                                  // queries left to the warp pass, reserved
+  const float* ext_in;     // pdg_precondition on a line-path level: the caller's gradient [n^3][3] ...
+  float* ext_out;          // ... and where its preconditioned form goes (null in a step)
   int count_nn;            // 1: k_nn / k_nn_hard add their candidate counts to counters[0]
 };
 
 enum Counter { CNT_NN_CANDIDATES = 0, CNT_NN_TIES = 1, CNT_NN_HARD = 2 };
 
-enum Stage { ST_Q = 0, ST_NNQ, ST_E, ST_MOVCH, ST_ADJ, ST_TILE, ST_JOB, ST_LOSSCH, ST_PLANE, ST_COL, ST_ADAM, NSTAGE };
+enum Stage { ST_Q = 0, ST_NNQ, ST_E, ST_MOVCH, ST_ADJ, ST_TILE, ST_JOB, ST_LOSSCH, ST_PLANE, ST_COL, ST_ADAM, ST_XTILE, NSTAGE };
 
 struct Plan {
   int n_jobs;
@@ -138,8 +137,41 @@ struct Plan {
 
 // Which preconditioner path takes a level of n vertices per axis: powers of two up to 128
 // (and n = 1) take the shared-memory plane path, 256 and the sizes with a factor 3 the
-// tile path with mixed radix-2/3 line transforms.
+// line path.
 __host__ __device__ __forceinline__ bool tile_level(int n) { return n > 128 || (n & (n - 1)) != 0; }
+
+// Line path: sizes, line pairs of a y or z tile, x-lines (per channel) of an x tile.  A stage
+// has about sqrt(n) work items per pair, so short lines go into larger tiles to fill a block.
+#define PDG_LINE_SIZES(X)                                                                                    \
+  X(3) X(6) X(9) X(12) X(18) X(24) X(27) X(36) X(48) X(54) X(72) X(81) X(96) X(108) X(144) X(162) X(192) \
+  X(216) X(243) X(256)
+// n = N1 x N2 with N1 <= N2, as even as the radices allow: the register DFTs of a line stay at
+// 16 points or fewer, but for 162, 216 (18) and 243 (27)
+__host__ __device__ constexpr int line_n1(int n) {
+  return n <= 6      ? 1
+         : n == 8    ? 2
+         : n <= 12   ? 3
+         : n == 16   ? 4
+         : n == 18   ? 3
+         : n == 24   ? 4
+         : n == 27   ? 3
+         : n == 32   ? 4
+         : n <= 54   ? 6
+         : n <= 72   ? 8
+         : n == 81   ? 9
+         : n == 96   ? 8
+         : n == 108  ? 9
+         : n == 128  ? 8
+         : n == 144  ? 12
+         : n == 162  ? 9
+         : n <= 216  ? 12
+         : n == 243  ? 9
+                     : 16;
+}
+__host__ __device__ constexpr int yz_pairs(int n) { return n >= 144 ? 16 : n >= 32 ? 32 : 64; }
+__host__ __device__ constexpr int x_lines(int n) { return n >= 64 ? 16 : n >= 24 ? 32 : 64; }
+__host__ __device__ constexpr int yz_tiles(int n) { return (n * n + 2 * yz_pairs(n) - 1) / (2 * yz_pairs(n)); }
+__host__ __device__ constexpr int x_tiles(int n) { return (n * n + x_lines(n) - 1) / x_lines(n); }
 
 __device__ __forceinline__ int find_job(const int* pre, int n_jobs, int item) {
   int lo = 0, hi = n_jobs;

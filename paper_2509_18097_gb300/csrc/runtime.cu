@@ -36,25 +36,8 @@ int grid_bits(long count, double per_cell = 8.0) {
   return std::min(std::max(b, 2), 7);
 }
 
-// Largest resolution of the levels the tile path preconditions, per size class (0: none).
-// Each class is launched with its own shared-memory size, so that small tile levels keep
-// several blocks per SM when a level above TILE_SPLIT shares the step (a batch).
-constexpr int TILE_SPLIT = 108;
-struct TileSizes {
-  int small = 0;  // tile levels of at most TILE_SPLIT vertices per axis
-  int big = 0;    // tile levels above TILE_SPLIT
-};
-TileSizes tile_sizes(int n) {
-  TileSizes t;
-  if (tile_level(n)) (n <= TILE_SPLIT ? t.small : t.big) = n;
-  return t;
-}
-TileSizes tmax(TileSizes a, TileSizes b) {
-  a.small = std::max(a.small, b.small);
-  a.big = std::max(a.big, b.big);
-  return a;
-}
-bool tgreater(TileSizes a, TileSizes b) { return a.small > b.small || a.big > b.big; }
+// n if the line path preconditions a level of that size, else 0
+int line_size(int n) { return tile_level(n) ? n : 0; }
 
 // 1, or 2..256 with no prime factor but 2 and 3 (the line transforms are radix-2/3 FFTs)
 bool valid_res(int n) {
@@ -118,7 +101,7 @@ struct pdg_ctx {
   float* stage = nullptr;  // [stage_pts][3] staging of host inputs
   int stage_pts = 0;
   int nmax = 1;
-  TileSizes ntile;  // largest resolutions among the levels the tile path preconditions
+  int nline = 0;  // largest resolution among the levels the line path preconditions
   cudaStream_t cap = nullptr, cap2 = nullptr;
   cudaGraphExec_t gexec = nullptr;
   int graph_kernels = 0;   // kernel nodes of gexec
@@ -147,7 +130,7 @@ struct pdg_batch {
   cudaStream_t cap = nullptr, cap2 = nullptr;
   cudaGraphExec_t gexec = nullptr;
   int graph_nmax = 0;
-  TileSizes graph_ntile;
+  int graph_nline = 0;
   bool dirty = true;  // membership changed since the last upload of the job table
   std::string err;
 };
@@ -166,7 +149,7 @@ struct Layout {
   size_t total = 0;
   size_t job, plan, flag, stage, op_job, op_plan;
   struct Lv {
-    size_t theta, theta_t, m, v, g, tmp, zmask, piv, piv_slow, mu, tw, tw4, cnt, rowptr, flag, act_v, act_ptr, ent, ccnt,
+    size_t theta, theta_t, m, v, g, tmp, zmask, piv, piv_slow, mu, tw, twm, tw4, cnt, rowptr, flag, act_v, act_ptr, ent, ccnt,
         coff, ckey, xs, n_active, csum;
     int cap;
   } lv[MAXL];
@@ -205,6 +188,7 @@ Layout make_layout(const pdg_config& c, int V, int E, int max_pts) {
     v.piv_slow = a.take<int>(1);
     v.mu = a.take<float>(n);
     v.tw = a.take<float2>(n);
+    v.twm = a.take<float2>(tile_level(n) ? n : 1);
     v.tw4 = a.take<float2>(n);
     v.cnt = a.take<int>(n3);
     v.rowptr = a.take<int>(n3 + 1);
@@ -338,9 +322,9 @@ enum StageIndex {
 // Stage i of a step; bump: the job_bump mode of the interpolation stage (1: optimisation
 // step, 2: evaluation); count: the nearest-neighbour instances that count candidates and
 // exact ties.  The plan's item prefixes must be current (refresh_plan).
-// nmax: the largest level resolution; ntile: the largest ones of the levels the tile path
-// preconditions, per size class
-void launch_stage(int i, const Plan* plan, int nmax, TileSizes ntile, int sms, cudaStream_t s, int bump = 1,
+// nmax: the largest level resolution; nline: the largest one of the levels the line path
+// preconditions (0: none)
+void launch_stage(int i, const Plan* plan, int nmax, int nline, int sms, cudaStream_t s, int bump = 1,
                   bool count = false) {
   const int grid = sms * 8;
   switch (i) {
@@ -362,8 +346,10 @@ void launch_stage(int i, const Plan* plan, int nmax, TileSizes ntile, int sms, c
       break;
     }
     case S_SOB_256:
-      if (ntile.small > 0) launch_sobolev_tiles(plan, sms, 0, TILE_SPLIT, ntile.small, s);
-      if (ntile.big > 0) launch_sobolev_tiles(plan, sms, TILE_SPLIT, 256, ntile.big, s);
+      if (nline == 0) break;
+      launch_sobolev_x(plan, sms, nline, true, s);
+      for (int p = YZ_FWD; p <= YZ_INV; ++p) launch_sobolev_yz(plan, sms, nline, p, s);
+      launch_sobolev_x(plan, sms, nline, false, s);
       break;
     case S_LOSS: launch_loss(plan, sms * 2, s); break;
   }
@@ -373,7 +359,7 @@ constexpr int ST_SOB_FIRST = S_SOB_XY_FWD, ST_SOB_LAST = S_SOB_256;  // precondi
 // Captures one step.  Two branches: the isometry kernel runs beside the moving grid's sort
 // and the nearest-neighbour passes (it needs only the deformed points), the loss reduction
 // beside the adjoint and the preconditioner (nothing downstream reads it).
-pdg_status capture_step(pdg_ctx* c, const Plan* plan, int nmax, TileSizes ntile, cudaStream_t cap, cudaStream_t cap2,
+pdg_status capture_step(pdg_ctx* c, const Plan* plan, int nmax, int nline, cudaStream_t cap, cudaStream_t cap2,
                         cudaGraphExec_t* out, std::string* err, int sms, int* n_kernels = nullptr) {
   cudaGraph_t g = nullptr;
   cudaEvent_t ev[4] = {};
@@ -389,22 +375,22 @@ pdg_status capture_step(pdg_ctx* c, const Plan* plan, int nmax, TileSizes ntile,
     return PDG_ERR_CUDA;
   }
   const bool count = c && c->h.count_nn;  // a batch graph never counts
-  launch_stage(S_INTERP, plan, nmax, ntile, sms, cap);  // starts the step of every job
+  launch_stage(S_INTERP, plan, nmax, nline, sms, cap);  // starts the step of every job
   cudaEventRecord(ev[0], cap);
   cudaStreamWaitEvent(cap2, ev[0], 0);
-  launch_stage(S_ISO, plan, nmax, ntile, sms, cap2);
+  launch_stage(S_ISO, plan, nmax, nline, sms, cap2);
   cudaEventRecord(ev[1], cap2);
-  launch_stage(S_MOV_SCAN, plan, nmax, ntile, sms, cap);
-  launch_stage(S_MOV_SCATTER, plan, nmax, ntile, sms, cap);
-  launch_stage(S_NN, plan, nmax, ntile, sms, cap, 1, count);
-  launch_stage(S_NN_HARD, plan, nmax, ntile, sms, cap, 1, count);
+  launch_stage(S_MOV_SCAN, plan, nmax, nline, sms, cap);
+  launch_stage(S_MOV_SCATTER, plan, nmax, nline, sms, cap);
+  launch_stage(S_NN, plan, nmax, nline, sms, cap, 1, count);
+  launch_stage(S_NN_HARD, plan, nmax, nline, sms, cap, 1, count);
   cudaStreamWaitEvent(cap, ev[1], 0);
-  launch_stage(S_ASSEMBLE, plan, nmax, ntile, sms, cap);
+  launch_stage(S_ASSEMBLE, plan, nmax, nline, sms, cap);
   cudaEventRecord(ev[2], cap);
   cudaStreamWaitEvent(cap2, ev[2], 0);
-  launch_stage(S_LOSS, plan, nmax, ntile, sms, cap2);
+  launch_stage(S_LOSS, plan, nmax, nline, sms, cap2);
   cudaEventRecord(ev[3], cap2);
-  for (int i = S_ADJOINT; i <= S_SOB_256; ++i) launch_stage(i, plan, nmax, ntile, sms, cap);  // adjoint, preconditioner, Adam
+  for (int i = S_ADJOINT; i <= S_SOB_256; ++i) launch_stage(i, plan, nmax, nline, sms, cap);  // adjoint, preconditioner, Adam
   cudaStreamWaitEvent(cap, ev[3], 0);
   e = cudaStreamEndCapture(cap, &g);
   for (auto& x : ev) cudaEventDestroy(x);
@@ -520,7 +506,8 @@ pdg_status pdg_create(const pdg_config* cfg, const float* template_xyz, int n_ve
   };
   if (cudaGetDevice(&c->dev) != cudaSuccess) return bail(PDG_ERR_CUDA);
   cudaDeviceGetAttribute(&c->sms, cudaDevAttrMultiProcessorCount, c->dev);
-  sobolev_configure();
+  sobolev_x_configure();
+  sobolev_yz_configure();
   sobolev_plane_configure();
 
   // edges to the host (validation + vertex -> edge lists)
@@ -594,7 +581,7 @@ pdg_status pdg_create(const pdg_config* cfg, const float* template_xyz, int n_ve
   c->stage = (float*)P(L.stage);
   c->stage_pts = std::max(n_verts, max_pts);
   std::vector<float> mu;
-  std::vector<float2> tw, tw4;
+  std::vector<float2> tw, tw4, twm;
   for (int l = 0; l < J.L; ++l) {
     Level& lv = J.lev[l];
     const auto& o = L.lv[l];
@@ -602,7 +589,6 @@ pdg_status pdg_create(const pdg_config* cfg, const float* template_xyz, int n_ve
     lv.n = n;
     lv.lg = (n & (n - 1)) == 0 ? ilog2(n) : -1;
     lv.n3 = n * n * n;
-    lv.tiles = 3 * ((n * n + TILE_LINES - 1) / TILE_LINES);  // one channel per tile
     lv.lr = (float)(cfg->lr0 * std::pow((double)cfg->lr_growth, l) * (cfg->precondition ? 1.0 : 0.1));
     lv.lam = (float)(cfg->lambda0 * std::pow((double)cfg->lambda_growth, l));
     for (int a = 0; a < 3; ++a) {
@@ -621,6 +607,7 @@ pdg_status pdg_create(const pdg_config* cfg, const float* template_xyz, int n_ve
     lv.piv_slow = (int*)P(o.piv_slow);
     lv.mu = (float*)P(o.mu);
     lv.tw = (float2*)P(o.tw);
+    lv.twm = (float2*)P(o.twm);
     lv.tw4 = (float2*)P(o.tw4);
     lv.cnt = (int*)P(o.cnt);
     lv.rowptr = (int*)P(o.rowptr);
@@ -635,7 +622,7 @@ pdg_status pdg_create(const pdg_config* cfg, const float* template_xyz, int n_ve
     lv.n_active = (int*)P(o.n_active);
     lv.csum = (int*)P(o.csum);
     c->nmax = std::max(c->nmax, n);
-    c->ntile = tmax(c->ntile, tile_sizes(n));
+    c->nline = std::max(c->nline, line_size(n));
     mu.resize(n);
     tw.resize(n);
     tw4.resize(n);
@@ -651,6 +638,13 @@ pdg_status pdg_create(const pdg_config* cfg, const float* template_xyz, int n_ve
         cudaMemcpyAsync(lv.tw, tw.data(), tw.size() * sizeof(float2), cudaMemcpyHostToDevice, s) != cudaSuccess ||
         cudaMemcpyAsync(lv.tw4, tw4.data(), n * sizeof(float2), cudaMemcpyHostToDevice, s) != cudaSuccess)
       return bail(PDG_ERR_CUDA);
+    if (tile_level(n)) {
+      const int n1 = line_n1(n);
+      twm.resize(n);
+      for (int i = 0; i < n; ++i) twm[i] = tw[(i / n1) * (i % n1)];
+      if (cudaMemcpyAsync(lv.twm, twm.data(), n * sizeof(float2), cudaMemcpyHostToDevice, s) != cudaSuccess)
+        return bail(PDG_ERR_CUDA);
+    }
     if (!tile_level(n)) launch_sobz_pivots(lv.piv, lv.piv_slow, lv.mu, n, lv.lam, s);
   }
   J.x = (float4*)P(L.x);
@@ -803,7 +797,7 @@ pdg_status pdg_step(pdg_ctx* c, int n_steps, void* cuda_stream) {
   if (!c->gexec) {
     // the captured launches must not start before this stream's pending set-up
     CU(c, cudaStreamSynchronize(s));
-    TRY(capture_step(c, c->dplan, c->nmax, c->ntile, c->cap, c->cap2, &c->gexec, &c->err, c->sms, &c->graph_kernels));
+    TRY(capture_step(c, c->dplan, c->nmax, c->nline, c->cap, c->cap2, &c->gexec, &c->err, c->sms, &c->graph_kernels));
   }
   TRY(refresh_plan(c, s));
   for (int i = 0; i < n_steps; ++i) CU(c, cudaGraphLaunch(c->gexec, s));
@@ -832,7 +826,7 @@ pdg_status pdg_profile_step(pdg_ctx* c, int n_steps, double* stage_ms, void* cud
   for (int k = 0; k < n_steps && st == PDG_OK; ++k) {
     for (int i = 0; i < N_STAGES; ++i) {
       cudaEventRecord(ev[i], s);
-      launch_stage(i, c->dplan, c->nmax, c->ntile, c->sms, s, 1, c->h.count_nn != 0);
+      launch_stage(i, c->dplan, c->nmax, c->nline, c->sms, s, 1, c->h.count_nn != 0);
     }
     cudaEventRecord(ev[N_STAGES], s);
     st = c->cuda(cudaEventSynchronize(ev[N_STAGES]), "profile step");
@@ -1027,7 +1021,7 @@ pdg_status pdg_eval(pdg_ctx* c, double* loss, void* cuda_stream) {
   cudaStream_t s = (cudaStream_t)cuda_stream;
   TRY(refresh_plan(c, s));
   for (int i = 0; i < N_STAGES; ++i)  // no preconditioner, no Adam, no step count
-    if (i < ST_SOB_FIRST || i > ST_SOB_LAST) launch_stage(i, c->dplan, c->nmax, c->ntile, c->sms, s, 2, c->h.count_nn != 0);
+    if (i < ST_SOB_FIRST || i > ST_SOB_LAST) launch_stage(i, c->dplan, c->nmax, c->nline, c->sms, s, 2, c->h.count_nn != 0);
   CU(c, cudaGetLastError());
   if (loss) {
     CU(c, cudaMemcpyAsync(loss, c->h.loss, 4 * sizeof(double), cudaMemcpyDeviceToHost, s));
@@ -1046,7 +1040,8 @@ pdg_status pdg_precondition(pdg_ctx* c, int level, const float* g, float* out, v
   float* tmp = nullptr;
   CU(c, cudaMallocAsync((void**)&tmp, bytes, s));
   CU(c, cudaMemcpyAsync(tmp, g, bytes, is_device_ptr(g) ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice, s));
-  launch_aos_to_soa(tmp, lv.g, lv.n3, s);
+  const bool line = line_size(lv.n) > 0;  // its x passes read and write [n^3][3] themselves
+  if (!line) launch_aos_to_soa(tmp, lv.g, lv.n3, s);
   // a one-level copy of the job that stores the preconditioned gradient instead of Adam
   Job oj = c->h;
   oj.L = 1;
@@ -1056,6 +1051,8 @@ pdg_status pdg_precondition(pdg_ctx* c, int level, const float* g, float* out, v
   oj.precondition = 1;
   oj.keep_pgrad = 1;
   oj.no_adam = 1;
+  oj.ext_in = line ? tmp : nullptr;
+  oj.ext_out = line ? tmp : nullptr;
   Plan op;
   std::memset(&op, 0, sizeof(op));
   op.n_jobs = 1;
@@ -1063,8 +1060,8 @@ pdg_status pdg_precondition(pdg_ctx* c, int level, const float* g, float* out, v
   CU(c, cudaMemcpyAsync(c->op_job, &oj, sizeof(Job), cudaMemcpyHostToDevice, s));
   CU(c, cudaMemcpyAsync(c->op_plan, &op, sizeof(Plan), cudaMemcpyHostToDevice, s));
   launch_plan(c->op_plan, s);
-  for (int i = ST_SOB_FIRST; i <= ST_SOB_LAST; ++i) launch_stage(i, c->op_plan, lv.n, tile_sizes(lv.n), c->sms, s);
-  launch_soa_to_aos(lv.tmp, tmp, lv.n3, s);
+  for (int i = ST_SOB_FIRST; i <= ST_SOB_LAST; ++i) launch_stage(i, c->op_plan, lv.n, line_size(lv.n), c->sms, s);
+  if (!line) launch_soa_to_aos(lv.tmp, tmp, lv.n3, s);
   CU(c, cudaGetLastError());
   const pdg_status st = copy_out(c, out, tmp, bytes, s);
   cudaFreeAsync(tmp, s);
@@ -1132,9 +1129,9 @@ pdg_status pdg_fit_mesh(pdg_ctx* c, const float* p0_xyz, int n_p0, int n_steps, 
   const int2* edges = J.edges;
   for (int k = 1; k <= n_steps; ++k) {
     launch_mesh_points(c->op_job, V, s);
-    for (int i = S_MOV_SCAN; i <= S_NN_HARD; ++i) launch_stage(i, c->op_plan, 1, TileSizes(), c->sms, s);
-    launch_stage(S_ASSEMBLE, c->op_plan, 1, TileSizes(), c->sms, s);
-    launch_stage(S_LOSS, c->op_plan, 1, TileSizes(), c->sms, s);
+    for (int i = S_MOV_SCAN; i <= S_NN_HARD; ++i) launch_stage(i, c->op_plan, 1, 0, c->sms, s);
+    launch_stage(S_ASSEMBLE, c->op_plan, 1, 0, c->sms, s);
+    launch_stage(S_LOSS, c->op_plan, 1, 0, c->sms, s);
     // (I + lambda L)^{-2} dL/dX by two solves, then Adam on the vertices
     launch_mesh_solve(J.v2e_ptr, J.v2e, edges, J.gy, h, r, d0, d1, V, lambda, (float)emax, iters, s);
     launch_mesh_solve(J.v2e_ptr, J.v2e, edges, h, pg, r, d0, d1, V, lambda, (float)emax, iters, s);
@@ -1217,14 +1214,14 @@ pdg_status pdg_batch_step(pdg_batch* b, int n_steps, void* cuda_stream) {
   if (b->n == 0 || n_steps == 0) return PDG_OK;
   cudaStream_t s = (cudaStream_t)cuda_stream;
   int nmax = 1, sms = 1;
-  TileSizes ntile;
+  int nline = 0;
   for (auto* c : b->members) {
     if (!c->in_frame) {
       b->err = "batch member outside a frame";
       return PDG_ERR_STATE;
     }
     nmax = std::max(nmax, c->nmax);
-    ntile = tmax(ntile, c->ntile);
+    nline = std::max(nline, c->nline);
     sms = c->sms;
   }
   if (b->dirty) {
@@ -1248,14 +1245,14 @@ pdg_status pdg_batch_step(pdg_batch* b, int n_steps, void* cuda_stream) {
     b->gens.resize(b->members.size());
     for (size_t i = 0; i < b->members.size(); ++i) b->gens[i] = b->members[i]->frame_gen;
   }
-  if (!b->gexec || nmax > b->graph_nmax || tgreater(ntile, b->graph_ntile)) {
+  if (!b->gexec || nmax > b->graph_nmax || nline > b->graph_nline) {
     if (b->gexec) cudaGraphExecDestroy(b->gexec);
     b->gexec = nullptr;
     if (cudaStreamSynchronize(s) != cudaSuccess) return PDG_ERR_CUDA;
-    const pdg_status st = capture_step(nullptr, b->dplan, std::max(nmax, b->graph_nmax), tmax(ntile, b->graph_ntile), b->cap, b->cap2, &b->gexec, &b->err, sms);
+    const pdg_status st = capture_step(nullptr, b->dplan, std::max(nmax, b->graph_nmax), std::max(nline, b->graph_nline), b->cap, b->cap2, &b->gexec, &b->err, sms);
     if (st != PDG_OK) return st;
     b->graph_nmax = std::max(nmax, b->graph_nmax);
-    b->graph_ntile = tmax(ntile, b->graph_ntile);
+    b->graph_nline = std::max(nline, b->graph_nline);
   }
   for (int i = 0; i < n_steps; ++i)
     if (cudaGraphLaunch(b->gexec, s) != cudaSuccess) return PDG_ERR_CUDA;
