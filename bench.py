@@ -109,8 +109,9 @@ class ClockSampler:
 
 # kernel of each profiled stage and the source file that defines it
 STAGE_KERNEL = {
-    "interp": ("k_interp", "k_points.cu"), "mov_scatter": ("k_mov_scatter", "k_points.cu"),
-    "nn": ("k_nn", "k_nn.cu"), "nn_hard": ("k_nn_hard", "k_nn.cu"), "adjoint": ("k_adjoint", "k_adjoint.cu"),
+    "interp": ("k_interp", "k_points.cu"), "boxes": ("k_boxes", "k_points.cu"),
+    "nn": ("k_nn", "k_nn.cu"), "nn_rev_mesh": ("k_nn", "k_nn.cu"), "nn_rev_pts": ("k_nn", "k_nn.cu"),
+    "adjoint": ("k_adjoint", "k_adjoint.cu"), "adjoint_rows": ("k_adjoint_rows", "k_adjoint.cu"),
     "sob_xy_fwd": ("k_sobp", "k_sobolev_plane.cu"), "sob_z": ("k_sobz", "k_sobolev_plane.cu"),
     "sob_xy_inv": ("k_sobp_inv", "k_sobolev_plane.cu"), "adam": ("k_adam", "k_sobolev_plane.cu"),
     "iso_edges": ("k_iso_edges", "k_points.cu"),
@@ -146,13 +147,9 @@ def max_over_ranks(value: float, dist=None, device=None) -> float:
     return float(t.item())
 
 
-def grid_bits(count, per_cell=8.0):
-    """log2 cells per axis of a nearest-neighbour grid (as the library chooses it): about
-    8 points per occupied cell for the target grid, 32 for the moving grid."""
-    import math
-
-    g = math.sqrt(max(count, 1) / per_cell)
-    return min(max(int(round(math.log2(max(g, 1.0)))), 2), 7)
+# stages that are one row of the step, profiled as several launches
+NN_STAGES = ("nn", "nn_rev_mesh", "nn_rev_pts")  # searches of the moving points, of the targets per moving set
+ADJOINT_STAGES = ("adjoint", "adjoint_rows")
 
 
 def active_vertices(x, res, lo=-1.5, hi=1.5):
@@ -191,7 +188,7 @@ def stage_model(stage, Q, V, M, E, res, act):
         return "hbm", Q * 24 + A * 12, "B"
     if stage == "adjoint":  # read dL/dy (16 B per point), write each touched grid gradient
         return "hbm", Q * 16 + A * 12, "B"
-    if stage in ("nn", "nn_hard"):
+    if stage in NN_STAGES:
         return "alu", None, "FLOP"
     if stage == "iso_edges":
         return "hbm", E * (8 + 4 + 4 + 12) + V * 12, "B"
@@ -199,11 +196,6 @@ def stage_model(stage, Q, V, M, E, res, act):
         return "hbm", Q * (12 + 12 + 12) + V * 12, "B"
     if stage == "loss":
         return "hbm", (Q + 2 * M + E) * 4, "B"
-    if stage == "mov_scan":
-        G3 = 2 * (1 << (3 * grid_bits(max(V, M), 32.0)))
-        return "hbm", G3 * 8, "B"
-    if stage == "mov_scatter":
-        return "hbm", Q * (4 + 12 + 16), "B"
     return "hbm", 0, "B"
 
 
@@ -531,7 +523,7 @@ def main():
     sm_mhz = clocks["sm_mhz"] or sm_max
     sms = torch.cuda.get_device_properties(dev).multi_processor_count
     fp32_peak = sms * 128 * 2 * sm_mhz * 1e6 / 1e12
-    nn_ms = prof["nn"] + prof["nn_hard"]
+    nn_ms = sum(prof[k] for k in NN_STAGES)
     stages = {}
     for k, ms in prof.items():
         b_, a_, u_ = stage_model(k, Q, V, M, E, w.res, act)
@@ -549,15 +541,15 @@ def main():
                            "TFLOP/s": round(8 * nn_cands / (nn_ms / 1e3) / 1e12, 3),
                            "frac_fp32": round(8 * nn_cands / (nn_ms / 1e3) / 1e12 / fp32_peak, 4)}
     grouped = dict(prof)
-    grouped["nn"] = nn_ms  # the search's two passes form one stage of the step
-    grouped.pop("nn_hard")
+    for name, parts in (("nn", NN_STAGES), ("adjoint", ADJOINT_STAGES)):
+        grouped[name] = sum(grouped.pop(k) for k in parts)
     dom = max(grouped, key=grouped.get)
     bound, amount, unit = stage_model(dom, Q, V, M, E, w.res, act)
     if bound == "alu":
         amount = 8.0 * nn_cands
         achieved = amount / (nn_ms / 1e3) / 1e12
         roof = {"bound": "alu", "achieved": achieved, "peak": fp32_peak, "unit": "TFLOP/s", "frac": achieved / fp32_peak,
-                "traffic": measured_traffic("nn"), "kernel": "k_nn + k_nn_hard",
+                "traffic": measured_traffic("nn"), "kernel": "k_nn (three launches)",
                 "algorithmic_flops": amount,
                 "peak_note": f"FP32 {sms} SMs x 128 FMA x 2 at {sm_mhz:.0f} MHz (measured clock); 8 FLOP per squared "
                              f"distance the search evaluated ({nn_cands:.4g} per step, counted by the kernels)"}

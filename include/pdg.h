@@ -157,8 +157,7 @@ enum pdg_buffer {
   PDG_BUF_SOURCE = 8,   /* current source cloud P_{t-1}, float [n_src][3] */
   PDG_BUF_COUNTERS = 9, /* uint64 [4] of the last step: squared distances the nearest-neighbour
                            search evaluated and queries decided by an exact tie (both counted
-                           only with PDG_DEBUG_COUNT_NN, else 0), queries left to the
-                           warp-cooperative ring search, 0 */
+                           only with PDG_DEBUG_COUNT_NN, else 0), 0, 0 */
   PDG_BUF_MESH_GRAD = 10, /* dL_mesh/dX of the last pdg_fit_mesh iteration, float [n_verts][3]
                              (PDG_ERR_STATE before a fit, or once a frame has begun since) */
   PDG_BUF_MESH_PGRAD = 11 /* the same preconditioned, (I + lambda L)^{-2} dL_mesh/dX */

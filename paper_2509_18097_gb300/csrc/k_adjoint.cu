@@ -90,49 +90,6 @@ __global__ void k_csr_compact(Job* __restrict__ Jp, int l) {
 }
 
 
-// The finest level's cell order of the query points (per frame): counting sort of the points
-// by interpolation cell (iz (n-1) + iy)(n-1) + ix, storing each point's fractions and index.
-// The interpolation takes its points in this order, so the lanes of a warp interpolate
-// between the same or neighbouring grid vertices.
-__device__ __forceinline__ int point_cell(const Job& J, const Level& lv, float px, float py, float pz, float& fx,
-                                          float& fy, float& fz) {
-  const int n = lv.n;
-  if (n == 1) {
-    fx = fy = fz = 0.f;
-    return 0;
-  }
-  int ix, iy, iz;
-  grid_coord(px, J.lo[0], lv.sc_hi[0], lv.sc_lo[0], n, ix, fx);
-  grid_coord(py, J.lo[1], lv.sc_hi[1], lv.sc_lo[1], n, iy, fy);
-  grid_coord(pz, J.lo[2], lv.sc_hi[2], lv.sc_lo[2], n, iz, fz);
-  return (iz * (n - 1) + iy) * (n - 1) + ix;
-}
-
-__global__ void k_cell_count(Job* __restrict__ Jp) {
-  const Job& J = *Jp;
-  const Level& lv = J.lev[J.L - 1];
-  for (int p = blockIdx.x * blockDim.x + threadIdx.x; p < J.Q; p += gridDim.x * blockDim.x) {
-    const float4 x = J.x[p];
-    float fx, fy, fz;
-    const int c = point_cell(J, lv, x.x, x.y, x.z, fx, fy, fz);
-    lv.ckey[p] = c;
-    atomicAdd(&lv.ccnt[c], 1);
-  }
-}
-
-__global__ void k_cell_fill(Job* __restrict__ Jp) {
-  const Job& J = *Jp;
-  const Level& lv = J.lev[J.L - 1];
-  for (int p = blockIdx.x * blockDim.x + threadIdx.x; p < J.Q; p += gridDim.x * blockDim.x) {
-    const float4 x = J.x[p];
-    float fx, fy, fz;
-    point_cell(J, lv, x.x, x.y, x.z, fx, fy, fz);
-    const int c = lv.ckey[p];
-    const int pos = lv.coff[c] + atomicSub(&lv.ccnt[c], 1) - 1;  // counts return to zero
-    lv.xs[pos] = make_float4(fx, fy, fz, __int_as_float(p));
-  }
-}
-
 void launch_csr_build(Job* J, const Job& hJ, cudaStream_t s) {
   const int grid = max(1, min((hJ.Q + 255) / 256, 4096));
   k_csr_count<<<grid, 256, 0, s>>>(J);
@@ -150,23 +107,15 @@ void launch_csr_build(Job* J, const Job& hJ, cudaStream_t s) {
     launch_scan_segments(&seg, 1, nullptr, nullptr, s);
     k_csr_compact<<<g2, 256, 0, s>>>(J, l);
   }
-  // the finest level's cell order
-  const Level& lf = hJ.lev[hJ.L - 1];
-  const int nc = lf.n > 1 ? (lf.n - 1) * (lf.n - 1) * (lf.n - 1) : 1;
-  k_cell_count<<<grid, 256, 0, s>>>(J);
-  ScanSeg seg{lf.ccnt, lf.coff, nc, lf.csum};
-  launch_scan_segments(&seg, 1, nullptr, nullptr, s);
-  k_cell_fill<<<grid, 256, 0, s>>>(J);
   launch_zmask(J, hJ, s);
 }
 
 // ------------------------------------------------------------------------------ per step
 
-// All levels of all jobs in one launch of 256-thread blocks.  Rows are summed by groups of
+// All levels of all jobs in two launches, side by side in the step.  Rows are summed by groups of
 // 2^adj_lg lanes, set by the plan kernel from the level's mean row length (a few dozen
-// entries per row on 128^3, thousands on 16^3): 32 >> adj_lg rows per warp, or a whole
-// block per row on levels whose rows average 512 entries or more.  A job's items are its
-// block rows first, then its warp groups, 8 to a block.  Each lane takes its entries in
+// entries per row on 128^3, thousands on 16^3): 32 >> adj_lg rows per warp (k_adjoint), or a whole
+// block per row on levels whose rows average 512 entries or more (k_adjoint_rows).  Each lane takes its entries in
 // batches of B: the B index and weight loads, then the B gathers (of dLoss/dz and dLoss/dt
 // with the Cayley payload), all issued before any of them is used (entries past the row's end
 // get weight 0), and loads its next batch's entries while those gathers are in flight.  All
@@ -328,30 +277,40 @@ __device__ __forceinline__ void group_row(const Job& J, const Level& lv, int r, 
   if (sub == 0 && r < na) store_row<C>(lv, r, finite, isc, A);
 }
 
-__global__ void __launch_bounds__(256, 4) k_adjoint(const Plan* __restrict__ P) {
+// The fixed-point scale of a job's step, from its bound on the point gradients: every term |w g| is
+// below 2^ex, so a scaled term is below 2^44 (the range of round_to_ll), and a row has at most Q
+// terms, so partial sums stay below 2^62.
+struct FxScale {
+  float sc, isc;
+  bool live, finite;
+};
+__device__ __forceinline__ FxScale fx_scale(const Job& J) {
+  FxScale f;
+  const float gm = __uint_as_float(*J.gmax);
+  f.finite = gm <= 3.0e38f;
+  f.live = gm > 0.f && f.finite;
+  int sh = 0;
+  if (f.live) {  // ex: gm = m 2^ex with m in [0.5, 1), as frexp
+    const unsigned gb = __float_as_uint(gm);
+    const int be = (int)(gb >> 23);
+    const int ex = be ? be - 126 : (31 - __clz((int)(gb & 0x7fffffu))) - 148;
+    sh = min(min(62 - (32 - __clz(J.Q)), 44) - ex, 126);
+  }
+  f.sc = exp2f((float)sh);
+  f.isc = exp2f((float)-sh);
+  return f;
+}
+
+// Levels with long rows: a block per row
+__global__ void __launch_bounds__(256, 4) k_adjoint_rows(const Plan* __restrict__ P) {
   __shared__ long long red[6][8];
   const int nj = P->n_jobs;
-  const int total = P->pre[ST_ADJ][nj];
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int total = P->pre[ST_ADJROW][nj];
   for (int it = blockIdx.x; it < total; it += gridDim.x) {  // block-uniform
-    const int j = find_job(P->pre[ST_ADJ], nj, it);
+    const int j = find_job(P->pre[ST_ADJROW], nj, it);
     const Job& J = *P->jobs[j];
-    int i = it - P->pre[ST_ADJ][j];
-    // fixed-point scale from the step's bound on the point gradients: every term |w g| < 2^ex,
-    // so a scaled term is below 2^44 (the range of round_to_ll), and a row has at most Q
-    // terms, so partial sums stay below 2^62
-    const float gm = __uint_as_float(*J.gmax);
-    const bool finite = gm <= 3.0e38f;
-    const bool live = gm > 0.f && finite;
-    int sh = 0;
-    if (live) {  // ex: gm = m 2^ex with m in [0.5, 1), as frexp
-      const unsigned gb = __float_as_uint(gm);
-      const int be = (int)(gb >> 23);
-      const int ex = be ? be - 126 : (31 - __clz((int)(gb & 0x7fffffu))) - 148;
-      sh = min(min(62 - (32 - __clz(J.Q)), 44) - ex, 126);
-    }
-    const float sc = exp2f((float)sh), isc = exp2f((float)-sh);
-    // block rows
+    int i = it - P->pre[ST_ADJROW][j];
+    const FxScale f = fx_scale(J);
     int l = 0;
     for (; l < J.L; ++l) {
       if (J.lev[l].adj_lg != 6) continue;
@@ -359,14 +318,23 @@ __global__ void __launch_bounds__(256, 4) k_adjoint(const Plan* __restrict__ P) 
       if (i < na) break;
       i -= na;
     }
-    if (l < J.L) {
-      if (J.C == 6) block_row<6>(J, J.lev[l], i, live, finite, sc, isc, red);
-      else block_row<3>(J, J.lev[l], i, live, finite, sc, isc, red);
-      continue;
-    }
-    // warp groups
-    int gi = i * 8 + warp, na = 0, lg = 0;
-    for (l = 0; l < J.L; ++l) {
+    if (l >= J.L) continue;
+    if (J.C == 6) block_row<6>(J, J.lev[l], i, f.live, f.finite, f.sc, f.isc, red);
+    else block_row<3>(J, J.lev[l], i, f.live, f.finite, f.sc, f.isc, red);
+  }
+}
+
+// The other levels: a warp per group of 32 >> adj_lg rows
+__global__ void __launch_bounds__(256, 4) k_adjoint(const Plan* __restrict__ P) {
+  const int nj = P->n_jobs;
+  const int total = P->pre[ST_ADJ][nj];
+  const int lane = threadIdx.x & 31;
+  for (int it = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; it < total; it += (gridDim.x * blockDim.x) >> 5) {
+    const int j = find_job(P->pre[ST_ADJ], nj, it);
+    const Job& J = *P->jobs[j];
+    const FxScale f = fx_scale(J);
+    int gi = it - P->pre[ST_ADJ][j], na = 0, lg = 0, l = 0;
+    for (; l < J.L; ++l) {
       lg = J.lev[l].adj_lg;
       if (lg == 6) continue;
       na = *J.lev[l].n_active;
@@ -374,13 +342,14 @@ __global__ void __launch_bounds__(256, 4) k_adjoint(const Plan* __restrict__ P) 
       if (gi < ng) break;
       gi -= ng;
     }
-    if (l >= J.L) continue;  // past the last group (whole warp)
+    if (l >= J.L) continue;
     const int r = (gi << (5 - lg)) + (lane >> lg);
-    if (J.C == 6) group_row<6>(J, J.lev[l], r, na, lg, live, finite, sc, isc);
-    else group_row<3>(J, J.lev[l], r, na, lg, live, finite, sc, isc);
+    if (J.C == 6) group_row<6>(J, J.lev[l], r, na, lg, f.live, f.finite, f.sc, f.isc);
+    else group_row<3>(J, J.lev[l], r, na, lg, f.live, f.finite, f.sc, f.isc);
   }
 }
 
+void launch_adjoint_rows(const Plan* P, int grid, cudaStream_t s) { k_adjoint_rows<<<grid, 256, 0, s>>>(P); }
 void launch_adjoint(const Plan* P, int grid, cudaStream_t s) { k_adjoint<<<grid, 256, 0, s>>>(P); }
 
 }  // namespace pdg

@@ -9,26 +9,28 @@
 
 namespace pdg {
 
-// y = x for the mesh vertices (the query points of the fit), their moving-grid keys and
-// counts, cleared reverse-Chamfer accumulators; the first thread clears the step's counters.
-__global__ void k_mesh_points(Job* __restrict__ Jp) {
+// y = x for the mesh vertices (the query points of the fit), their tree nodes (a block each, in
+// the slot order of the fit's start), cleared reverse-Chamfer accumulators; the first thread
+// clears the step's counters.
+__global__ void __launch_bounds__(NODE) k_mesh_points(Job* __restrict__ Jp) {
   const Job& J = *Jp;
   if (blockIdx.x == 0 && threadIdx.x == 0) {
-    *J.hard_count = 0;
     *J.gmax = 0u;
     J.counters[CNT_NN_CANDIDATES] = 0ull;
     J.counters[CNT_NN_TIES] = 0ull;
-    J.counters[CNT_NN_HARD] = 0ull;
   }
-  for (int p = blockIdx.x * blockDim.x + threadIdx.x; p < J.V; p += gridDim.x * blockDim.x) {
-    const float4 x = J.x[p];
-    J.y[p] = make_float4(x.x, x.y, x.z, 0.f);
-    const int key = cell_key(J.mov, x.x, x.y, x.z, 0);
-    J.mov.keys[p] = key;
-    atomicAdd(&J.mov.hist[key], 1);
-    J.acc[3 * p + 0] = 0;
-    J.acc[3 * p + 1] = 0;
-    J.acc[3 * p + 2] = 0;
+  const int nodes = (J.V + NODE - 1) / NODE;
+  for (int nd = blockIdx.x; nd < nodes; nd += gridDim.x) {
+    const int p = J.mov.perm[nd * NODE + threadIdx.x];
+    float4 x = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (p >= 0) {
+      x = J.x[p];
+      J.y[p] = make_float4(x.x, x.y, x.z, 0.f);
+      J.acc[3 * p + 0] = 0;
+      J.acc[3 * p + 1] = 0;
+      J.acc[3 * p + 2] = 0;
+    }
+    store_node(J.mov, nd, x.x, x.y, x.z, p >= 0);
   }
 }
 
@@ -99,7 +101,7 @@ __global__ void k_mesh_adam(float4* __restrict__ x, const float4* __restrict__ g
 
 static inline int mesh_blocks(int n) { return max(1, min((n + 255) / 256, 4096)); }
 
-void launch_mesh_points(Job* J, int V, cudaStream_t s) { k_mesh_points<<<mesh_blocks(V), 256, 0, s>>>(J); }
+void launch_mesh_points(Job* J, int V, cudaStream_t s) { k_mesh_points<<<mesh_blocks(V), NODE, 0, s>>>(J); }
 
 void launch_mesh_solve(const int* v2e_ptr, const int* v2e, const int2* edges, const float4* b, float4* h, float4* r,
                        float4* d0, float4* d1, int V, float lam, float emax, int iters, cudaStream_t s) {

@@ -2,146 +2,53 @@
 // its gradient.  Four searches per step: template vertices and source points (the moving
 // sets) against the target cloud, and the target cloud against each moving set.
 //
-// The target (per frame) and the moving sets (per step) are counting-sorted into uniform
-// cell grids (see CellGrid, about 32 points per occupied cell).  A first kernel searches
-// every query's 3x3x3 cell box with one thread per query, starting from the query's
-// neighbour of the previous step, queries taken in cell order so neighbouring lanes read the
-// same cells (cells that cannot beat the best distance found so far are skipped).  The
-// answer is certified when the best squared distance is below the squared distance from the
-// query to the searched box's open faces (with a margin covering the rounding of the cell
-// assignment); otherwise the same thread searches the next shell (up to NN_RTHREAD), and a
-// query still uncertified is appended to a per-job list that a second, warp-cooperative
-// kernel searches ring by ring (lanes split the rows of each shell, a
-// __shfl min-reduction over (d^2, index) packed in 64 bits picks the lexicographic minimum,
-// i.e. the lowest index on ties), falling back to an exhaustive scan of the set beyond
-// NN_RMAX rings.  Both kernels compare candidates with the same fp32 expression, so the
-// result is the exact lexicographic minimum of (fp32 d^2, index) over the whole set.
+// A warp takes 32 / SUB neighbouring queries (consecutive slots of their own tree), SUB lanes each,
+// through the box tree of the searched set together (see Tree).  At the upper levels the 32 lanes
+// test 32 boxes against the box of the warp's queries: a box farther away than the worst of the
+// warp's best distances holds nothing for any query.  The leaves that survive are listed; each
+// sub-lane of a query takes every SUB-th of them, tests it against its own query and best distance,
+// and evaluates its 8 points (two points per packed FP32 instruction).  Queries start from their
+// neighbour of the previous step, a point of the set, so the bounds are tight from the first box on.
+//
+// Why this split.  About 8 leaves per query pass its own bound (100k points, neighbours 4 spacings
+// away), 26 that of any of 32 neighbouring queries: a warp of 32 queries evaluates 3 times what one
+// query needs, and its chain of dependent box loads (about 20 us whatever the size) leaves a small
+// problem waiting.  Fewer queries per warp shorten both and repeat the upper levels.  Step times,
+// SUB = 1 / 2 / 4 / 8: 100k points 275 / 268 / 272 / 307 us, 20k (Cayley) 288 / 278 / 280 / 285,
+// 2k 66 / 62 / 58 / 57; so SUB = 8 below 4 warps of 32 queries per SM and 2 above.
+// What bounds it: register write-back of L1 loads (a leaf is 96 bytes to every lane) and latency,
+// 0.5 instructions per cycle and scheduler.  It replaces a thread per query over 3x3x3 boxes of
+// 32-point cells with the moving points re-sorted each step: at 100k points (searches, sort, ring
+// pass) 157 us of launches; the order of the points is now the frame's, and only boxes are redone.
+//
+// Exactness: candidates are compared with one fp32 expression (sqdist).  The bounds use the same
+// operations in the same order on differences that rounding cannot carry past the true ones
+// (subtraction, product and fused sum are monotone in fp32), so a box's bound never exceeds the
+// fp32 squared distance of a point in it, and only strictly larger bounds are skipped.  The result
+// is the exact lexicographic minimum of (fp32 d^2, index) over the whole set.
 #include <float.h>
 
 #include "kernels.h"
 
 namespace pdg {
 
-// Best candidate so far; `tie` (counting instance only): another point had exactly the same
-// squared distance (the lowest index decided), which the step reports as a count.
-struct Best {
-  float d2;
-  int idx;
-  bool tie;
-};
-
-// COUNT: the instance used when the context counts (PDG_DEBUG_COUNT_NN); it also tracks
-// exact ties.  The two instances take the same minimum.
-template <bool COUNT>
-__device__ __forceinline__ void consider(Best& b, const float4 p, float qx, float qy, float qz) {
-  const float d2 = sqdist(qx, qy, qz, p.x, p.y, p.z);
-  if (d2 <= b.d2) {  // rarely taken; the index decides only between equal distances
-    const int id = __float_as_int(p.w);
-    if (COUNT) {
-      if (d2 < b.d2) {
-        b.d2 = d2;
-        b.idx = id;
-        b.tie = false;
-      } else if (id != b.idx) {
-        b.tie = true;
-        b.idx = min(b.idx, id);
-      }
-    } else if (d2 < b.d2 || id < b.idx) {
-      b.d2 = d2;
-      b.idx = id;
-    }
-  }
-}
-
-// Squared lower bound on the distance from q to any point assigned to a cell outside the
-// box [c - r, c + r] (per axis, clipped to the grid).  FLT_MAX if the box covers the grid.
-__device__ __forceinline__ float outside_bound2(const CellGrid& g, float qx, float qy, float qz, int cx, int cy,
-                                                int cz, int r) {
-  const int G = 1 << g.bits;
-  const float q[3] = {qx, qy, qz};
-  const int c[3] = {cx, cy, cz};
-  float d = FLT_MAX;
-  float hmin = FLT_MAX;
-#pragma unroll
-  for (int a = 0; a < 3; ++a) {
-    hmin = fminf(hmin, g.h[a]);
-    if (c[a] - r > 0) d = fminf(d, q[a] - (g.lo[a] + (float)(c[a] - r) * g.h[a]));
-    if (c[a] + r < G - 1) d = fminf(d, (g.lo[a] + (float)(c[a] + r + 1) * g.h[a]) - q[a]);
-  }
-  if (d == FLT_MAX) return FLT_MAX;
-  d -= 1e-4f * hmin;  // cell assignment and face positions are rounded in fp32
-  if (d <= 0.f) return 0.f;
-  return d * d * (1.f - 4e-6f);
-}
-
-// Lower bounds on the distance from q to the points assigned to other cells of its grid.
-// m[a] / p[a]: distance from q to the lower / upper face of its own cell along axis a, less
-// the same rounding margin as above (negative for a query clamped into a boundary cell).
-// A cell d steps away along a (d < 0 below) lies beyond that face plus |d| - 1 cells.
-struct FaceBounds {
-  float m[3], p[3], h[3];
-};
-
-__device__ __forceinline__ FaceBounds face_bounds(const CellGrid& g, float qx, float qy, float qz, int cx, int cy,
-                                                  int cz) {
-  const float q[3] = {qx, qy, qz};
-  const int c[3] = {cx, cy, cz};
-  const float margin = 1e-4f * fminf(g.h[0], fminf(g.h[1], g.h[2]));
-  FaceBounds f;
-#pragma unroll
-  for (int a = 0; a < 3; ++a) {
-    f.m[a] = q[a] - (g.lo[a] + (float)c[a] * g.h[a]) - margin;
-    f.p[a] = (g.lo[a] + (float)(c[a] + 1) * g.h[a]) - q[a] - margin;
-    f.h[a] = g.h[a];
-  }
-  return f;
-}
-
-// squared lower bound contributed by axis a for a cell d steps away (0 for d = 0), shrunk by
-// the relative rounding of a squared distance; the bound of a cell is the sum over its axes
-__device__ __forceinline__ float axis_lb(const FaceBounds& f, int a, int d) {
-  if (d == 0) return 0.f;
-  const float t = fmaxf((d < 0 ? f.m[a] : f.p[a]) + (float)(abs(d) - 1) * f.h[a], 0.f);
-  return t * t * (1.f - 4e-6f);
-}
+constexpr int NN_THREADS = 128;
 
 // ------------------------------------------------------------------------------ finalise
 
-// Resolves a query item of a job into its point, grid and set.
-// items [0, Q): forward queries in moving-grid order; [Q, Q + 2M): reverse queries
-// (set 0 then set 1) in target-grid order.
 struct QueryRef {
   float x, y, z;
-  int id;    // Q index (forward) or target index (reverse)
-  int set;   // grid set searched
-  bool fwd;
+  int id;    // Q index (forward) or target index (reverse), -1: padding
+  int set;   // moving set searched (reverse)
 };
-
-__device__ __forceinline__ QueryRef resolve(const Job& J, int item) {
-  QueryRef q;
-  float4 p;
-  if (item < J.Q) {
-    p = J.mov.pts[item];
-    q.fwd = true;
-    q.set = 0;
-  } else {
-    const int r = item - J.Q;
-    q.set = r >= J.M ? 1 : 0;
-    p = J.tgt.pts[r - q.set * J.M];
-    q.fwd = false;
-  }
-  q.x = p.x; q.y = p.y; q.z = p.z;
-  q.id = __float_as_int(p.w);
-  return q;
-}
 
 // The loss term phi(s) = s e^{-alpha s} and the gradient 2 phi'(s) (a - b) of a matched
 // pair (Sec. 3.4); phi'(s) = e^{-alpha s}(1 - alpha s), or e^{-alpha s} with the stop-gradient.
-template <bool COUNT>
-__device__ __forceinline__ void finalize(const Job& J, const QueryRef& q, const Best& b) {
-  if (COUNT && b.tie) atomicAdd(J.counters + CNT_NN_TIES, 1ull);
-  if (b.idx == 0x7fffffff || !(b.d2 < FLT_MAX)) {  // nothing found (non-finite coordinates)
-    if (q.fwd) {
+// d2, idx: the nearest point (idx < 0: none found, non-finite coordinates).
+template <bool FWD>
+__device__ __forceinline__ void finalize(const Job& J, const QueryRef& q, float d2, int idx) {
+  if (idx < 0) {
+    if (FWD) {
       J.loss_fwd[q.id] = __int_as_float(0x7fc00000);
       J.gfwd[q.id] = make_float4(0.f, 0.f, 0.f, 0.f);
       J.nn_fwd[q.id] = -1;
@@ -151,254 +58,361 @@ __device__ __forceinline__ void finalize(const Job& J, const QueryRef& q, const 
     }
     return;
   }
-  const float s = b.d2;
+  const float s = d2;
   const float e = expf(-J.alpha * s);
   const float phi = s * e;
   const float dphi = J.stopgrad ? e : e * (1.f - J.alpha * s);
-  if (q.fwd) {  // moving point a = q -> target point b
-    const float4 t = J.tgt4[b.idx];
+  if (FWD) {  // moving point a = q -> target point b
+    const float4 t = J.tgt4[idx];
     const bool mesh = q.id < J.V;
     const float coef = 2.f * dphi * (mesh ? J.w_mesh / (float)J.V : J.w_pts / (float)(J.Q - J.V));
     J.loss_fwd[q.id] = phi;
     J.gfwd[q.id] = make_float4(coef * (q.x - t.x), coef * (q.y - t.y), coef * (q.z - t.z), 0.f);
-    J.nn_fwd[q.id] = b.idx;
+    J.nn_fwd[q.id] = idx;
   } else {  // target point q -> moving point a of set q.set; the gradient goes to a
-    const float4 a = J.y[b.idx];
+    const float4 a = J.y[idx];
     J.loss_rev[q.set * J.M + q.id] = phi;
-    J.nn_rev[q.set * J.M + q.id] = b.idx - (q.set ? J.V : 0);
+    J.nn_rev[q.set * J.M + q.id] = idx - (q.set ? J.V : 0);
     const float c = 2.f * dphi;
-    unsigned long long* acc = reinterpret_cast<unsigned long long*>(J.acc + 3 * (size_t)b.idx);
+    unsigned long long* acc = reinterpret_cast<unsigned long long*>(J.acc + 3 * (size_t)idx);
     atomicAdd(acc + 0, (unsigned long long)to_fx(c * (a.x - q.x)));
     atomicAdd(acc + 1, (unsigned long long)to_fx(c * (a.y - q.y)));
     atomicAdd(acc + 2, (unsigned long long)to_fx(c * (a.z - q.z)));
   }
 }
 
-// ------------------------------------------------------------------------------ shells
+// ------------------------------------------------------------------------------ bounds
 
-template <bool COUNT>
-__device__ __forceinline__ void scan_range(const CellGrid& g, int s, int e, float qx, float qy, float qz, Best& b,
-                                           int& nc) {
-  if (COUNT) nc += e - s;
-  for (int k = s; k < e; ++k) consider<COUNT>(b, __ldg(g.pts + k), qx, qy, qz);
-}
+struct Box {
+  float4 a;  // lo x, lo y, lo z, hi x
+  float2 c;  // hi y, hi z
+};
 
-// adds the candidate counts of the lanes of one job to its counter (counting instance)
-__device__ __forceinline__ void count_candidates(const Job& J, int j, int nc) {
-  const unsigned act = __activemask();
-  const unsigned same = __match_any_sync(act, j);
-  const unsigned s = __reduce_add_sync(same, (unsigned)nc);
-  if ((threadIdx.x & 31) == __ffs(same) - 1) atomicAdd(J.counters + CNT_NN_CANDIDATES, (unsigned long long)s);
-}
-
-// Candidates of row (dy, dz) of shell r around cell (cx, cy, cz): rows on the shell's
-// y/z boundary over the x range [cx - r, cx + r], the others only at x = cx -/+ r.  Cells
-// whose lower bound is above min(cap, best so far) are skipped (strictly above: an equal
-// distance with a lower index must still be seen).
-template <bool COUNT>
-__device__ __forceinline__ void scan_shell_row(const CellGrid& g, int base, int G, int cx, int cy, int cz, int r,
-                                               int dy, int dz, float qx, float qy, float qz, const FaceBounds& fb,
-                                               float cap, Best& b, int& nc) {
-  const int yy = cy + dy, zz = cz + dz;
-  if (yy < 0 || yy >= G || zz < 0 || zz >= G) return;
-  const float lim = fminf(cap, b.d2);
-  const float lyz = axis_lb(fb, 1, dy) + axis_lb(fb, 2, dz);
-  if (lyz > lim) return;
-  const int rk = base + row_key(yy, zz, g.bits);
-  if (max(abs(dy), abs(dz)) == r) {
-    int x0 = max(cx - r, 0), x1 = min(cx + r, G - 1);
-    while (x0 < cx && lyz + axis_lb(fb, 0, x0 - cx) > lim) ++x0;
-    while (x1 > cx && lyz + axis_lb(fb, 0, x1 - cx) > lim) --x1;
-    scan_range<COUNT>(g, __ldg(g.off + rk + x0), __ldg(g.off + rk + x1 + 1), qx, qy, qz, b, nc);
-  } else {
-    if (cx - r >= 0 && !(lyz + axis_lb(fb, 0, -r) > fminf(cap, b.d2)))
-      scan_range<COUNT>(g, __ldg(g.off + rk + cx - r), __ldg(g.off + rk + cx - r + 1), qx, qy, qz, b, nc);
-    if (cx + r < G && !(lyz + axis_lb(fb, 0, r) > fminf(cap, b.d2)))
-      scan_range<COUNT>(g, __ldg(g.off + rk + cx + r), __ldg(g.off + rk + cx + r + 1), qx, qy, qz, b, nc);
-  }
-}
-
-// ------------------------------------------------------------------------------ thread pass
-
-template <bool COUNT>
-__global__ void __launch_bounds__(256) k_nn(const Plan* __restrict__ P) {
-  const int nj = P->n_jobs;
-  const int total = P->pre[ST_NNQ][nj];
-  for (int it = blockIdx.x * blockDim.x + threadIdx.x; it < total; it += gridDim.x * blockDim.x) {
-    const int j = find_job(P->pre[ST_NNQ], nj, it);
-    const Job& J = *P->jobs[j];
-    const int item = it - P->pre[ST_NNQ][j];
-    const QueryRef q = resolve(J, item);
-    const CellGrid& g = q.fwd ? J.tgt : J.mov;
-    const int G = 1 << g.bits;
-    const int base = q.set * G * G * G;
-    const int cx = cell_coord(q.x, g.lo[0], g.inv_h[0], G);
-    const int cy = cell_coord(q.y, g.lo[1], g.inv_h[1], G);
-    const int cz = cell_coord(q.z, g.lo[2], g.inv_h[2], G);
-    Best b{FLT_MAX, 0x7fffffff, false};
-    int nc = 0;  // candidates evaluated (profiling)
-    // warm start: the query's neighbour of the previous step (of this frame), at its current
-    // position, compared with the same expression as every other candidate.  It is one of
-    // the set's points, so the search below, which skips only cells that cannot hold a
-    // distance <= the best, still ends at the exact lexicographic minimum; starting close to
-    // it lets that pruning work from the first cell.
-    {
-      const int w = q.fwd ? J.nn_fwd[q.id] : J.nn_rev[q.set * J.M + q.id];
-      if (w >= 0) {
-        const int gid = q.fwd ? w : w + (q.set ? J.V : 0);
-        const float4 p = q.fwd ? J.tgt4[w] : J.y[gid];
-        b.d2 = sqdist(q.x, q.y, q.z, p.x, p.y, p.z);
-        b.idx = gid;
-      }
-    }
-    // ring 1: the 3x3x3 box, the query's own cell first.  A neighbouring cell is skipped
-    // when a lower bound on the squared distance to anything assigned to it is already above
-    // the best one: it can hold neither the minimum nor an equal distance with a lower index.
-    const FaceBounds fb = face_bounds(g, q.x, q.y, q.z, cx, cy, cz);
-    {
-      int rk = base + row_key(cy, cz, g.bits);
-      scan_range<COUNT>(g, __ldg(g.off + rk + cx), __ldg(g.off + rk + cx + 1), q.x, q.y, q.z, b, nc);
-      if (cx > 0 && !(axis_lb(fb, 0, -1) > b.d2))
-        scan_range<COUNT>(g, __ldg(g.off + rk + cx - 1), __ldg(g.off + rk + cx), q.x, q.y, q.z, b, nc);
-      if (cx < G - 1 && !(axis_lb(fb, 0, 1) > b.d2))
-        scan_range<COUNT>(g, __ldg(g.off + rk + cx + 1), __ldg(g.off + rk + cx + 2), q.x, q.y, q.z, b, nc);
-      // the other 8 x-rows: the 4 sharing a face with the query's row, then the 4 diagonal
-      for (int k = 0; k < 8; ++k) {
-        int dy, dz;
-        if (k < 4) {
-          dy = k < 2 ? (k & 1 ? 1 : -1) : 0;
-          dz = k < 2 ? 0 : (k & 1 ? 1 : -1);
-        } else {
-          dy = k & 1 ? 1 : -1;
-          dz = k & 2 ? 1 : -1;
-        }
-        const int yy = cy + dy, zz = cz + dz;
-        if (yy < 0 || yy >= G || zz < 0 || zz >= G) continue;
-        const float lyz = axis_lb(fb, 1, dy) + axis_lb(fb, 2, dz);
-        if (lyz > b.d2) continue;
-        const int x0 = cx > 0 && !(lyz + axis_lb(fb, 0, -1) > b.d2) ? cx - 1 : cx;
-        const int x1 = cx < G - 1 && !(lyz + axis_lb(fb, 0, 1) > b.d2) ? cx + 1 : cx;
-        rk = base + row_key(yy, zz, g.bits);
-        scan_range<COUNT>(g, __ldg(g.off + rk + x0), __ldg(g.off + rk + x1 + 1), q.x, q.y, q.z, b, nc);
-      }
-    }
-    int r = 1;
-    bool done = b.d2 < outside_bound2(g, q.x, q.y, q.z, cx, cy, cz, 1);
-    while (!done && r < NN_RTHREAD) {
-      ++r;
-      for (int dz = -r; dz <= r; ++dz)
-        for (int dy = -r; dy <= r; ++dy)
-          scan_shell_row<COUNT>(g, base, G, cx, cy, cz, r, dy, dz, q.x, q.y, q.z, fb, FLT_MAX, b, nc);
-      done = b.d2 < outside_bound2(g, q.x, q.y, q.z, cx, cy, cz, r);
-    }
-    if (COUNT) count_candidates(J, j, nc);
-    if (done) {
-      finalize<COUNT>(J, q, b);
-    } else {  // ring reached in the low 16 bits, the tie flag above them
-      const int slot = atomicAdd(J.hard_count, 1);
-      J.hard[slot] = make_int4(item, r | (COUNT && b.tie ? 0x10000 : 0), __float_as_int(b.d2), b.idx);
-    }
-  }
-}
-
-// ------------------------------------------------------------------------------ warp pass
-
-__device__ __forceinline__ unsigned long long pack(const Best& b) {
-  return ((unsigned long long)__float_as_uint(b.d2) << 32) | (unsigned)b.idx;
-}
-
-// lexicographic (d2, idx) minimum over the warp; every lane receives it
-template <bool COUNT>
-__device__ __forceinline__ Best warp_min(const Best& b) {
-  unsigned long long m = pack(b);
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    const unsigned long long t = __shfl_xor_sync(0xffffffffu, m, o);
-    m = t < m ? t : m;
-  }
-  Best r;
-  r.d2 = __uint_as_float((unsigned)(m >> 32));
-  r.idx = (int)(unsigned)(m & 0xffffffffu);
-  // an exact tie: a lane saw a tie at the minimum, or another lane's best has the same
-  // distance with another index
-  r.tie = COUNT && __any_sync(0xffffffffu, b.d2 == r.d2 && (b.tie || b.idx != r.idx));
+__device__ __forceinline__ Box load_box(const float4* b, int i) {
+  Box r;
+  r.a = __ldg(b + 2 * i);
+  r.c = __ldg(reinterpret_cast<const float2*>(b + 2 * i + 1));
   return r;
 }
 
-template <bool COUNT>
-__global__ void __launch_bounds__(256) k_nn_hard(const Plan* __restrict__ P) {
-  __shared__ int hpre[MAXJ + 1];
-  const int nj = P->n_jobs;
-  if (threadIdx.x == 0) {
-    int acc = 0;
-    for (int j = 0; j < nj; ++j) {
-      hpre[j] = acc;
-      acc += *P->jobs[j]->hard_count;
-    }
-    hpre[nj] = acc;
-    if (blockIdx.x == 0)
-      for (int j = 0; j < nj; ++j) P->jobs[j]->counters[CNT_NN_HARD] = (unsigned long long)(hpre[j + 1] - hpre[j]);
-  }
-  __syncthreads();
-  const int total = hpre[nj];
-  const int lane = threadIdx.x & 31;
-  const int nwarps = (gridDim.x * blockDim.x) >> 5;
-  for (int w = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; w < total; w += nwarps) {
-    int lo = 0, hi = nj;
-    while (hi - lo > 1) {
-      const int mid = (lo + hi) >> 1;
-      if (hpre[mid] <= w) lo = mid; else hi = mid;
-    }
-    const Job& J = *P->jobs[lo];
-    const int4 h = J.hard[w - hpre[lo]];
-    const QueryRef q = resolve(J, h.x);
-    const CellGrid& g = q.fwd ? J.tgt : J.mov;
-    const int G = 1 << g.bits;
-    const int base = q.set * G * G * G;
-    const int cx = cell_coord(q.x, g.lo[0], g.inv_h[0], G);
-    const int cy = cell_coord(q.y, g.lo[1], g.inv_h[1], G);
-    const int cz = cell_coord(q.z, g.lo[2], g.inv_h[2], G);
-    const FaceBounds fb = face_bounds(g, q.x, q.y, q.z, cx, cy, cz);
-    // continue from the thread pass: its best is lane 0's starting candidate, and the best
-    // of the warp after each ring bounds what every lane still has to look at
-    Best b{FLT_MAX, 0x7fffffff, false};
-    if (lane == 0) {
-      b.d2 = __int_as_float(h.z);
-      b.idx = h.w;
-      b.tie = (h.y & 0x10000) != 0;
-    }
-    Best best{__int_as_float(h.z), h.w, false};
-    bool done = false;
-    int nc = 0;
-    for (int r = (h.y & 0xffff) + 1; r <= NN_RMAX && !done; ++r) {
-      const int side = 2 * r + 1;
-      for (int ri = lane; ri < side * side; ri += 32)
-        scan_shell_row<COUNT>(g, base, G, cx, cy, cz, r, ri % side - r, ri / side - r, q.x, q.y, q.z, fb, best.d2,
-                              b, nc);
-      best = warp_min<COUNT>(b);
-      done = best.d2 < outside_bound2(g, q.x, q.y, q.z, cx, cy, cz, r);
-    }
-    if (!done) {  // exhaustive scan of the set
-      const int s = __ldg(g.off + base), e = __ldg(g.off + base + G * G * G);
-      for (int k = s + lane; k < e; k += 32) consider<COUNT>(b, __ldg(g.pts + k), q.x, q.y, q.z);
-      if (COUNT) nc += (e - s + 31 - lane) / 32;
-      best = warp_min<COUNT>(b);
-    }
-    if (COUNT) {
-      const unsigned s = __reduce_add_sync(0xffffffffu, (unsigned)nc);
-      if (lane == 0) atomicAdd(J.counters + CNT_NN_CANDIDATES, (unsigned long long)s);
-    }
-    if (lane == 0) finalize<COUNT>(J, q, best);
+// fp32 lower bound on sqdist between any point in [l, h] and any point of the box
+__device__ __forceinline__ float box_lb(const Box& b, float lx, float ly, float lz, float hx, float hy, float hz) {
+  const float dx = fmaxf(fmaxf(__fsub_rn(b.a.x, hx), __fsub_rn(lx, b.a.w)), 0.f);
+  const float dy = fmaxf(fmaxf(__fsub_rn(b.a.y, hy), __fsub_rn(ly, b.c.x)), 0.f);
+  const float dz = fmaxf(fmaxf(__fsub_rn(b.a.z, hz), __fsub_rn(lz, b.c.y)), 0.f);
+  return __fmaf_rn(dz, dz, __fmaf_rn(dy, dy, __fmul_rn(dx, dx)));
+}
+
+// minimum / maximum over the warp (signed floats as order-preserving integers)
+__device__ __forceinline__ int ord(float f) {
+  const int i = __float_as_int(f);
+  return i < 0 ? i ^ 0x7fffffff : i;
+}
+__device__ __forceinline__ float warp_min(float f) {
+  const int m = __reduce_min_sync(0xffffffffu, ord(f));
+  return __int_as_float(m < 0 ? m ^ 0x7fffffff : m);
+}
+__device__ __forceinline__ float warp_max(float f) {
+  const int m = __reduce_max_sync(0xffffffffu, ord(f));
+  return __int_as_float(m < 0 ? m ^ 0x7fffffff : m);
+}
+
+// ------------------------------------------------------------------------------ leaves
+
+typedef unsigned long long f32x2;
+__device__ __forceinline__ f32x2 pack2(float a, float b) {
+  f32x2 r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
+  return r;
+}
+__device__ __forceinline__ float2 unpack2(f32x2 v) {
+  float2 r;
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(v));
+  return r;
+}
+__device__ __forceinline__ f32x2 add2(f32x2 a, f32x2 b) {
+  f32x2 r;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ f32x2 mul2(f32x2 a, f32x2 b) {
+  f32x2 r;
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ f32x2 fma2(f32x2 a, f32x2 b, f32x2 c) {
+  f32x2 r;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+  return r;
+}
+
+// Squared distances to the 8 points of a leaf, bitwise sqdist (its differences only change sign)
+struct NegQuery {
+  f32x2 x, y, z;  // (-q, -q) per axis
+};
+__device__ __forceinline__ void leaf_d2(const float* pts, int leaf, const NegQuery& q, float (&d)[LEAF]) {
+  const ulonglong2* p = reinterpret_cast<const ulonglong2*>(pts + (size_t)leaf * (3 * LEAF));
+  const ulonglong2 xa = __ldg(p), xb = __ldg(p + 1), ya = __ldg(p + 2), yb = __ldg(p + 3), za = __ldg(p + 4),
+                   zb = __ldg(p + 5);
+  const f32x2 x[4] = {xa.x, xa.y, xb.x, xb.y}, y[4] = {ya.x, ya.y, yb.x, yb.y}, z[4] = {za.x, za.y, zb.x, zb.y};
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    const f32x2 dx = add2(x[k], q.x), dy = add2(y[k], q.y), dz = add2(z[k], q.z);
+    const float2 s = unpack2(fma2(dz, dz, fma2(dy, dy, mul2(dx, dx))));
+    d[2 * k] = s.x;
+    d[2 * k + 1] = s.y;
   }
 }
 
-void launch_nn(const Plan* P, int grid, cudaStream_t s, bool count) {
-  if (count) k_nn<true><<<grid, 256, 0, s>>>(P);
-  else k_nn<false><<<grid, 256, 0, s>>>(P);
+// lowest index among a leaf's points at squared distance d2 (and how many there are)
+__device__ __forceinline__ int leaf_index(const Tree& T, int leaf, const NegQuery& q, float d2, int& count) {
+  float d[LEAF];
+  leaf_d2(T.pts, leaf, q, d);
+  int id = 0x7fffffff;
+  count = 0;
+#pragma unroll
+  for (int k = 0; k < LEAF; ++k)
+    if (d[k] == d2) {
+      id = min(id, __ldg(T.perm + leaf * LEAF + k));
+      ++count;
+    }
+  return id;
 }
-void launch_nn_hard(const Plan* P, int grid, cudaStream_t s, bool count) {
-  if (count) k_nn_hard<true><<<grid, 256, 0, s>>>(P);
-  else k_nn_hard<false><<<grid, 256, 0, s>>>(P);
+
+// Best so far of a lane: d2, and the leaf that holds a point at that distance (-1: none yet).
+// tie: another leaf holds an equally near point.
+struct Best {
+  float d2;
+  int leaf;
+  bool tie;
+};
+
+__device__ __forceinline__ void eval_leaf(const Tree& T, int leaf, const NegQuery& q, Best& b) {
+  float d[LEAF];
+  leaf_d2(T.pts, leaf, q, d);
+  const float m = fminf(fminf(fminf(d[0], d[1]), fminf(d[2], d[3])), fminf(fminf(d[4], d[5]), fminf(d[6], d[7])));
+  if (m < b.d2) {
+    b.d2 = m;
+    b.leaf = leaf;
+    b.tie = false;
+  } else if (m == b.d2 && b.leaf >= 0 && leaf != b.leaf) {  // an exact tie: keep the leaf with the lower index
+    int c;
+    if (leaf_index(T, leaf, q, m, c) < leaf_index(T, b.leaf, q, m, c)) b.leaf = leaf;
+    b.tie = true;
+  }
+}
+
+// ------------------------------------------------------------------------------ search
+
+struct WarpBox {
+  float lx, ly, lz, hx, hy, hz;
+};
+
+// A warp's traversal.  SUB lanes share a query (lane = sub (32 / SUB) + query): each takes other leaves,
+// and their results are merged at the end.
+template <int SUB, bool COUNT>
+struct Search {
+  static constexpr int QPW = 32 / SUB, LIST = 64;
+  const Tree& T;
+  QueryRef q;
+  NegQuery nq;
+  WarpBox w;
+  Best b;
+  float lim;   // no worse than the best distance of the query's lanes: what is farther is skipped
+  float wmax;  // largest lim of the warp
+  int* list;   // the warp's list of leaves to look at
+  int n;
+  int nc;      // candidates evaluated by this lane (counting instance)
+
+  __device__ __forceinline__ void update_limits() {
+    lim = fminf(lim, b.d2);
+#pragma unroll
+    for (int o = QPW; o < 32; o <<= 1) lim = fminf(lim, __shfl_xor_sync(0xffffffffu, lim, o));
+    wmax = __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(fmaxf(lim, 0.f))));
+  }
+
+  __device__ __forceinline__ bool wanted(int leaf) const {
+    return box_lb(load_box(T.lbox, leaf), q.x, q.y, q.z, q.x, q.y, q.z) <= lim;
+  }
+
+  // looks at the listed leaves, one per sub-lane at a time
+  __device__ __forceinline__ void flush() {
+    __syncwarp();
+#pragma unroll 1
+    for (int i = 0; i < n; i += SUB) {
+      const int k = i + threadIdx.x % 32 / QPW;
+      const int leaf = list[min(k, n - 1)];
+      if (k < n && wanted(leaf)) {
+        eval_leaf(T, leaf, nq, b);
+        lim = fminf(lim, b.d2);
+        if (COUNT) nc += LEAF;
+      }
+    }
+    __syncwarp();
+    n = 0;
+    update_limits();
+  }
+
+  // lists the leaves of a node that the warp's box may need
+  __device__ __forceinline__ void node(int nd) {
+    const int lane = threadIdx.x & 31;
+    const bool in = box_lb(load_box(T.lbox, nd * 32 + lane), w.lx, w.ly, w.lz, w.hx, w.hy, w.hz) <= wmax;
+    const unsigned m = __ballot_sync(0xffffffffu, in);
+    if (in) list[n + __popc(m & ((1u << lane) - 1u))] = nd * 32 + lane;
+    n += __popc(m);
+    if (n > LIST - 32) flush();
+  }
+};
+
+// items: SUB warps for each 32 queries (ST_NNF: moving slots, template set first; ST_NNR: target
+// slots, searched in the tree of the moving set `set`)
+template <bool FWD, int SUB, bool COUNT>
+__global__ void __launch_bounds__(NN_THREADS, 8) k_nn(const Plan* __restrict__ P, int set) {
+  constexpr int ST = FWD ? ST_NNF : ST_NNR, QPW = 32 / SUB;
+  __shared__ int lists[NN_THREADS / 32][Search<SUB, COUNT>::LIST];
+  const int nj = P->n_jobs;
+  const int total = P->pre[ST][nj] * SUB;
+  const int lane = threadIdx.x & 31;
+  for (int it = (blockIdx.x * NN_THREADS + threadIdx.x) >> 5; it < total; it += gridDim.x * (NN_THREADS / 32)) {
+    const int j = find_job(P->pre[ST], nj, it / SUB);
+    const Job& J = *P->jobs[j];
+    const int t = it / SUB - P->pre[ST][j];
+    const Tree& own = FWD ? J.mov : J.tgt;
+    Search<SUB, COUNT> s{FWD ? J.tgt : J.mov};
+    QueryRef& q = s.q;
+    q.set = FWD ? 0 : set;
+    int slot = 32 * t + it % SUB * QPW + lane % QPW;
+    if (FWD) {
+      const int w0 = (J.V + 31) / 32;
+      if (t >= w0) slot += mov_set(J, 1).slot0 - 32 * w0;
+    }
+    const SetRange r = FWD ? set_range(0, 0, J.M) : mov_set(J, q.set);
+    const float* p = own.pts + (size_t)(slot / LEAF) * (3 * LEAF) + slot % LEAF;
+    q.id = own.perm[slot];
+    q.x = p[0];
+    q.y = p[LEAF];
+    q.z = p[2 * LEAF];
+    // a query with a NaN coordinate has no nearest point; like a padding lane it asks for nothing
+    const bool live = q.id >= 0 && q.x == q.x && q.y == q.y && q.z == q.z;
+    s.b = Best{live ? FLT_MAX : -1.f, -1, false};
+    if (live) {
+      // Warm start: the distance of the previous step's neighbour (k_nn_seed's point in a frame's first
+      // step) at its current position, one ulp up, so that its own leaf counts as an improvement and
+      // records itself.
+      const int w = FWD ? J.nn_fwd[q.id] : J.nn_rev[q.set * J.M + q.id];
+      if (w >= 0) {
+        const float4 c = FWD ? J.tgt4[w] : J.y[w + (q.set ? J.V : 0)];
+        const float d2 = sqdist(q.x, q.y, q.z, c.x, c.y, c.z);
+        if (d2 < FLT_MAX) s.b.d2 = __uint_as_float(__float_as_uint(d2) + 1u);
+      }
+    }
+    s.nq = NegQuery{pack2(-q.x, -q.x), pack2(-q.y, -q.y), pack2(-q.z, -q.z)};
+    const float inf = __int_as_float(0x7f800000);
+    WarpBox& w = s.w;
+    w.lx = warp_min(live ? q.x : inf);
+    w.ly = warp_min(live ? q.y : inf);
+    w.lz = warp_min(live ? q.z : inf);
+    w.hx = warp_max(live ? q.x : -inf);
+    w.hy = warp_max(live ? q.y : -inf);
+    w.hz = warp_max(live ? q.z : -inf);
+    s.list = lists[threadIdx.x >> 5];
+    s.n = s.nc = 0;
+    s.lim = s.b.d2;
+    s.update_limits();
+    if (__any_sync(0xffffffffu, live)) {
+      for (int s0 = 0; s0 < r.supers; s0 += 32) {
+        float lbs = inf;
+        if (s0 + lane < r.supers)
+          lbs = box_lb(load_box(s.T.sbox, r.super0 + s0 + lane), w.lx, w.ly, w.lz, w.hx, w.hy, w.hz);
+        unsigned ms = __ballot_sync(0xffffffffu, lbs <= s.wmax);
+        while (ms) {
+          const int sn = s0 + __ffs(ms) - 1;
+          ms &= ms - 1;
+          float lbn = inf;
+          if (32 * sn + lane < r.nodes)
+            lbn = box_lb(load_box(s.T.nbox, r.node0 + 32 * sn + lane), w.lx, w.ly, w.lz, w.hx, w.hy, w.hz);
+          unsigned mn = __ballot_sync(0xffffffffu, lbn <= s.wmax);
+          while (mn) {
+            const int nd = r.node0 + 32 * sn + __ffs(mn) - 1;
+            mn &= mn - 1;
+            // the warp's box can be much larger than its queries (a jump of the curve): ask the lanes
+            const Box box = load_box(s.T.nbox, nd);
+            if (__any_sync(0xffffffffu, box_lb(box, q.x, q.y, q.z, q.x, q.y, q.z) <= s.lim)) s.node(nd);
+          }
+        }
+      }
+      if (s.n) s.flush();
+    }
+    if (COUNT) {
+      const unsigned c = __reduce_add_sync(0xffffffffu, q.id >= 0 ? (unsigned)s.nc : 0u);
+      if (lane == 0) atomicAdd(J.counters + CNT_NN_CANDIDATES, (unsigned long long)c);
+    }
+    int idx = -1;
+    bool tie = s.b.tie;
+    if (s.b.leaf >= 0) {
+      int count;
+      idx = leaf_index(s.T, s.b.leaf, s.nq, s.b.d2, count);
+      tie = tie || count > 1;
+    }
+    float d2 = idx >= 0 ? s.b.d2 : inf;
+#pragma unroll
+    for (int o = QPW; o < 32; o <<= 1) {  // the lexicographic minimum over the query's lanes
+      const float d = __shfl_xor_sync(0xffffffffu, d2, o);
+      const int i = __shfl_xor_sync(0xffffffffu, idx, o);
+      const bool ti = __shfl_xor_sync(0xffffffffu, tie, o);
+      if (i >= 0 && (d < d2 || idx < 0)) {
+        d2 = d;
+        idx = i;
+        tie = ti;
+      } else if (i >= 0 && d == d2) {
+        tie = tie || ti || i != idx;
+        idx = min(idx, i);
+      }
+    }
+    if (q.id >= 0 && lane < QPW) {
+      if (COUNT && idx >= 0 && tie) atomicAdd(J.counters + CNT_NN_TIES, 1ull);
+      finalize<FWD>(J, q, d2, idx);
+    }
+    __syncwarp();
+  }
+}
+
+// A frame's first neighbours: a point of the query's own cell of the searched set's sort, or the next
+// one along the curve where that cell is empty.  Any point of the set will do; without one the first
+// step's searches would start from no bound (first evaluation at 100k points: about 100 us more).
+__global__ void k_nn_seed(Job* __restrict__ Jp) {
+  const Job& J = *Jp;
+  const int total = J.Q + (J.N > 0 ? 2 : 1) * J.M;
+  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < total; i += gridDim.x * blockDim.x) {
+    if (i < J.Q) {
+      const float4 x = J.x[i];
+      J.nn_fwd[i] = J.tgt.perm[min(J.tgt.off[cell_key(J.tgt, x.x, x.y, x.z, 0)], J.M - 1)];
+    } else {
+      const int set = i - J.Q >= J.M, t = i - J.Q - set * J.M;
+      const float4 x = J.tgt4[t];
+      const SetRange r = mov_set(J, set);
+      const int pos = J.mov.off[cell_key(J.mov, x.x, x.y, x.z, set)] - (set ? J.V : 0);
+      J.nn_rev[i - J.Q] = J.mov.perm[r.slot0 + min(pos, r.n - 1)] - (set ? J.V : 0);
+    }
+  }
+}
+
+void launch_nn_seed(Job* J, const Job& hJ, cudaStream_t s) {
+  const int n = hJ.Q + 2 * hJ.M;
+  k_nn_seed<<<std::min((n + 255) / 256, 4096), 256, 0, s>>>(J);
+}
+
+template <int SUB>
+static void launch_nn_sub(const Plan* P, int grid, cudaStream_t s, int set, bool count) {
+  if (set < 0 && count) k_nn<true, SUB, true><<<grid, NN_THREADS, 0, s>>>(P, 0);
+  else if (set < 0) k_nn<true, SUB, false><<<grid, NN_THREADS, 0, s>>>(P, 0);
+  else if (count) k_nn<false, SUB, true><<<grid, NN_THREADS, 0, s>>>(P, set);
+  else k_nn<false, SUB, false><<<grid, NN_THREADS, 0, s>>>(P, set);
+}
+
+void launch_nn(const Plan* P, int grid, cudaStream_t s, int set, int sub, bool count) {
+  if (sub == 2) launch_nn_sub<2>(P, grid, s, set, count);
+  else launch_nn_sub<8>(P, grid, s, set, count);
 }
 
 }  // namespace pdg

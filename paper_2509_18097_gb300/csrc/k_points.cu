@@ -11,11 +11,9 @@ namespace pdg {
 // bump = 1: a new optimisation step (advances the Adam step count and its bias corrections
 // and clears the per-step counters); bump = 2: an evaluation (clears the counters only).
 __device__ __forceinline__ void job_bump(const Job& J, int bump) {
-  *J.hard_count = 0;
   *J.gmax = 0u;
   J.counters[CNT_NN_CANDIDATES] = 0ull;
   J.counters[CNT_NN_TIES] = 0ull;
-  J.counters[CNT_NN_HARD] = 0ull;
   if (bump == 1) {
     const int k = *J.step + 1;
     *J.step = k;
@@ -33,13 +31,15 @@ __global__ void k_plan(Plan* P) {
   const int nj = P->n_jobs;
   for (int j = threadIdx.x; j < nj; j += blockDim.x) {
     Job* J = P->jobs[j];
-    const int G = 1 << J->mov.bits;
     cnt[ST_Q][j] = J->Q;
     // reverse queries into the source set only when there is one (a template-mesh fit has none)
     const int nrs = J->N > 0 ? 2 : 1;
-    cnt[ST_NNQ][j] = J->Q + nrs * J->M;
+    const SetRange s0 = mov_set(*J, 0), s1 = mov_set(*J, 1);
+    cnt[ST_NODE][j] = s0.nodes + s1.nodes;
+    cnt[ST_SUPER][j] = s0.supers + s1.supers;
+    cnt[ST_NNF][j] = (J->V + 31) / 32 + (J->N + 31) / 32;  // warps of 32 queries
+    cnt[ST_NNR][j] = (J->M + 31) / 32;  // per moving set
     cnt[ST_E][j] = J->E;
-    cnt[ST_MOVCH][j] = (2 * G * G * G + SCAN_CHUNK - 1) / SCAN_CHUNK;
     int a = 0, t = 0, xt = 0, p3 = 0, cols = 0, ad = 0;
     int aw = 0;
     // the levels' loads are independent: issue them level-parallel (a dependent chain of
@@ -53,7 +53,7 @@ __global__ void k_plan(Plan* P) {
 #pragma unroll
     for (int l = 0; l < MAXL; ++l) {
       if (l >= L) break;
-      // adjoint (in blocks of 8 warps): 2^adj_lg lanes per row, 8 to 16 entries per lane
+      // adjoint: 2^adj_lg lanes per row, 8 to 16 entries per lane
       // (a row holds one entry per point in the 8 cells around its vertex: a few dozen on
       // fine levels, thousands on coarse ones), so a warp sums 32 >> adj_lg rows; rows of
       // 512 entries or more on average (adj_lg = 6) get a whole block each
@@ -75,7 +75,8 @@ __global__ void k_plan(Plan* P) {
         ad += (J->lev[l].n3 + 3) >> 2;
       }
     }
-    cnt[ST_ADJ][j] = a + ((aw + 7) >> 3);
+    cnt[ST_ADJROW][j] = a;
+    cnt[ST_ADJ][j] = aw;
     cnt[ST_TILE][j] = t;
     cnt[ST_XTILE][j] = xt;
     cnt[ST_PLANE][j] = J->C * p3;
@@ -175,49 +176,73 @@ __device__ __forceinline__ float3 deform_point(const Job& J, float3 x, float3& z
   return make_float3(2.f * u.x - x.x + t.x, 2.f * u.y - x.y + t.y, 2.f * u.z - x.z + t.z);
 }
 
-// y = x + u(x) on Q; the cell key of y in the moving grid (set 0: template, set 1: source)
-// and its count; clears the point's fixed-point reverse-Chamfer accumulator.  The thread of
-// a job's first point also starts the job's step (job_bump; bump 0: none).  Points are taken
-// in the finest level's cell order (the per-frame sort of the adjoint), so the lanes of a
-// warp interpolate between the same or neighbouring grid vertices.
-__global__ void k_interp(const Plan* __restrict__ P, int bump) {
+// y = x + u(x) on Q, in the slot order of the moving tree: a block takes one node, so the lanes of
+// a warp interpolate between the same or neighbouring grid vertices, and stores the node's points
+// and boxes on the way; clears the point's fixed-point reverse-Chamfer accumulator.  The thread of
+// a job's first slot also starts the job's step (job_bump; bump 0: none).
+__global__ void __launch_bounds__(NODE) k_interp(const Plan* __restrict__ P, int bump) {
   const int nj = P->n_jobs;
-  const int total = P->pre[ST_Q][nj];
-  for (int it = blockIdx.x * blockDim.x + threadIdx.x; it < total; it += gridDim.x * blockDim.x) {
-    const int j = find_job(P->pre[ST_Q], nj, it);
+  const int total = P->pre[ST_NODE][nj];
+  for (int it = blockIdx.x; it < total; it += gridDim.x) {
+    const int j = find_job(P->pre[ST_NODE], nj, it);
     const Job& J = *P->jobs[j];
-    const int p = __float_as_int(__ldg(&J.lev[J.L - 1].xs[it - P->pre[ST_Q][j]].w));
-    if (bump && p == 0) job_bump(J, bump);
-    const float4 x = J.x[p];
-    float3 z, u;
-    const float3 yy = deform_point(J, make_float3(x.x, x.y, x.z), z, u);
-    const float4 y = make_float4(yy.x, yy.y, yy.z, 0.f);
-    J.y[p] = y;
-    if (J.C == 6) {
-      J.zq[p] = make_float4(z.x, z.y, z.z, 0.f);
-      J.uq[p] = make_float4(u.x, u.y, u.z, 0.f);
+    const int nd = it - P->pre[ST_NODE][j];
+    const int slot = nd * NODE + threadIdx.x;
+    if (bump && slot == 0) job_bump(J, bump);
+    const float4 x = __ldg(J.xs + slot);
+    const int p = __float_as_int(x.w);
+    float3 yy = make_float3(0.f, 0.f, 0.f);
+    if (p >= 0) {
+      float3 z, u;
+      yy = deform_point(J, make_float3(x.x, x.y, x.z), z, u);
+      J.y[p] = make_float4(yy.x, yy.y, yy.z, 0.f);
+      if (J.C == 6) {
+        J.zq[p] = make_float4(z.x, z.y, z.z, 0.f);
+        J.uq[p] = make_float4(u.x, u.y, u.z, 0.f);
+      }
+      J.acc[3 * p + 0] = 0;
+      J.acc[3 * p + 1] = 0;
+      J.acc[3 * p + 2] = 0;
     }
-    const int key = cell_key(J.mov, y.x, y.y, y.z, p < J.V ? 0 : 1);
-    J.mov.keys[p] = key;
-    atomicAdd(&J.mov.hist[key], 1);
-    J.acc[3 * p + 0] = 0;
-    J.acc[3 * p + 1] = 0;
-    J.acc[3 * p + 2] = 0;
+    store_node(J.mov, nd, yy.x, yy.y, yy.z, p >= 0);
   }
 }
 
-// scatter of the moving points into key order (counts return to zero)
-__global__ void k_mov_scatter(const Plan* __restrict__ P) {
+// boxes of 32 nodes [node0 + 32 s, node0 + nodes) of a set, by one warp
+__device__ __forceinline__ void super_box(const Tree& T, const SetRange& r, int s) {
+  const int lane = threadIdx.x & 31;
+  const float inf = __int_as_float(0x7f800000);
+  const int nd = 32 * s + lane;
+  float4 a = make_float4(inf, inf, inf, -inf), c = make_float4(-inf, -inf, 0.f, 0.f);
+  if (nd < r.nodes) {
+    a = T.nbox[2 * (r.node0 + nd)];
+    c = T.nbox[2 * (r.node0 + nd) + 1];
+  }
+  float b[6] = {a.x, a.y, a.z, a.w, c.x, c.y};
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1)
+#pragma unroll
+    for (int k = 0; k < 6; ++k) {
+      const float v = __shfl_xor_sync(0xffffffffu, b[k], o);
+      b[k] = k < 3 ? fminf(b[k], v) : fmaxf(b[k], v);
+    }
+  if (lane == 0) {
+    T.sbox[2 * (r.super0 + s)] = make_float4(b[0], b[1], b[2], b[3]);
+    T.sbox[2 * (r.super0 + s) + 1] = make_float4(b[4], b[5], 0.f, 0.f);
+  }
+}
+
+// super-node boxes of the moving trees, a warp each
+__global__ void __launch_bounds__(64) k_boxes(const Plan* __restrict__ P) {
   const int nj = P->n_jobs;
-  const int total = P->pre[ST_Q][nj];
-  for (int it = blockIdx.x * blockDim.x + threadIdx.x; it < total; it += gridDim.x * blockDim.x) {
-    const int j = find_job(P->pre[ST_Q], nj, it);
+  const int total = P->pre[ST_SUPER][nj];
+  for (int it = blockIdx.x * 2 + (threadIdx.x >> 5); it < total; it += gridDim.x * 2) {
+    const int j = find_job(P->pre[ST_SUPER], nj, it);
     const Job& J = *P->jobs[j];
-    const int p = it - P->pre[ST_Q][j];
-    const int key = J.mov.keys[p];
-    const int pos = J.mov.off[key] + atomicSub(&J.mov.hist[key], 1) - 1;
-    const float4 y = J.y[p];
-    J.mov.pts[pos] = make_float4(y.x, y.y, y.z, __int_as_float(p));
+    const int s = it - P->pre[ST_SUPER][j];
+    const SetRange r0 = mov_set(J, 0);
+    if (s < r0.supers) super_box(J.mov, r0, s);
+    else super_box(J.mov, mov_set(J, 1), s - r0.supers);
   }
 }
 
@@ -408,6 +433,7 @@ __global__ void k_frame_points(Job* J) {
   }
 }
 
+// Tree builds (per frame): cell keys and counts, scatter of the indices into slot order
 __global__ void k_tgt_keys(Job* J) {
   for (int p = blockIdx.x * blockDim.x + threadIdx.x; p < J->M; p += gridDim.x * blockDim.x) {
     const float4 t = J->tgt4[p];
@@ -420,9 +446,52 @@ __global__ void k_tgt_keys(Job* J) {
 __global__ void k_tgt_scatter(Job* J) {
   for (int p = blockIdx.x * blockDim.x + threadIdx.x; p < J->M; p += gridDim.x * blockDim.x) {
     const int key = J->tgt.keys[p];
-    const int pos = J->tgt.off[key] + atomicSub(&J->tgt.hist[key], 1) - 1;
-    const float4 t = J->tgt4[p];
-    J->tgt.pts[pos] = make_float4(t.x, t.y, t.z, __int_as_float(p));
+    J->tgt.perm[J->tgt.off[key] + atomicSub(&J->tgt.hist[key], 1) - 1] = p;
+  }
+}
+
+// target points and boxes, a block per node
+__global__ void __launch_bounds__(NODE) k_tgt_nodes(Job* J) {
+  const int nodes = (J->M + NODE - 1) / NODE;
+  for (int nd = blockIdx.x; nd < nodes; nd += gridDim.x) {
+    const int slot = nd * NODE + threadIdx.x;
+    const bool in = slot < J->M;
+    if (!in) J->tgt.perm[slot] = -1;
+    const float4 t = in ? J->tgt4[J->tgt.perm[slot]] : make_float4(0.f, 0.f, 0.f, 0.f);
+    store_node(J->tgt, nd, t.x, t.y, t.z, in);
+  }
+}
+
+__global__ void __launch_bounds__(32) k_tgt_boxes(Job* J) {
+  const SetRange r = set_range(0, 0, J->M);
+  for (int s = blockIdx.x; s < r.supers; s += gridDim.x) super_box(J->tgt, r, s);
+}
+
+__global__ void k_mov_keys(Job* J) {
+  for (int p = blockIdx.x * blockDim.x + threadIdx.x; p < J->Q; p += gridDim.x * blockDim.x) {
+    const float4 x = J->x[p];
+    const int key = cell_key(J->mov, x.x, x.y, x.z, p < J->V ? 0 : 1);
+    J->mov.keys[p] = key;
+    atomicAdd(&J->mov.hist[key], 1);
+  }
+}
+
+__global__ void k_mov_scatter(Job* J) {
+  const SetRange r0 = mov_set(*J, 0), r1 = mov_set(*J, 1);
+  const int i0 = blockIdx.x * blockDim.x + threadIdx.x, step = gridDim.x * blockDim.x;
+  for (int p = i0; p < J->Q; p += step) {
+    const int key = J->mov.keys[p];
+    const int pos = J->mov.off[key] + atomicSub(&J->mov.hist[key], 1) - 1;
+    const int slot = p < J->V ? pos : r1.slot0 + pos - J->V;
+    const float4 x = J->x[p];
+    J->xs[slot] = make_float4(x.x, x.y, x.z, __int_as_float(p));
+    J->mov.perm[slot] = p;
+  }
+  const int pad0 = r0.nodes * NODE - r0.n, pad1 = r1.nodes * NODE - r1.n;
+  for (int i = i0; i < pad0 + pad1; i += step) {
+    const int slot = i < pad0 ? r0.n + i : r1.slot0 + r1.n + i - pad0;
+    J->xs[slot] = make_float4(0.f, 0.f, 0.f, __int_as_float(-1));
+    J->mov.perm[slot] = -1;
   }
 }
 
@@ -453,7 +522,7 @@ static inline int blocks_for(int n, int threads) { return max(1, min((n + thread
 
 void launch_plan(Plan* P, cudaStream_t s) { k_plan<<<1, 256, 0, s>>>(P); }
 void launch_interp(const Plan* P, int grid, cudaStream_t s, int bump) { k_interp<<<grid, 256, 0, s>>>(P, bump); }
-void launch_mov_scatter(const Plan* P, int grid, cudaStream_t s) { k_mov_scatter<<<grid, 256, 0, s>>>(P); }
+void launch_boxes(const Plan* P, int grid, cudaStream_t s) { k_boxes<<<grid, 64, 0, s>>>(P); }
 void launch_iso_edges(const Plan* P, int grid, cudaStream_t s) { k_iso_edges<<<grid, 256, 0, s>>>(P); }
 void launch_assemble(const Plan* P, int grid, cudaStream_t s) { k_assemble<<<grid, 256, 0, s>>>(P); }
 void launch_loss(const Plan* P, int grid, cudaStream_t s) {
@@ -530,13 +599,23 @@ void launch_copy_int(const int* in, int* out, int n, cudaStream_t s) {
   k_copy_int<<<blocks_for(n, 256), 256, 0, s>>>(in, out, n);
 }
 
-// target cell grid of the frame: keys + counts, exclusive scan, scatter
+// target tree of the frame: keys + counts, exclusive scan, scatter, boxes
 void launch_tgt_build(Job* J, const Job& hJ, cudaStream_t s) {
   k_tgt_keys<<<blocks_for(hJ.M, 256), 256, 0, s>>>(J);
-  const int G = 1 << hJ.tgt.bits;
-  ScanSeg seg{hJ.tgt.hist, hJ.tgt.off, G * G * G, hJ.tgt.csum};
+  ScanSeg seg{hJ.tgt.hist, hJ.tgt.off, 1 << (3 * hJ.tgt.bits), hJ.tgt.csum};
   launch_scan_segments(&seg, 1, nullptr, nullptr, s);
   k_tgt_scatter<<<blocks_for(hJ.M, 256), 256, 0, s>>>(J);
+  const SetRange r = set_range(0, 0, hJ.M);
+  k_tgt_nodes<<<min(r.nodes, 4096), NODE, 0, s>>>(J);
+  k_tgt_boxes<<<min(r.supers, 4096), 32, 0, s>>>(J);
+}
+
+// slot order of the moving sets for the frame (from x)
+void launch_mov_build(Job* J, const Job& hJ, cudaStream_t s) {
+  k_mov_keys<<<blocks_for(hJ.Q, 256), 256, 0, s>>>(J);
+  ScanSeg seg{hJ.mov.hist, hJ.mov.off, 2 << (3 * hJ.mov.bits), hJ.mov.csum};
+  launch_scan_segments(&seg, 1, nullptr, nullptr, s);
+  k_mov_scatter<<<blocks_for(hJ.Q, 256), 256, 0, s>>>(J);
 }
 
 }  // namespace pdg

@@ -9,13 +9,13 @@ namespace pdg {
 // per step (plan-driven; `grid` = blocks of the persistent launch)
 void launch_plan(Plan* P, cudaStream_t s);
 void launch_interp(const Plan* P, int grid, cudaStream_t s, int bump);
-void launch_mov_scan(const Plan* P, int grid, cudaStream_t s);
-void launch_mov_scatter(const Plan* P, int grid, cudaStream_t s);
-// count: the instance that counts candidates and exact ties
-void launch_nn(const Plan* P, int grid, cudaStream_t s, bool count);
-void launch_nn_hard(const Plan* P, int grid, cudaStream_t s, bool count);
+void launch_boxes(const Plan* P, int grid, cudaStream_t s);
+// set < 0: the moving points' searches in the target tree, else the targets' in the tree of a moving
+// set; sub: lanes per query (2 or 8); count: the instance that counts candidates and exact ties
+void launch_nn(const Plan* P, int grid, cudaStream_t s, int set, int sub, bool count);
 void launch_iso_edges(const Plan* P, int grid, cudaStream_t s);
 void launch_assemble(const Plan* P, int grid, cudaStream_t s);
+void launch_adjoint_rows(const Plan* P, int grid, cudaStream_t s);
 void launch_adjoint(const Plan* P, int grid, cudaStream_t s);
 // line path (256 and sizes with a factor 3); nmax: the largest level it takes in the plan
 enum YzPass { YZ_FWD = 0, YZ_Z, YZ_INV };
@@ -30,6 +30,8 @@ void launch_unpack4(const float4* in, float* out, int n, cudaStream_t s);
 void launch_check_finite(const float* in, int n, int* flag, cudaStream_t s);
 void launch_frame_points(Job* J, int Q, int E, cudaStream_t s);
 void launch_tgt_build(Job* J, const Job& hJ, cudaStream_t s);
+void launch_mov_build(Job* J, const Job& hJ, cudaStream_t s);
+void launch_nn_seed(Job* J, const Job& hJ, cudaStream_t s);
 void launch_csr_build(Job* J, const Job& hJ, cudaStream_t s);
 void launch_end_frame(Job* J, int V, cudaStream_t s);
 void launch_deform(const Job* J, const float* in, float* out, int n, cudaStream_t s);

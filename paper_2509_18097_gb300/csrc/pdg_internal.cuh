@@ -13,26 +13,29 @@ constexpr int MAXJ = 256;            // jobs (contexts) per batch
 constexpr int MAXL = PDG_MAX_LEVELS; // grid levels
 constexpr int SCAN_CHUNK = 4096;     // elements per scan chunk (1024 threads x 4)
 constexpr int SCAN_THREADS = 1024;
-constexpr int NN_RMAX = 8;           // ring radius after which a query is searched exhaustively
-constexpr int NN_RTHREAD = 2;        // rings searched by the one-thread-per-query pass
+constexpr int LEAF = 8;              // points per leaf of a point tree
+constexpr int NODE = 32 * LEAF;      // points per node (32 leaves); 32 nodes make a super node
 constexpr int LOSS_CHUNK = 2048;     // elements per loss-reduction chunk
 constexpr double FX_SCALE = 1099511627776.0;  // 2^40: fixed-point scale of the reverse Chamfer sums
 
-// A uniform cell grid over the domain used by the exact nearest-neighbour search.
-// G = 2^bits cells per axis.  Keys are (interleave(cy, cz) << bits) | cx, so the cells of
-// one x-row are contiguous and rows follow a 2-D Morton order in (y, z).  A grid may hold
-// `nsets` point sets in one key space (set s occupies keys [s G^3, (s+1) G^3)).
-struct CellGrid {
+// A static-order box tree over the points of one or two sets, searched by k_nn.cu.  A set's points
+// are sorted once per frame by the Hilbert index of their cell (`bits` per axis over the domain);
+// slots of NODE consecutive points form a node, 32 nodes a super node, LEAF points a leaf.  A set
+// starts on a node boundary, and its last node is padded with points at +infinity.  The order only
+// decides how tight the boxes are: the search is exact for any order and any coordinates.
+struct Tree {
   int bits;
-  int nsets;
   float lo[3];
-  float inv_h[3];  // G / (hi - lo)
-  float h[3];      // (hi - lo) / G
-  int* hist;       // [nsets G^3] per-cell counts; all zero between builds
-  int* off;        // [nsets G^3 + 1] exclusive prefix of hist
+  float inv_h[3];  // 2^bits / (hi - lo)
+  int* hist;       // [sets 8^bits] per-cell counts; all zero between builds
+  int* off;        // [sets 8^bits + 1] exclusive prefix of hist
   int* keys;       // [points] key of each point (scratch of the build)
-  float4* pts;     // [points] points sorted by key; .w = original index (int bits)
   int* csum;       // scan chunk sums scratch
+  int* perm;       // [slots] index of the slot's point, -1: padding
+  float* pts;      // [leaves][3][LEAF] coordinates
+  float4* lbox;    // [leaves][2] box of a leaf: (lo x, lo y, lo z, hi x), (hi y, hi z, -, -)
+  float4* nbox;    // [nodes][2]
+  float4* sbox;    // [super nodes][2], set 0 first
 };
 
 struct Level {
@@ -62,11 +65,6 @@ struct Level {
   int* act_v;     // [cap] active vertices (ascending)
   int* act_ptr;   // [cap + 1] entry range of each active vertex
   int2* ent;      // [8 Q] entries: (point, bits of the trilinear weight / L)
-  // finest level only: the query points in cell order, (iz (n-1) + iy)(n-1) + ix (per frame)
-  int* ccnt;      // [cells] points per cell (zero between builds)
-  int* coff;      // [cells + 1] exclusive prefix of ccnt
-  int* ckey;      // [Q] cell of each point (scratch of the build)
-  float4* xs;     // [Q] points in cell order: (fx, fy, fz, point index bits)
   int* n_active;  // device scalar
   int* csum;      // scan scratch
   int adj_lg;     // adjoint: log2 of the lanes per row, 6 = a block per row (set by the plan kernel)
@@ -94,8 +92,8 @@ struct Job {
   float* loss_fwd;         // [Q] phi(d^2) of each forward query
   float* loss_rev;         // [2 max_pts] phi(d^2) of each reverse query (set 0 then set 1)
   float* loss_iso;         // [E] |r_e|
-  int* nn_fwd;             // [Q] (-1 before the first search of a frame)
-  int* nn_rev;             // [2 max_pts] (-1 before the first search of a frame)
+  int* nn_fwd;             // [Q] (before the first search of a frame: its seed)
+  int* nn_rev;             // [2 max_pts] (before the first search of a frame: its seed)
   float4* edge_d;          // [E] sgn(r) (y_i - y_j) / (|y_i - y_j| E)
   const int2* edges;       // [E]
   float* e_prev;           // [E] rest lengths from X_{t-1}
@@ -104,27 +102,26 @@ struct Job {
   float4* src4;            // [max_pts] current source cloud P_{t-1}
   float4* tgt4;            // [max_pts] target P_t
   float4* verts4;          // [V] current deformed template X_{t-1}
-  CellGrid tgt;            // target grid, one set, built per frame
-  CellGrid mov;            // moving grid, two sets (template, source), rebuilt every step
-  int4* hard;              // [Q + 2 max_pts] queries left by the thread pass: (item, ring, d2 bits, idx)
+  Tree tgt;                // target points, built per frame
+  Tree mov;                // two sets (template, source): order of the frame's x, boxes of the step's y
+  float4* xs;              // [slots of mov] undeformed point and its index (bits) in slot order
   float* loss_part;        // [loss chunks][5] partial sums
   unsigned* gmax;          // max |dLoss/dy| component of the step (float bits; sets the adjoint's fixed-point scale)
-  int* hard_count;         // device scalar
   int* step;               // Adam step count k
   float* bias;             // [2] 1 / (1 - beta1^k), 1 / sqrt(1 - beta2^k) of the current step
   double* loss;            // [4] total, cd_mesh, cd_pts, iso of the last step
   int* status;             // sticky error flags (1: non-finite loss)
   unsigned long long* counters;  // [4] of the last step: NN candidates evaluated (counted only
                                  // when count_nn), NN queries decided by an exact tie,
-                                 // queries left to the warp pass, reserved
+                                 // 0, reserved
   const float* ext_in;     // pdg_precondition on a line-path level: the caller's gradient [n^3][3] ...
   float* ext_out;          // ... and where its preconditioned form goes (null in a step)
-  int count_nn;            // 1: k_nn / k_nn_hard add their candidate counts to counters[0]
+  int count_nn;            // 1: k_nn adds its candidate count to counters[0]
 };
 
-enum Counter { CNT_NN_CANDIDATES = 0, CNT_NN_TIES = 1, CNT_NN_HARD = 2 };
+enum Counter { CNT_NN_CANDIDATES = 0, CNT_NN_TIES = 1 };
 
-enum Stage { ST_Q = 0, ST_NNQ, ST_E, ST_MOVCH, ST_ADJ, ST_TILE, ST_JOB, ST_LOSSCH, ST_PLANE, ST_COL, ST_ADAM, ST_XTILE, NSTAGE };
+enum Stage { ST_Q = 0, ST_NODE, ST_SUPER, ST_NNF, ST_NNR, ST_E, ST_ADJ, ST_TILE, ST_JOB, ST_ADJROW, ST_LOSSCH, ST_PLANE, ST_COL, ST_ADAM, ST_XTILE, NSTAGE };
 
 struct Plan {
   int n_jobs;
@@ -182,16 +179,25 @@ __device__ __forceinline__ int find_job(const int* pre, int n_jobs, int item) {
   return lo;
 }
 
-__host__ __device__ __forceinline__ uint32_t part1by1(uint32_t v) {
-  v &= 0xFFu;
-  v = (v | (v << 4)) & 0x0F0Fu;
-  v = (v | (v << 2)) & 0x3333u;
-  v = (v | (v << 1)) & 0x5555u;
-  return v;
+// Sets of a tree as slot ranges.
+struct SetRange {
+  int slot0, n;    // first slot, points
+  int node0, nodes;
+  int super0, supers;
+};
+__host__ __device__ __forceinline__ SetRange set_range(int node0, int super0, int n) {
+  SetRange r;
+  r.slot0 = node0 * NODE;
+  r.n = n;
+  r.node0 = node0;
+  r.nodes = (n + NODE - 1) / NODE;
+  r.super0 = super0;
+  r.supers = (r.nodes + 31) / 32;
+  return r;
 }
-
-__host__ __device__ __forceinline__ int row_key(int cy, int cz, int bits) {
-  return (int)((part1by1((uint32_t)cy) | (part1by1((uint32_t)cz) << 1)) << bits);
+__device__ __forceinline__ SetRange mov_set(const Job& J, int set) {
+  const SetRange a = set_range(0, 0, J.V);
+  return set ? set_range(a.nodes, a.supers, J.N) : a;
 }
 
 __device__ __forceinline__ int cell_coord(float p, float lo, float inv_h, int G) {
@@ -201,12 +207,81 @@ __device__ __forceinline__ int cell_coord(float p, float lo, float inv_h, int G)
   return min(max(c, 0), G - 1);
 }
 
-__device__ __forceinline__ int cell_key(const CellGrid& g, float x, float y, float z, int set) {
-  int G = 1 << g.bits;
-  int cx = cell_coord(x, g.lo[0], g.inv_h[0], G);
-  int cy = cell_coord(y, g.lo[1], g.inv_h[1], G);
-  int cz = cell_coord(z, g.lo[2], g.inv_h[2], G);
-  return set * (G * G * G) + row_key(cy, cz, g.bits) + cx;
+// Index of a cell along the Hilbert curve of 8^bits cells (the transposed-axes algorithm of
+// Skilling, "Programming the Hilbert curve", 2004): unlike along the Morton curve, consecutive cells
+// are neighbours, so 32 consecutive points rarely straddle distant parts of the surface.
+__device__ __forceinline__ int hilbert3(int x, int y, int z, int bits) {
+  int X[3] = {x, y, z};
+  for (int q = 1 << (bits - 1); q > 1; q >>= 1) {
+    const int p = q - 1;
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+      if (X[i] & q) {
+        X[0] ^= p;
+      } else {
+        const int t = (X[0] ^ X[i]) & p;
+        X[0] ^= t;
+        X[i] ^= t;
+      }
+    }
+  }
+  X[1] ^= X[0];
+  X[2] ^= X[1];
+  int t = 0;
+  for (int q = 1 << (bits - 1); q > 1; q >>= 1)
+    if (X[2] & q) t ^= q - 1;
+  int key = 0;
+  for (int b = bits - 1; b >= 0; --b)
+#pragma unroll
+    for (int i = 0; i < 3; ++i) key = (key << 1) | (((X[i] ^ t) >> b) & 1);
+  return key;
+}
+
+__device__ __forceinline__ int cell_key(const Tree& g, float x, float y, float z, int set) {
+  const int G = 1 << g.bits;
+  const int cx = cell_coord(x, g.lo[0], g.inv_h[0], G);
+  const int cy = cell_coord(y, g.lo[1], g.inv_h[1], G);
+  const int cz = cell_coord(z, g.lo[2], g.inv_h[2], G);
+  return (set << (3 * g.bits)) + hilbert3(cx, cy, cz, g.bits);
+}
+
+// Stores the points of one node (thread t of 256: slot NODE nd + t; valid = false: padding) and
+// the boxes of its leaves and of the node.  All 256 threads of the block; synchronises.
+__device__ __forceinline__ void store_node(const Tree& T, int nd, float x, float y, float z, bool valid) {
+  __shared__ float wbox[8][6];
+  const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
+  const float inf = __int_as_float(0x7f800000);
+  const int leaf = nd * (NODE / LEAF) + t / LEAF;
+  float* p = T.pts + (size_t)leaf * (3 * LEAF) + (t & (LEAF - 1));
+  p[0] = valid ? x : inf;
+  p[LEAF] = valid ? y : inf;
+  p[2 * LEAF] = valid ? z : inf;
+  float b[6] = {valid ? x : inf, valid ? y : inf, valid ? z : inf, valid ? x : -inf, valid ? y : -inf, valid ? z : -inf};
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    if (o == LEAF && (lane & (LEAF - 1)) == 0) {
+      T.lbox[2 * leaf] = make_float4(b[0], b[1], b[2], b[3]);
+      T.lbox[2 * leaf + 1] = make_float4(b[4], b[5], 0.f, 0.f);
+    }
+#pragma unroll
+    for (int k = 0; k < 6; ++k) {
+      const float v = __shfl_xor_sync(0xffffffffu, b[k], o);
+      b[k] = k < 3 ? fminf(b[k], v) : fmaxf(b[k], v);
+    }
+  }
+  if (lane == 0)
+#pragma unroll
+    for (int k = 0; k < 6; ++k) wbox[warp][k] = b[k];
+  __syncthreads();
+  if (t == 0) {
+#pragma unroll
+    for (int w = 1; w < 8; ++w)
+#pragma unroll
+      for (int k = 0; k < 6; ++k) b[k] = k < 3 ? fminf(b[k], wbox[w][k]) : fmaxf(b[k], wbox[w][k]);
+    T.nbox[2 * nd] = make_float4(b[0], b[1], b[2], b[3]);
+    T.nbox[2 * nd + 1] = make_float4(b[4], b[5], 0.f, 0.f);
+  }
+  __syncthreads();
 }
 
 // squared distance, difference form; the same expression everywhere so that candidate

@@ -28,9 +28,9 @@ struct Arena {
   }
 };
 
-// Cells per axis (log2) of a nearest-neighbour grid over `count` points on a surface, with
-// about `per_cell` points in an occupied cell.
-int grid_bits(long count, double per_cell = 8.0) {
+// Cells per axis (log2) of a point tree's sort over `count` points on a surface, with about
+// `per_cell` points in an occupied cell: a leaf of 8 points then spans one or two cells.
+int grid_bits(long count, double per_cell = 6.0) {
   const double g = std::sqrt(std::max(count, 1L) / per_cell);
   int b = (int)std::lround(std::log2(std::max(g, 1.0)));
   return std::min(std::max(b, 2), 7);
@@ -38,6 +38,62 @@ int grid_bits(long count, double per_cell = 8.0) {
 
 // n if the line path preconditions a level of that size, else 0
 int line_size(int n) { return tile_level(n) ? n : 0; }
+
+// What the launches of a step are sized by: the largest levels, and the blocks each kernel has work
+// for (at a context's capacity; for a batch the sum over its members), at most the cap beyond which
+// a kernel's blocks loop over its items.  A fixed number of blocks would do, but an empty block
+// still costs its launch: 4864 of them about 4 us.
+struct Shape {
+  int sms = 1;
+  int nmax = 1;   // largest level resolution
+  int nline = 0;  // largest resolution among the levels the line path preconditions (0: none)
+  int nodes = 0, supers = 0;  // interpolation, upper boxes
+  int nnf = 0, nnr = 0;       // searches: warps of 32 queries, of the moving points and of the targets
+
+  // Lanes per query of the searches: 8 while that leaves no more than 32 warps per SM (a warp's own
+  // latency counts), else 2 (see k_nn.cu)
+  int nn_sub() const { return nnf + 2 * nnr < 4 * sms ? 8 : 2; }
+  int nn_grid(int warps) const { return std::max(1, std::min((warps * nn_sub() + 3) / 4, 32 * sms)); }
+
+  static void cap(int& v, long add, long most) { v = (int)std::min(v + add, most); }
+  // V, N points in the two moving sets, M targets
+  void add_points(long V, long N, long M) {
+    const long vn = (V + NODE - 1) / NODE, pn = (N + NODE - 1) / NODE;
+    cap(nodes, vn + pn, 8L * sms);
+    cap(supers, ((vn + 31) / 32 + (pn + 31) / 32 + 1) / 2, sms);
+    cap(nnf, (V + 31) / 32 + (N + 31) / 32, 128L * sms);
+    cap(nnr, (M + 31) / 32, 128L * sms);
+  }
+  void add_level(int n) {
+    nmax = std::max(nmax, n);
+    nline = std::max(nline, line_size(n));
+  }
+  void add(const Shape& o) {  // a batch's member
+    sms = o.sms;
+    nmax = std::max(nmax, o.nmax);
+    nline = std::max(nline, o.nline);
+    cap(nodes, o.nodes, 8L * sms);
+    cap(supers, o.supers, sms);
+    cap(nnf, o.nnf, 128L * sms);
+    cap(nnr, o.nnr, 128L * sms);
+  }
+  // componentwise maximum; true if it grew
+  bool grow(const Shape& o) {
+    bool g = false;
+    auto m = [&](int& a, int b) {
+      g = g || b > a;
+      a = std::max(a, b);
+    };
+    m(sms, o.sms);
+    m(nmax, o.nmax);
+    m(nline, o.nline);
+    m(nodes, o.nodes);
+    m(supers, o.supers);
+    m(nnf, o.nnf);
+    m(nnr, o.nnr);
+    return g;
+  }
+};
 
 // 1, or 2..256 with no prime factor but 2 and 3 (the line transforms are radix-2/3 FFTs)
 bool valid_res(int n) {
@@ -76,6 +132,20 @@ bool is_device_ptr(const void* p) {
   return a.type == cudaMemoryTypeDevice || a.type == cudaMemoryTypeManaged;
 }
 
+// the streams of a step's capture
+struct Streams {
+  cudaStream_t s[3] = {};
+  bool create() {
+    for (auto& x : s)
+      if (cudaStreamCreateWithFlags(&x, cudaStreamNonBlocking) != cudaSuccess) return false;
+    return true;
+  }
+  void destroy() {
+    for (auto& x : s)
+      if (x) cudaStreamDestroy(x);
+  }
+};
+
 }  // namespace
 
 // --------------------------------------------------------------------------------- context
@@ -100,9 +170,8 @@ struct pdg_ctx {
   bool mesh_valid = false; // a template-mesh fit has run (PDG_BUF_MESH_* readable)
   float* stage = nullptr;  // [stage_pts][3] staging of host inputs
   int stage_pts = 0;
-  int nmax = 1;
-  int nline = 0;  // largest resolution among the levels the line path preconditions
-  cudaStream_t cap = nullptr, cap2 = nullptr;
+  Shape shape;  // of its step at capacity
+  Streams cap;  // of the capture
   cudaGraphExec_t gexec = nullptr;
   int graph_kernels = 0;   // kernel nodes of gexec
   bool plan_stale = true;  // dplan's item prefixes predate the current frame
@@ -127,10 +196,9 @@ struct pdg_batch {
   Plan* dplan = nullptr;
   Plan* hplan = nullptr;  // pinned host copy
   std::vector<unsigned long long> gens;  // members' frame_gen when dplan's prefixes were computed
-  cudaStream_t cap = nullptr, cap2 = nullptr;
+  Streams cap;  // of the capture
   cudaGraphExec_t gexec = nullptr;
-  int graph_nmax = 0;
-  int graph_nline = 0;
+  Shape graph_shape;  // what gexec was captured for
   bool dirty = true;  // membership changed since the last upload of the job table
   std::string err;
 };
@@ -149,16 +217,18 @@ struct Layout {
   size_t total = 0;
   size_t job, plan, flag, stage, op_job, op_plan;
   struct Lv {
-    size_t theta, theta_t, m, v, g, tmp, zmask, piv, piv_slow, mu, tw, twm, tw4, cnt, rowptr, flag, act_v, act_ptr, ent, ccnt,
-        coff, ckey, xs, n_active, csum;
+    size_t theta, theta_t, m, v, g, tmp, zmask, piv, piv_slow, mu, tw, twm, tw4, cnt, rowptr, flag, act_v, act_ptr, ent, n_active,
+        csum;
     int cap;
   } lv[MAXL];
   size_t x, y, gfwd, gy, zq, uq, gz, acc, loss_fwd, loss_rev, loss_iso, nn_fwd, nn_rev, edge_d, edges, e_prev, v2e_ptr, v2e;
   size_t src4, tgt4, verts4;
-  size_t t_hist, t_off, t_keys, t_pts, t_csum, m_hist, m_off, m_keys, m_pts, m_csum;
-  size_t hard, hard_count, step, bias, loss, status, loss_part, gmax, counters;
+  struct Tr {
+    size_t hist, off, keys, csum, perm, pts, lbox, nbox, sbox;
+    int bits;
+  } tgt, mov;
+  size_t xs, step, bias, loss, status, loss_part, gmax, counters;
   size_t mesh;  // template-mesh fit: 7 float4 [V] arrays (gradient copy, solves, Adam moments)
-  int tbits, mbits;
 };
 
 Layout make_layout(const pdg_config& c, int V, int E, int max_pts) {
@@ -196,12 +266,6 @@ Layout make_layout(const pdg_config& c, int V, int E, int max_pts) {
     v.act_v = a.take<int>(v.cap);
     v.act_ptr = a.take<int>(v.cap + 1);
     v.ent = a.take<int2>(8 * (size_t)Q);
-    const bool fin = l == c.n_levels - 1;  // the cell order is kept for the finest level only
-    const size_t cells = fin ? (n > 1 ? (n - 1) * (n - 1) * (n - 1) : 1) : 1;
-    v.ccnt = a.take<int>(cells);
-    v.coff = a.take<int>(cells + 1);
-    v.ckey = a.take<int>(fin ? Q : 1);
-    v.xs = a.take<float4>(fin ? Q : 1);
     v.n_active = a.take<int>(1);
     v.csum = a.take<int>((n3 + 1) / SCAN_CHUNK + 2);
   }
@@ -226,26 +290,24 @@ Layout make_layout(const pdg_config& c, int V, int E, int max_pts) {
   L.src4 = a.take<float4>(max_pts);
   L.tgt4 = a.take<float4>(max_pts);
   L.verts4 = a.take<float4>(V);
-  // about 32 points per occupied cell in both NN grids: during a fit the nearest neighbour is
-  // often one or two spacings of a finer grid away, and the 3x3x3 box of these cells
-  // certifies almost every query in the one-thread-per-query pass (the moving grid is also
-  // rebuilt every step, its offsets a scan over all its cells)
-  L.tbits = grid_bits(max_pts, 32.0);
-  L.mbits = grid_bits(std::max(V, max_pts), 32.0);
-  const size_t tG3 = size_t(1) << (3 * L.tbits), mG3 = size_t(1) << (3 * L.mbits);
-  L.t_hist = a.take<int>(tG3);
-  L.t_off = a.take<int>(tG3 + 1);
-  L.t_keys = a.take<int>(max_pts);
-  L.t_pts = a.take<float4>(max_pts);
-  L.t_csum = a.take<int>(tG3 / SCAN_CHUNK + 2);
-  L.m_hist = a.take<int>(2 * mG3);
-  L.m_off = a.take<int>(2 * mG3 + 1);
-  L.m_keys = a.take<int>(Q);
-  L.m_pts = a.take<float4>(Q);
-  L.m_csum = a.take<int>(2 * mG3 / SCAN_CHUNK + 2);
-  L.hard = a.take<int4>(Q + 2 * (size_t)max_pts);
+  auto tree = [&](Layout::Tr& t, int sets, long count, int points, int nodes) {
+    t.bits = grid_bits(count);
+    const size_t cells = (size_t)sets << (3 * t.bits);
+    t.hist = a.take<int>(cells);
+    t.off = a.take<int>(cells + 1);
+    t.keys = a.take<int>(points);
+    t.csum = a.take<int>(cells / SCAN_CHUNK + 2);
+    t.perm = a.take<int>((size_t)nodes * NODE);
+    t.pts = a.take<float>((size_t)nodes * NODE * 3);
+    t.lbox = a.take<float4>((size_t)nodes * (NODE / LEAF) * 2);
+    t.nbox = a.take<float4>((size_t)nodes * 2);
+    t.sbox = a.take<float4>(((size_t)nodes / 32 + 2) * 2);
+  };
+  const int vn = (V + NODE - 1) / NODE, pn = (max_pts + NODE - 1) / NODE;
+  tree(L.tgt, 1, max_pts, max_pts, pn);
+  tree(L.mov, 2, std::max(V, max_pts), Q, vn + pn);
+  L.xs = a.take<float4>((size_t)(vn + pn) * NODE);
   L.loss_part = a.take<float>(5 * ((Q + 2 * (size_t)max_pts + std::max(E, 1)) / LOSS_CHUNK + 2));
-  L.hard_count = a.take<int>(1);
   L.step = a.take<int>(1);
   L.bias = a.take<float>(2);
   L.loss = a.take<double>(4);
@@ -310,59 +372,60 @@ pdg_status upload_job(pdg_ctx* c, cudaStream_t s) {
 
 // The step as an explicit list of stages; the graph capture and the profiling path launch
 // exactly the same sequence.
-const char* const STAGE_NAMES[] = {"interp",     "mov_scan",   "mov_scatter", "nn",          "nn_hard",
-                                   "iso_edges",  "assemble",   "adjoint",     "sob_xy_fwd",  "sob_z",
-                                   "sob_xy_inv", "adam",       "sobolev_256", "loss"};
+const char* const STAGE_NAMES[] = {"interp",       "boxes",   "nn",         "nn_rev_mesh", "nn_rev_pts", "iso_edges",
+                                   "assemble",     "adjoint_rows", "adjoint", "sob_xy_fwd",  "sob_z",      "sob_xy_inv",
+                                   "adam",         "sobolev_256", "loss"};
 constexpr int N_STAGES = sizeof(STAGE_NAMES) / sizeof(STAGE_NAMES[0]);
 enum StageIndex {
-  S_INTERP = 0, S_MOV_SCAN, S_MOV_SCATTER, S_NN, S_NN_HARD, S_ISO, S_ASSEMBLE, S_ADJOINT,
+  S_INTERP = 0, S_BOXES, S_NN, S_NN_REV0, S_NN_REV1, S_ISO, S_ASSEMBLE, S_ADJOINT_ROWS, S_ADJOINT,
   S_SOB_XY_FWD, S_SOB_Z, S_SOB_XY_INV, S_ADAM, S_SOB_256, S_LOSS
 };
 
 // Stage i of a step; bump: the job_bump mode of the interpolation stage (1: optimisation
 // step, 2: evaluation); count: the nearest-neighbour instances that count candidates and
 // exact ties.  The plan's item prefixes must be current (refresh_plan).
-// nmax: the largest level resolution; nline: the largest one of the levels the line path
-// preconditions (0: none)
-void launch_stage(int i, const Plan* plan, int nmax, int nline, int sms, cudaStream_t s, int bump = 1,
-                  bool count = false) {
+void launch_stage(int i, const Plan* plan, const Shape& sh, cudaStream_t s, int bump = 1, bool count = false) {
+  const int sms = sh.sms;
   const int grid = sms * 8;
   switch (i) {
-    case S_INTERP: launch_interp(plan, grid, s, bump); break;
-    case S_MOV_SCAN: launch_mov_scan(plan, sms * 2, s); break;
-    case S_MOV_SCATTER: launch_mov_scatter(plan, grid, s); break;
-    case S_NN: launch_nn(plan, grid * 2, s, count); break;
-    case S_NN_HARD: launch_nn_hard(plan, sms * 4, s, count); break;
+    case S_INTERP: launch_interp(plan, sh.nodes, s, bump); break;
+    case S_BOXES: launch_boxes(plan, sh.supers, s); break;
+    case S_NN: launch_nn(plan, sh.nn_grid(sh.nnf), s, -1, sh.nn_sub(), count); break;
+    case S_NN_REV0: launch_nn(plan, sh.nn_grid(sh.nnr), s, 0, sh.nn_sub(), count); break;
+    case S_NN_REV1: launch_nn(plan, sh.nn_grid(sh.nnr), s, 1, sh.nn_sub(), count); break;
     case S_ISO: launch_iso_edges(plan, grid, s); break;
     case S_ASSEMBLE: launch_assemble(plan, grid, s); break;
+    case S_ADJOINT_ROWS: launch_adjoint_rows(plan, grid, s); break;
     case S_ADJOINT: launch_adjoint(plan, grid * 2, s); break;
     case S_SOB_XY_FWD:
     case S_SOB_Z:
     case S_SOB_XY_INV:
     case S_ADAM: {
-      const int ps = plane_smem_max(nmax);
+      const int ps = plane_smem_max(sh.nmax);
       const int per_sm = std::max(1, std::min(8, (227 * 1024) / ps));
-      launch_sobolev_plane(plan, sms * per_sm, nmax, s, i - S_SOB_XY_FWD);
+      launch_sobolev_plane(plan, sms * per_sm, sh.nmax, s, i - S_SOB_XY_FWD);
       break;
     }
     case S_SOB_256:
-      if (nline == 0) break;
-      launch_sobolev_x(plan, sms, nline, true, s);
-      for (int p = YZ_FWD; p <= YZ_INV; ++p) launch_sobolev_yz(plan, sms, nline, p, s);
-      launch_sobolev_x(plan, sms, nline, false, s);
+      if (sh.nline == 0) break;
+      launch_sobolev_x(plan, sms, sh.nline, true, s);
+      for (int p = YZ_FWD; p <= YZ_INV; ++p) launch_sobolev_yz(plan, sms, sh.nline, p, s);
+      launch_sobolev_x(plan, sms, sh.nline, false, s);
       break;
     case S_LOSS: launch_loss(plan, sms * 2, s); break;
   }
 }
 constexpr int ST_SOB_FIRST = S_SOB_XY_FWD, ST_SOB_LAST = S_SOB_256;  // preconditioner and Adam stages
 
-// Captures one step.  Two branches: the isometry kernel runs beside the moving grid's sort
-// and the nearest-neighbour passes (it needs only the deformed points), the loss reduction
-// beside the adjoint and the preconditioner (nothing downstream reads it).
-pdg_status capture_step(pdg_ctx* c, const Plan* plan, int nmax, int nline, cudaStream_t cap, cudaStream_t cap2,
-                        cudaGraphExec_t* out, std::string* err, int sms, int* n_kernels = nullptr) {
+// Captures one step.  Branches: the searches of the moving points (in the target tree, which needs
+// no boxes of this step) and the isometry beside the moving trees' upper boxes and the targets'
+// searches, one per moving set; the two adjoint kernels beside each other; the loss reduction beside
+// the adjoint and the preconditioner (nothing downstream reads it).
+pdg_status capture_step(pdg_ctx* c, const Plan* plan, const Shape& sh, const Streams& st, cudaGraphExec_t* out,
+                        std::string* err, int* n_kernels = nullptr) {
+  const cudaStream_t cap = st.s[0], cap2 = st.s[1], cap3 = st.s[2];
   cudaGraph_t g = nullptr;
-  cudaEvent_t ev[4] = {};
+  cudaEvent_t ev[7] = {};
   for (auto& e : ev)
     if (cudaEventCreateWithFlags(&e, cudaEventDisableTiming) != cudaSuccess) {
       *err = "cudaEventCreate failed";
@@ -375,23 +438,29 @@ pdg_status capture_step(pdg_ctx* c, const Plan* plan, int nmax, int nline, cudaS
     return PDG_ERR_CUDA;
   }
   const bool count = c && c->h.count_nn;  // a batch graph never counts
-  launch_stage(S_INTERP, plan, nmax, nline, sms, cap);  // starts the step of every job
-  cudaEventRecord(ev[0], cap);
-  cudaStreamWaitEvent(cap2, ev[0], 0);
-  launch_stage(S_ISO, plan, nmax, nline, sms, cap2);
-  cudaEventRecord(ev[1], cap2);
-  launch_stage(S_MOV_SCAN, plan, nmax, nline, sms, cap);
-  launch_stage(S_MOV_SCATTER, plan, nmax, nline, sms, cap);
-  launch_stage(S_NN, plan, nmax, nline, sms, cap, 1, count);
-  launch_stage(S_NN_HARD, plan, nmax, nline, sms, cap, 1, count);
-  cudaStreamWaitEvent(cap, ev[1], 0);
-  launch_stage(S_ASSEMBLE, plan, nmax, nline, sms, cap);
-  cudaEventRecord(ev[2], cap);
-  cudaStreamWaitEvent(cap2, ev[2], 0);
-  launch_stage(S_LOSS, plan, nmax, nline, sms, cap2);
-  cudaEventRecord(ev[3], cap2);
-  for (int i = S_ADJOINT; i <= S_SOB_256; ++i) launch_stage(i, plan, nmax, nline, sms, cap);  // adjoint, preconditioner, Adam
-  cudaStreamWaitEvent(cap, ev[3], 0);
+  int n_ev = 0;
+  auto after = [&](cudaStream_t to, cudaStream_t from) {  // `to` goes on after what `from` holds now
+    cudaEventRecord(ev[n_ev], from);
+    cudaStreamWaitEvent(to, ev[n_ev++], 0);
+  };
+  launch_stage(S_INTERP, plan, sh, cap);  // starts the step of every job
+  after(cap2, cap);
+  launch_stage(S_BOXES, plan, sh, cap2);
+  after(cap3, cap2);
+  launch_stage(S_NN_REV0, plan, sh, cap2, 1, count);
+  launch_stage(S_NN_REV1, plan, sh, cap3, 1, count);
+  launch_stage(S_NN, plan, sh, cap, 1, count);
+  launch_stage(S_ISO, plan, sh, cap);
+  after(cap, cap2);
+  after(cap, cap3);
+  launch_stage(S_ASSEMBLE, plan, sh, cap);
+  after(cap2, cap);
+  launch_stage(S_ADJOINT_ROWS, plan, sh, cap2);
+  launch_stage(S_ADJOINT, plan, sh, cap);
+  after(cap, cap2);
+  launch_stage(S_LOSS, plan, sh, cap2);
+  for (int i = S_SOB_XY_FWD; i <= S_SOB_256; ++i) launch_stage(i, plan, sh, cap);  // preconditioner, Adam
+  after(cap, cap2);
   e = cudaStreamEndCapture(cap, &g);
   for (auto& x : ev) cudaEventDestroy(x);
   if (e != cudaSuccess) {
@@ -478,8 +547,7 @@ const char* pdg_last_error(const pdg_ctx* c) { return c ? c->err.c_str() : "cont
 void pdg_destroy(pdg_ctx* c) {
   if (!c) return;
   if (c->gexec) cudaGraphExecDestroy(c->gexec);
-  if (c->cap) cudaStreamDestroy(c->cap);
-  if (c->cap2) cudaStreamDestroy(c->cap2);
+  c->cap.destroy();
   if (c->arena) cudaFree(c->arena);
   delete c;
 }
@@ -506,6 +574,8 @@ pdg_status pdg_create(const pdg_config* cfg, const float* template_xyz, int n_ve
   };
   if (cudaGetDevice(&c->dev) != cudaSuccess) return bail(PDG_ERR_CUDA);
   cudaDeviceGetAttribute(&c->sms, cudaDevAttrMultiProcessorCount, c->dev);
+  c->shape.sms = c->sms;
+  c->shape.add_points(n_verts, max_pts, max_pts);
   sobolev_x_configure();
   sobolev_yz_configure();
   sobolev_plane_configure();
@@ -615,14 +685,9 @@ pdg_status pdg_create(const pdg_config* cfg, const float* template_xyz, int n_ve
     lv.act_v = (int*)P(o.act_v);
     lv.act_ptr = (int*)P(o.act_ptr);
     lv.ent = (int2*)P(o.ent);
-    lv.ccnt = (int*)P(o.ccnt);
-    lv.coff = (int*)P(o.coff);
-    lv.ckey = (int*)P(o.ckey);
-    lv.xs = (float4*)P(o.xs);
     lv.n_active = (int*)P(o.n_active);
     lv.csum = (int*)P(o.csum);
-    c->nmax = std::max(c->nmax, n);
-    c->nline = std::max(c->nline, line_size(n));
+    c->shape.add_level(n);
     mu.resize(n);
     tw.resize(n);
     tw4.resize(n);
@@ -668,26 +733,26 @@ pdg_status pdg_create(const pdg_config* cfg, const float* template_xyz, int n_ve
   J.src4 = (float4*)P(L.src4);
   J.tgt4 = (float4*)P(L.tgt4);
   J.verts4 = (float4*)P(L.verts4);
-  auto grid_init = [&](CellGrid& g, int bits, int nsets, size_t hist, size_t off, size_t keys, size_t pts, size_t csum) {
-    g.bits = bits;
-    g.nsets = nsets;
-    const int G = 1 << bits;
+  auto tree_init = [&](Tree& t, const Layout::Tr& o) {
+    t.bits = o.bits;
     for (int a = 0; a < 3; ++a) {
-      g.lo[a] = cfg->lo[a];
-      g.inv_h[a] = (float)(G / ((double)cfg->hi[a] - cfg->lo[a]));
-      g.h[a] = (float)(((double)cfg->hi[a] - cfg->lo[a]) / G);
+      t.lo[a] = cfg->lo[a];
+      t.inv_h[a] = (float)((1 << o.bits) / ((double)cfg->hi[a] - cfg->lo[a]));
     }
-    g.hist = (int*)P(hist);
-    g.off = (int*)P(off);
-    g.keys = (int*)P(keys);
-    g.pts = (float4*)P(pts);
-    g.csum = (int*)P(csum);
+    t.hist = (int*)P(o.hist);
+    t.off = (int*)P(o.off);
+    t.keys = (int*)P(o.keys);
+    t.csum = (int*)P(o.csum);
+    t.perm = (int*)P(o.perm);
+    t.pts = (float*)P(o.pts);
+    t.lbox = (float4*)P(o.lbox);
+    t.nbox = (float4*)P(o.nbox);
+    t.sbox = (float4*)P(o.sbox);
   };
-  grid_init(J.tgt, L.tbits, 1, L.t_hist, L.t_off, L.t_keys, L.t_pts, L.t_csum);
-  grid_init(J.mov, L.mbits, 2, L.m_hist, L.m_off, L.m_keys, L.m_pts, L.m_csum);
-  J.hard = (int4*)P(L.hard);
+  tree_init(J.tgt, L.tgt);
+  tree_init(J.mov, L.mov);
+  J.xs = (float4*)P(L.xs);
   J.loss_part = (float*)P(L.loss_part);
-  J.hard_count = (int*)P(L.hard_count);
   J.step = (int*)P(L.step);
   J.bias = (float*)P(L.bias);
   J.loss = (double*)P(L.loss);
@@ -720,8 +785,7 @@ pdg_status pdg_create(const pdg_config* cfg, const float* template_xyz, int n_ve
     if (cudaMemcpyAsync(c->dplan, &hp, sizeof(Plan), cudaMemcpyHostToDevice, s) != cudaSuccess)
       return bail(PDG_ERR_CUDA);
   }
-  if (cudaStreamCreateWithFlags(&c->cap, cudaStreamNonBlocking) != cudaSuccess ||
-      cudaStreamCreateWithFlags(&c->cap2, cudaStreamNonBlocking) != cudaSuccess)
+  if (!c->cap.create())
     return bail(PDG_ERR_CUDA);
   if (cudaStreamSynchronize(s) != cudaSuccess) return bail(PDG_ERR_CUDA);
   *out = c;
@@ -774,11 +838,10 @@ pdg_status pdg_begin_frame(pdg_ctx* c, const float* target_xyz, int n_tgt, void*
   }
   CU(c, cudaMemsetAsync(J.step, 0, sizeof(int), s));
   CU(c, cudaMemsetAsync(J.status, 0, sizeof(int), s));
-  // no previous neighbours in a new frame (-1: the NN search starts cold)
-  CU(c, cudaMemsetAsync(J.nn_fwd, 0xff, sizeof(int) * (size_t)J.Q, s));
-  CU(c, cudaMemsetAsync(J.nn_rev, 0xff, sizeof(int) * 2 * (size_t)c->max_pts, s));
   CU(c, cudaMemsetAsync(J.loss, 0, 4 * sizeof(double), s));
   launch_tgt_build(c->dJ, J, s);
+  launch_mov_build(c->dJ, J, s);
+  launch_nn_seed(c->dJ, J, s);
   launch_csr_build(c->dJ, J, s);
   CU(c, cudaGetLastError());
   c->in_frame = true;
@@ -797,7 +860,7 @@ pdg_status pdg_step(pdg_ctx* c, int n_steps, void* cuda_stream) {
   if (!c->gexec) {
     // the captured launches must not start before this stream's pending set-up
     CU(c, cudaStreamSynchronize(s));
-    TRY(capture_step(c, c->dplan, c->nmax, c->nline, c->cap, c->cap2, &c->gexec, &c->err, c->sms, &c->graph_kernels));
+    TRY(capture_step(c, c->dplan, c->shape, c->cap, &c->gexec, &c->err, &c->graph_kernels));
   }
   TRY(refresh_plan(c, s));
   for (int i = 0; i < n_steps; ++i) CU(c, cudaGraphLaunch(c->gexec, s));
@@ -826,7 +889,7 @@ pdg_status pdg_profile_step(pdg_ctx* c, int n_steps, double* stage_ms, void* cud
   for (int k = 0; k < n_steps && st == PDG_OK; ++k) {
     for (int i = 0; i < N_STAGES; ++i) {
       cudaEventRecord(ev[i], s);
-      launch_stage(i, c->dplan, c->nmax, c->nline, c->sms, s, 1, c->h.count_nn != 0);
+      launch_stage(i, c->dplan, c->shape, s, 1, c->h.count_nn != 0);
     }
     cudaEventRecord(ev[N_STAGES], s);
     st = c->cuda(cudaEventSynchronize(ev[N_STAGES]), "profile step");
@@ -1021,7 +1084,7 @@ pdg_status pdg_eval(pdg_ctx* c, double* loss, void* cuda_stream) {
   cudaStream_t s = (cudaStream_t)cuda_stream;
   TRY(refresh_plan(c, s));
   for (int i = 0; i < N_STAGES; ++i)  // no preconditioner, no Adam, no step count
-    if (i < ST_SOB_FIRST || i > ST_SOB_LAST) launch_stage(i, c->dplan, c->nmax, c->nline, c->sms, s, 2, c->h.count_nn != 0);
+    if (i < ST_SOB_FIRST || i > ST_SOB_LAST) launch_stage(i, c->dplan, c->shape, s, 2, c->h.count_nn != 0);
   CU(c, cudaGetLastError());
   if (loss) {
     CU(c, cudaMemcpyAsync(loss, c->h.loss, 4 * sizeof(double), cudaMemcpyDeviceToHost, s));
@@ -1060,7 +1123,10 @@ pdg_status pdg_precondition(pdg_ctx* c, int level, const float* g, float* out, v
   CU(c, cudaMemcpyAsync(c->op_job, &oj, sizeof(Job), cudaMemcpyHostToDevice, s));
   CU(c, cudaMemcpyAsync(c->op_plan, &op, sizeof(Plan), cudaMemcpyHostToDevice, s));
   launch_plan(c->op_plan, s);
-  for (int i = ST_SOB_FIRST; i <= ST_SOB_LAST; ++i) launch_stage(i, c->op_plan, lv.n, line_size(lv.n), c->sms, s);
+  Shape sh;
+  sh.sms = c->sms;
+  sh.add_level(lv.n);
+  for (int i = ST_SOB_FIRST; i <= ST_SOB_LAST; ++i) launch_stage(i, c->op_plan, sh, s);
   if (!line) launch_soa_to_aos(lv.tmp, tmp, lv.n3, s);
   CU(c, cudaGetLastError());
   const pdg_status st = copy_out(c, out, tmp, bytes, s);
@@ -1114,11 +1180,11 @@ pdg_status pdg_fit_mesh(pdg_ctx* c, const float* p0_xyz, int n_p0, int n_steps, 
   float4* av = am + V;
   CU(c, cudaMemcpyAsync(J.x, J.verts4, sizeof(float4) * V, cudaMemcpyDeviceToDevice, s));  // X_0 being fitted
   CU(c, cudaMemsetAsync(am, 0, 2 * sizeof(float4) * (size_t)V, s));
-  CU(c, cudaMemsetAsync(J.nn_fwd, 0xff, sizeof(int) * (size_t)V, s));
-  CU(c, cudaMemsetAsync(J.nn_rev, 0xff, sizeof(int) * (size_t)n_p0, s));
   CU(c, cudaMemsetAsync(J.loss, 0, 4 * sizeof(double), s));
   CU(c, cudaMemsetAsync(J.status, 0, sizeof(int), s));
   launch_tgt_build(c->op_job, mj, s);
+  launch_mov_build(c->op_job, mj, s);
+  launch_nn_seed(c->op_job, mj, s);
   // Chebyshev interval: the Laplacian's eigenvalues lie in [0, 2 max degree] (Gershgorin), so
   // those of I + lambda L in [1, emax]; iterations for a relative error below 1e-7 in exact
   // arithmetic, 2 sqrt(kappa) q^k <= 1e-7 with q = (sqrt(kappa) - 1) / (sqrt(kappa) + 1)
@@ -1127,11 +1193,14 @@ pdg_status pdg_fit_mesh(pdg_ctx* c, const float* p0_xyz, int n_p0, int n_steps, 
   const double q = (sk - 1.0) / (sk + 1.0);
   const int iters = q > 0.0 ? (int)std::ceil(std::log(1e-7 / (2.0 * sk)) / std::log(q)) : 1;
   const int2* edges = J.edges;
+  Shape sh;
+  sh.sms = c->sms;
+  sh.add_points(V, 0, n_p0);
   for (int k = 1; k <= n_steps; ++k) {
     launch_mesh_points(c->op_job, V, s);
-    for (int i = S_MOV_SCAN; i <= S_NN_HARD; ++i) launch_stage(i, c->op_plan, 1, 0, c->sms, s);
-    launch_stage(S_ASSEMBLE, c->op_plan, 1, 0, c->sms, s);
-    launch_stage(S_LOSS, c->op_plan, 1, 0, c->sms, s);
+    for (int i = S_BOXES; i <= S_NN_REV0; ++i) launch_stage(i, c->op_plan, sh, s);
+    launch_stage(S_ASSEMBLE, c->op_plan, sh, s);
+    launch_stage(S_LOSS, c->op_plan, sh, s);
     // (I + lambda L)^{-2} dL/dX by two solves, then Adam on the vertices
     launch_mesh_solve(J.v2e_ptr, J.v2e, edges, J.gy, h, r, d0, d1, V, lambda, (float)emax, iters, s);
     launch_mesh_solve(J.v2e_ptr, J.v2e, edges, h, pg, r, d0, d1, V, lambda, (float)emax, iters, s);
@@ -1171,8 +1240,7 @@ pdg_status pdg_batch_create(int max_jobs, pdg_batch** out) {
   pdg_batch* b = new pdg_batch();
   b->max_jobs = max_jobs;
   if (dev_malloc((void**)&b->dplan, sizeof(Plan)) != cudaSuccess || cudaMallocHost(&b->hplan, sizeof(Plan)) != cudaSuccess ||
-      cudaStreamCreateWithFlags(&b->cap, cudaStreamNonBlocking) != cudaSuccess ||
-      cudaStreamCreateWithFlags(&b->cap2, cudaStreamNonBlocking) != cudaSuccess) {
+      !b->cap.create()) {
     cudaGetLastError();
     pdg_batch_destroy(b);
     return PDG_ERR_OOM;
@@ -1185,8 +1253,7 @@ pdg_status pdg_batch_create(int max_jobs, pdg_batch** out) {
 void pdg_batch_destroy(pdg_batch* b) {
   if (!b) return;
   if (b->gexec) cudaGraphExecDestroy(b->gexec);
-  if (b->cap) cudaStreamDestroy(b->cap);
-  if (b->cap2) cudaStreamDestroy(b->cap2);
+  b->cap.destroy();
   if (b->dplan) cudaFree(b->dplan);
   if (b->hplan) cudaFreeHost(b->hplan);
   delete b;
@@ -1213,16 +1280,13 @@ pdg_status pdg_batch_step(pdg_batch* b, int n_steps, void* cuda_stream) {
   if (!b || n_steps < 0) return PDG_ERR_INVALID;
   if (b->n == 0 || n_steps == 0) return PDG_OK;
   cudaStream_t s = (cudaStream_t)cuda_stream;
-  int nmax = 1, sms = 1;
-  int nline = 0;
+  Shape sh;
   for (auto* c : b->members) {
     if (!c->in_frame) {
       b->err = "batch member outside a frame";
       return PDG_ERR_STATE;
     }
-    nmax = std::max(nmax, c->nmax);
-    nline = std::max(nline, c->nline);
-    sms = c->sms;
+    sh.add(c->shape);
   }
   if (b->dirty) {
     // publish the membership (stream-ordered; the pinned host copy is rewritten only after
@@ -1245,14 +1309,14 @@ pdg_status pdg_batch_step(pdg_batch* b, int n_steps, void* cuda_stream) {
     b->gens.resize(b->members.size());
     for (size_t i = 0; i < b->members.size(); ++i) b->gens[i] = b->members[i]->frame_gen;
   }
-  if (!b->gexec || nmax > b->graph_nmax || nline > b->graph_nline) {
+  Shape need = b->graph_shape;
+  if (need.grow(sh) || !b->gexec) {
     if (b->gexec) cudaGraphExecDestroy(b->gexec);
     b->gexec = nullptr;
     if (cudaStreamSynchronize(s) != cudaSuccess) return PDG_ERR_CUDA;
-    const pdg_status st = capture_step(nullptr, b->dplan, std::max(nmax, b->graph_nmax), std::max(nline, b->graph_nline), b->cap, b->cap2, &b->gexec, &b->err, sms);
+    const pdg_status st = capture_step(nullptr, b->dplan, need, b->cap, &b->gexec, &b->err);
     if (st != PDG_OK) return st;
-    b->graph_nmax = std::max(nmax, b->graph_nmax);
-    b->graph_nline = std::max(nline, b->graph_nline);
+    b->graph_shape = need;
   }
   for (int i = 0; i < n_steps; ++i)
     if (cudaGraphLaunch(b->gexec, s) != cudaSuccess) return PDG_ERR_CUDA;
