@@ -26,7 +26,12 @@ class GridLoss(torch.autograd.Function):
             else:
                 B.pdg_write_theta(handle, l, t.numpy())
             res.append(th.shape)
-        loss = B.pdg_eval(handle)
+        dev0 = thetas[0].device
+        if dev0.type == "cuda":  # the loss stays on the device: nothing waits for the evaluation
+            B.pdg_eval_async(handle)
+            loss = B.pdg_read(handle, B.BUF_LOSS, 0, torch.empty(4, dtype=torch.float64, device=dev0))[0]
+        else:
+            loss = torch.tensor(B.pdg_eval(handle)[0], dtype=torch.float64, device=dev0)
         grads = []
         for l, shp in enumerate(res):
             n3 = int(np.prod(shp[:-1]))
@@ -35,12 +40,17 @@ class GridLoss(torch.autograd.Function):
             B.pdg_read(handle, B.BUF_GRAD, l, g if g.is_cuda else g.numpy())
             grads.append(g.reshape(shp).to(thetas[l].dtype))
         fctx.save_for_backward(*grads)
-        return torch.tensor(loss[0], dtype=torch.float64, device=thetas[0].device)
+        return loss
 
     @staticmethod
     def backward(fctx, grad_out):
-        grads = fctx.saved_tensors
-        return (None, *[g * grad_out.to(g.dtype) for g in grads])
+        scale = {}  # grad_out in each dtype of the grids, converted once
+        out = []
+        for g in fctx.saved_tensors:
+            if g.dtype not in scale:
+                scale[g.dtype] = grad_out.to(g.dtype)
+            out.append(g * scale[g.dtype])
+        return (None, *out)
 
 
 def grid_loss(handle, thetas):

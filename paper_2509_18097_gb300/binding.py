@@ -131,7 +131,8 @@ def _stream(stream):
         return C.c_void_p(int(stream))
     import torch
 
-    if torch.cuda.is_available():
+    # is_available() asks the driver each time; an initialised CUDA is available
+    if torch.cuda.is_initialized() or torch.cuda.is_available():
         return C.c_void_p(torch.cuda.current_stream().cuda_stream)
     return C.c_void_p(0)
 
@@ -269,6 +270,11 @@ def pdg_eval(ctx, stream=None) -> np.ndarray:
     out = (C.c_double * 4)()
     _check(load().pdg_eval(ctx, out, _stream(stream)), ctx)
     return np.array(out[:], np.float64)
+
+
+def pdg_eval_async(ctx, stream=None):
+    """pdg_eval without the losses on the host: nothing is waited for (PDG_BUF_LOSS holds them)."""
+    _check(load().pdg_eval(ctx, None, _stream(stream)), ctx)
 
 
 def pdg_fit_mesh(ctx, p0, n_steps: int, lam: float = MESH_LAMBDA, lr: float = MESH_LR, stream=None) -> pdg_fit_stats:

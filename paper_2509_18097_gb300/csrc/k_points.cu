@@ -97,6 +97,17 @@ __global__ void k_plan(Plan* P) {
   }
 }
 
+// the job record (by value, in the launch's arguments) and the plan that holds it alone
+__global__ void k_op_job(const __grid_constant__ Job job, Job* dJ, Plan* dP) {
+  const unsigned* src = reinterpret_cast<const unsigned*>(&job);
+  unsigned* dst = reinterpret_cast<unsigned*>(dJ);
+  for (int i = threadIdx.x; i < (int)(sizeof(Job) / 4); i += blockDim.x) dst[i] = src[i];
+  if (threadIdx.x == 0) {
+    dP->n_jobs = 1;
+    dP->jobs[0] = dJ;
+  }
+}
+
 // ------------------------------------------------------------------------------ (a) eval
 
 // Trilinear interpolation of one level's values at a point (Eq. 1; vertex-aligned levels,
@@ -521,6 +532,11 @@ __global__ void k_deform(const Job* __restrict__ J, const float* __restrict__ in
 static inline int blocks_for(int n, int threads) { return max(1, min((n + threads - 1) / threads, 4096)); }
 
 void launch_plan(Plan* P, cudaStream_t s) { k_plan<<<1, 256, 0, s>>>(P); }
+void launch_op_plan(const Job& job, Job* dJ, Plan* dP, cudaStream_t s) {
+  static_assert(sizeof(Job) % 4 == 0, "copied word by word");
+  k_op_job<<<1, 256, 0, s>>>(job, dJ, dP);
+  launch_plan(dP, s);
+}
 void launch_interp(const Plan* P, int grid, cudaStream_t s, int bump) { k_interp<<<grid, 256, 0, s>>>(P, bump); }
 void launch_boxes(const Plan* P, int grid, cudaStream_t s) { k_boxes<<<grid, 64, 0, s>>>(P); }
 void launch_iso_edges(const Plan* P, int grid, cudaStream_t s) { k_iso_edges<<<grid, 256, 0, s>>>(P); }

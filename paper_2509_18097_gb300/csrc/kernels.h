@@ -8,6 +8,8 @@ namespace pdg {
 
 // per step (plan-driven; `grid` = blocks of the persistent launch)
 void launch_plan(Plan* P, cudaStream_t s);
+// a record and a plan for one job, from the launch's arguments (nothing is copied from host memory)
+void launch_op_plan(const Job& job, Job* dJ, Plan* dP, cudaStream_t s);
 void launch_interp(const Plan* P, int grid, cudaStream_t s, int bump);
 void launch_boxes(const Plan* P, int grid, cudaStream_t s);
 // set < 0: the moving points' searches in the target tree, else the targets' in the tree of a moving

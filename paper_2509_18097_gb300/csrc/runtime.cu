@@ -122,6 +122,18 @@ cudaError_t dev_malloc(void** p, size_t bytes) {
   return cudaMalloc(p, bytes);
 }
 
+// Device memory that the current device's kernels may use as floats: where a buffer is not (host
+// memory, another GPU's, not on a 4-byte boundary) the calls go through a copy instead.
+bool kernel_ptr(const void* p, int dev) {
+  cudaPointerAttributes a;
+  if (cudaPointerGetAttributes(&a, p) != cudaSuccess) {
+    cudaGetLastError();
+    return false;
+  }
+  if (a.type != cudaMemoryTypeManaged && !(a.type == cudaMemoryTypeDevice && a.device == dev)) return false;
+  return (reinterpret_cast<uintptr_t>(p) & 3) == 0;
+}
+
 bool is_device_ptr(const void* p) {
   if (!p) return false;
   cudaPointerAttributes a;
@@ -1033,8 +1045,11 @@ pdg_status pdg_read(pdg_ctx* c, int which, int level, void* out, size_t out_byte
   if (which == PDG_BUF_NN_FWD) return copy_out(c, out, J.nn_fwd, need, s);
   if (which == PDG_BUF_NN_REV) return copy_out(c, out, J.nn_rev, need, s);
   if (which == PDG_BUF_COUNTERS) return copy_out(c, out, J.counters, need, s);
-  float* tmp = nullptr;
-  CU(c, cudaMallocAsync((void**)&tmp, need, s));
+  // straight into a device buffer; a stream-ordered allocation would be given back to the system at the
+  // next synchronisation and cost about 200 us each time
+  const bool direct = kernel_ptr(out, c->dev);
+  float* tmp = static_cast<float*>(out);
+  if (!direct) CU(c, cudaMallocAsync((void**)&tmp, need, s));
   switch (which) {
     case PDG_BUF_THETA:
       launch_unpack_theta(J.lev[level].theta, J.lev[level].theta_t, tmp, J.lev[level].n3, J.C, s);
@@ -1049,6 +1064,7 @@ pdg_status pdg_read(pdg_ctx* c, int which, int level, void* out, size_t out_byte
     case PDG_BUF_MESH_GRAD: launch_unpack4(J.gy, tmp, c->V, s); break;
     case PDG_BUF_MESH_PGRAD: launch_unpack4(c->mesh + 4 * (size_t)c->V, tmp, c->V, s); break;
   }
+  if (direct) return c->cuda(cudaGetLastError(), "read");
   const pdg_status st = copy_out(c, out, tmp, need, s);
   cudaFreeAsync(tmp, s);
   return st;
@@ -1100,11 +1116,15 @@ pdg_status pdg_precondition(pdg_ctx* c, int level, const float* g, float* out, v
   cudaStream_t s = (cudaStream_t)cuda_stream;
   const Level& lv = c->h.lev[level];
   const size_t bytes = sizeof(float) * 3 * (size_t)lv.n3;
+  // device buffers are read and written in place (every read of g precedes the first write of out)
+  const bool direct_g = kernel_ptr(g, c->dev), direct_out = kernel_ptr(out, c->dev);
   float* tmp = nullptr;
-  CU(c, cudaMallocAsync((void**)&tmp, bytes, s));
-  CU(c, cudaMemcpyAsync(tmp, g, bytes, is_device_ptr(g) ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice, s));
+  if (!direct_g || !direct_out) CU(c, cudaMallocAsync((void**)&tmp, bytes, s));
+  if (!direct_g) CU(c, cudaMemcpyAsync(tmp, g, bytes, is_device_ptr(g) ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice, s));
+  const float* gin = direct_g ? g : tmp;
+  float* gout = direct_out ? out : tmp;
   const bool line = line_size(lv.n) > 0;  // its x passes read and write [n^3][3] themselves
-  if (!line) launch_aos_to_soa(tmp, lv.g, lv.n3, s);
+  if (!line) launch_aos_to_soa(gin, lv.g, lv.n3, s);
   // a one-level copy of the job that stores the preconditioned gradient instead of Adam
   Job oj = c->h;
   oj.L = 1;
@@ -1114,24 +1134,22 @@ pdg_status pdg_precondition(pdg_ctx* c, int level, const float* g, float* out, v
   oj.precondition = 1;
   oj.keep_pgrad = 1;
   oj.no_adam = 1;
-  oj.ext_in = line ? tmp : nullptr;
-  oj.ext_out = line ? tmp : nullptr;
-  Plan op;
-  std::memset(&op, 0, sizeof(op));
-  op.n_jobs = 1;
-  op.jobs[0] = c->op_job;
-  CU(c, cudaMemcpyAsync(c->op_job, &oj, sizeof(Job), cudaMemcpyHostToDevice, s));
-  CU(c, cudaMemcpyAsync(c->op_plan, &op, sizeof(Plan), cudaMemcpyHostToDevice, s));
-  launch_plan(c->op_plan, s);
+  oj.ext_in = line ? gin : nullptr;
+  oj.ext_out = line ? gout : nullptr;
+  launch_op_plan(oj, c->op_job, c->op_plan, s);
   Shape sh;
   sh.sms = c->sms;
   sh.add_level(lv.n);
-  for (int i = ST_SOB_FIRST; i <= ST_SOB_LAST; ++i) launch_stage(i, c->op_plan, sh, s);
-  if (!line) launch_soa_to_aos(lv.tmp, tmp, lv.n3, s);
+  if (line) launch_stage(S_SOB_256, c->op_plan, sh, s);
+  else
+    for (int i = S_SOB_XY_FWD; i <= S_SOB_XY_INV; ++i) launch_stage(i, c->op_plan, sh, s);
+  if (!line) {
+    launch_soa_to_aos(lv.tmp, gout, lv.n3, s);
+    CU(c, cudaMemsetAsync(lv.g, 0, bytes, s));
+  }
   CU(c, cudaGetLastError());
-  const pdg_status st = copy_out(c, out, tmp, bytes, s);
-  cudaFreeAsync(tmp, s);
-  CU(c, cudaMemsetAsync(lv.g, 0, bytes, s));
+  const pdg_status st = direct_out ? PDG_OK : copy_out(c, out, tmp, bytes, s);
+  if (tmp) cudaFreeAsync(tmp, s);
   CU(c, cudaStreamSynchronize(s));
   return st;
 }
@@ -1164,13 +1182,7 @@ pdg_status pdg_fit_mesh(pdg_ctx* c, const float* p0_xyz, int n_p0, int n_steps, 
   mj.w_pts = 0.f;
   mj.w_iso = 0.f;
   mj.count_nn = 0;
-  CU(c, cudaMemcpyAsync(c->op_job, &mj, sizeof(Job), cudaMemcpyHostToDevice, s));
-  Plan op;
-  std::memset(&op, 0, sizeof(op));
-  op.n_jobs = 1;
-  op.jobs[0] = c->op_job;
-  CU(c, cudaMemcpyAsync(c->op_plan, &op, sizeof(Plan), cudaMemcpyHostToDevice, s));
-  launch_plan(c->op_plan, s);
+  launch_op_plan(mj, c->op_job, c->op_plan, s);
   float4* h = c->mesh;
   float4* r = h + V;
   float4* d0 = r + V;
