@@ -1,6 +1,7 @@
 // Host-side launchers of the libpdg kernels (each defined next to its kernels).
 #pragma once
 #include <algorithm>
+#include <vector>
 
 #include "pdg_internal.cuh"
 
@@ -59,10 +60,21 @@ void launch_sobz_pivots(float* piv, int* slow, const float* mu, int n, float lam
 
 // template-mesh fit (k_mesh.cu)
 void launch_mesh_points(Job* J, int V, cudaStream_t s);
-void launch_mesh_solve(const int* v2e_ptr, const int* v2e, const int2* edges, const float4* b, float4* h, float4* r,
-                       float4* d0, float4* d1, int V, float lam, float emax, int iters, cudaStream_t s);
-void launch_mesh_adam(float4* x, const float4* g, float4* m, float4* v, int V, float lr, float b1, float b2, float eps,
-                      float bias1, float ibias2, cudaStream_t s);
+// (I + lambda L)^{-2} b by two Chebyshev solves, then Adam on x
+struct MeshSolve {
+  const int *ptr, *nbr;  // neighbour lists of the vertices
+  const float4* b;       // right-hand side
+  float4 *h, *r, *d0, *d1;
+  float4 *pg;            // the result
+  float4 *x, *m, *v;
+  float2* coef;          // [iters] constants of the recurrence (mesh_coef)
+  unsigned* bar;         // grid barrier
+  int* err;              // set when the barrier's wait ran out
+  int V, iters;
+  float lam, inv_theta, lr, b1, b2, eps, bias1, ibias2;
+};
+void mesh_coef(std::vector<float2>& coef, int iters, float emax);
+cudaError_t launch_mesh_solve(MeshSolve a, float emax, int sms, cudaStream_t s);
 
 // misc conversions
 void launch_soa_to_aos(const float* in, float* out, int n3, cudaStream_t s, int C = 3);

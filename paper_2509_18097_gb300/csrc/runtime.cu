@@ -178,6 +178,9 @@ struct pdg_ctx {
   Plan* op_plan = nullptr;
   int* dflag = nullptr;
   float4* mesh = nullptr;  // [7][V]: h, r, d0, d1, preconditioned gradient, Adam m, Adam v
+  int* nbr = nullptr;      // [2E] neighbours of each vertex, v2e_ptr's ranges
+  float2* coef = nullptr;  // [MESH_ITERS_MAX] constants of the solves
+  unsigned* bar = nullptr; // grid barrier of the solves, and their error flag
   int max_degree = 0;      // largest vertex degree of the mesh (bounds the Laplacian's spectrum)
   bool mesh_valid = false; // a template-mesh fit has run (PDG_BUF_MESH_* readable)
   float* stage = nullptr;  // [stage_pts][3] staging of host inputs
@@ -225,6 +228,9 @@ struct pdg_batch {
 namespace {
 
 // sizes of every buffer of a context (used by pdg_query_bytes and pdg_create)
+// Chebyshev iterations of a template-mesh solve at the largest lambda times degree (1e5): 5125
+constexpr int MESH_ITERS_MAX = 5200;
+
 struct Layout {
   size_t total = 0;
   size_t job, plan, flag, stage, op_job, op_plan;
@@ -240,6 +246,7 @@ struct Layout {
     int bits;
   } tgt, mov;
   size_t xs, step, bias, loss, status, loss_part, gmax, counters;
+  size_t nbr, coef, bar;
   size_t mesh;  // template-mesh fit: 7 float4 [V] arrays (gradient copy, solves, Adam moments)
 };
 
@@ -327,6 +334,9 @@ Layout make_layout(const pdg_config& c, int V, int E, int max_pts) {
   L.gmax = a.take<unsigned>(1);
   L.counters = a.take<unsigned long long>(4);
   L.mesh = a.take<float4>(7 * (size_t)V);
+  L.nbr = a.take<int>(std::max(2 * E, 1));
+  L.coef = a.take<float2>(MESH_ITERS_MAX);
+  L.bar = a.take<unsigned>(2);
   L.total = (a.off + 255) & ~size_t(255);
   return L;
 }
@@ -621,6 +631,9 @@ pdg_status pdg_create(const pdg_config* cfg, const float* template_xyz, int n_ve
     }
   }
 
+  std::vector<int> nbr(c->v2e.size());
+  for (size_t k = 0; k < 2 * (size_t)n_edges; ++k) nbr[k] = he[2 * (size_t)(c->v2e[k] >> 1) + (c->v2e[k] & 1 ? 0 : 1)];
+
   const Layout L = make_layout(*cfg, n_verts, n_edges, max_pts);
   if (dev_malloc((void**)&c->arena, L.total) != cudaSuccess) {
     cudaGetLastError();
@@ -660,6 +673,9 @@ pdg_status pdg_create(const pdg_config* cfg, const float* template_xyz, int n_ve
   c->op_plan = (Plan*)P(L.op_plan);
   c->dflag = (int*)P(L.flag);
   c->mesh = (float4*)P(L.mesh);
+  c->nbr = (int*)P(L.nbr);
+  c->coef = (float2*)P(L.coef);
+  c->bar = (unsigned*)P(L.bar);
   c->stage = (float*)P(L.stage);
   c->stage_pts = std::max(n_verts, max_pts);
   std::vector<float> mu;
@@ -774,7 +790,8 @@ pdg_status pdg_create(const pdg_config* cfg, const float* template_xyz, int n_ve
 
   if (n_edges) {
     if (cudaMemcpyAsync((void*)J.edges, he.data(), he.size() * 4, cudaMemcpyHostToDevice, s) != cudaSuccess ||
-        cudaMemcpyAsync((void*)J.v2e, c->v2e.data(), c->v2e.size() * 4, cudaMemcpyHostToDevice, s) != cudaSuccess)
+        cudaMemcpyAsync((void*)J.v2e, c->v2e.data(), c->v2e.size() * 4, cudaMemcpyHostToDevice, s) != cudaSuccess ||
+        cudaMemcpyAsync(c->nbr, nbr.data(), nbr.size() * 4, cudaMemcpyHostToDevice, s) != cudaSuccess)
       return bail(PDG_ERR_CUDA);
   }
   if (cudaMemcpyAsync((void*)J.v2e_ptr, c->v2e_ptr.data(), c->v2e_ptr.size() * 4, cudaMemcpyHostToDevice, s) !=
@@ -1204,7 +1221,32 @@ pdg_status pdg_fit_mesh(pdg_ctx* c, const float* p0_xyz, int n_p0, int n_steps, 
   const double sk = std::sqrt(emax);
   const double q = (sk - 1.0) / (sk + 1.0);
   const int iters = q > 0.0 ? (int)std::ceil(std::log(1e-7 / (2.0 * sk)) / std::log(q)) : 1;
-  const int2* edges = J.edges;
+  MeshSolve ms{};
+  ms.ptr = J.v2e_ptr;
+  ms.nbr = c->nbr;
+  ms.b = J.gy;
+  ms.h = h;
+  ms.r = r;
+  ms.d0 = d0;
+  ms.d1 = d1;
+  ms.pg = pg;
+  ms.x = J.x;
+  ms.m = am;
+  ms.v = av;
+  ms.coef = c->coef;
+  ms.bar = c->bar;
+  ms.err = reinterpret_cast<int*>(c->bar + 1);
+  ms.V = V;
+  ms.iters = iters;
+  ms.lam = lambda;
+  ms.lr = lr;
+  ms.b1 = J.beta1;
+  ms.b2 = J.beta2;
+  ms.eps = J.eps;
+  CU(c, cudaMemsetAsync(ms.err, 0, sizeof(int), s));
+  std::vector<float2> coef;
+  mesh_coef(coef, iters, (float)emax);
+  CU(c, cudaMemcpyAsync(c->coef, coef.data(), sizeof(float2) * coef.size(), cudaMemcpyHostToDevice, s));
   Shape sh;
   sh.sms = c->sms;
   sh.add_points(V, 0, n_p0);
@@ -1214,22 +1256,20 @@ pdg_status pdg_fit_mesh(pdg_ctx* c, const float* p0_xyz, int n_p0, int n_steps, 
     launch_stage(S_ASSEMBLE, c->op_plan, sh, s);
     launch_stage(S_LOSS, c->op_plan, sh, s);
     // (I + lambda L)^{-2} dL/dX by two solves, then Adam on the vertices
-    launch_mesh_solve(J.v2e_ptr, J.v2e, edges, J.gy, h, r, d0, d1, V, lambda, (float)emax, iters, s);
-    launch_mesh_solve(J.v2e_ptr, J.v2e, edges, h, pg, r, d0, d1, V, lambda, (float)emax, iters, s);
-    const float bias1 = (float)(1.0 / (1.0 - std::pow((double)J.beta1, k)));
-    const float ibias2 = (float)(1.0 / std::sqrt(1.0 - std::pow((double)J.beta2, k)));
-    launch_mesh_adam(J.x, pg, am, av, V, lr, J.beta1, J.beta2, J.eps, bias1, ibias2, s);
-    CU(c, cudaGetLastError());
+    ms.bias1 = (float)(1.0 / (1.0 - std::pow((double)J.beta1, k)));
+    ms.ibias2 = (float)(1.0 / std::sqrt(1.0 - std::pow((double)J.beta2, k)));
+    CU(c, launch_mesh_solve(ms, (float)emax, c->sms, s));
   }
   CU(c, cudaMemcpyAsync(J.verts4, J.x, sizeof(float4) * V, cudaMemcpyDeviceToDevice, s));
   double loss[4];
-  int status = 0;
+  int status = 0, gave_up = 0;
   CU(c, cudaMemcpyAsync(loss, J.loss, sizeof(loss), cudaMemcpyDeviceToHost, s));
   CU(c, cudaMemcpyAsync(&status, J.status, sizeof(int), cudaMemcpyDeviceToHost, s));
+  CU(c, cudaMemcpyAsync(&gave_up, ms.err, sizeof(int), cudaMemcpyDeviceToHost, s));
   CU(c, cudaStreamSynchronize(s));
   c->mesh_valid = n_steps > 0;
   c->plan_stale = true;  // the frame plan is recomputed at the next frame
-  const pdg_status st = status ? PDG_ERR_NONFINITE : PDG_OK;
+  const pdg_status st = gave_up ? PDG_ERR_TIMEOUT : status ? PDG_ERR_NONFINITE : PDG_OK;
   if (stats) {
     stats->loss_total = loss[0];
     stats->cd_mesh = loss[1];
@@ -1239,7 +1279,8 @@ pdg_status pdg_fit_mesh(pdg_ctx* c, const float* p0_xyz, int n_p0, int n_steps, 
     stats->status = st;
     stats->nn_ties = -1;
   }
-  if (st != PDG_OK) c->err = "a loss became NaN or Inf during the mesh fit";
+  if (st != PDG_OK)
+    c->err = gave_up ? "a wait of the mesh solves ran out" : "a loss became NaN or Inf during the mesh fit";
   return st;
 }
 

@@ -1,0 +1,31 @@
+"""The template-mesh solves in one launch (k_mesh.cu, k_mesh_solve): one, two and four vertices per
+thread, a mesh too large for it (a launch per iteration), vertices with more neighbours than a
+thread holds and with none.  One iteration each, every stage against the oracle on the GPU's own
+input, at the tolerances of test_gpu_mesh.py (two Chebyshev solves to 1e-7, their FP32 recurrences
+within 1.1e-6 of max|result|)."""
+import numpy as np
+import pytest
+
+from paper_2509_18097_gb300 import synth
+from tests import test_gpu_mesh as M
+
+pytestmark = pytest.mark.gpu
+
+
+def cloud(n=2000):
+    r = np.random.Generator(np.random.PCG64(5))
+    return (synth.torus_points(r, n) * 1.02).astype(np.float32)
+
+
+# one thread block takes 512 vertices times those per thread, on at most 152 SMs
+@pytest.mark.parametrize("nu,nv", [(27, 19), (396, 198), (560, 280), (800, 400)])
+def test_torus(nu, nv):
+    v, _, e = synth.torus_mesh(nu, nv)
+    M.check_one_step(v, e, cloud())
+
+
+def test_hub_and_isolated_vertices():
+    r = np.random.Generator(np.random.PCG64(6))
+    v = synth.torus_points(r, 60).astype(np.float32)
+    e = np.stack([np.zeros(40, np.int32), np.arange(1, 41, dtype=np.int32)], 1)  # vertices 41..59 have no edge
+    M.check_one_step(v, e, cloud(300))
