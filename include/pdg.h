@@ -259,7 +259,7 @@ pdg_status pdg_load_state(pdg_ctx* ctx, const void* host_buf, size_t n, void* cu
  * out = (I + lambda L)^{-2} g per channel on a res^3 vertex grid (L the free-boundary
  * 6-neighbour graph Laplacian), computed by the same preconditioner kernels as
  * pdg_precondition, without a context and without allocating: its scratch lives in one
- * fixed file-scope device array of about 6.5 MB (two res^3 x 3 float buffers and the z-solve
+ * fixed file-scope device array of about 3.7 MB (a res^3 x 3 float buffer and the z-solve
  * pivot table at the maximum res, plus small tables and records), which every GPU that loads
  * the library keeps until the process exits.
  *  - g, out: DEVICE pointers of the current device to float [res^3][3] ((z*res + y)*res + x);

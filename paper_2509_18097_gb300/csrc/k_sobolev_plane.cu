@@ -171,15 +171,25 @@ __device__ __forceinline__ void plane_write2(float* plane, int r, int x, float2 
 // j = t + N1 m of the even/odd reordering v[j] = x[dsrc(j)].  Each thread loads the pairs
 // (x[2s], x[2s+1]) at s = t + N1 m' (m' < N2/2): the even element is its own v[s], the odd
 // one is v[n - 1 - s] of lane t ^ (N1 - 1).
-template <int N1, int N2>
+// EXT: the elements are 3 floats apart (a caller's [n^3][3] array).
+template <int N1, int N2, bool EXT>
 __device__ __forceinline__ void load_fwd_rows(const float* __restrict__ rowA, const float* __restrict__ rowB, int t,
                                               float2 (&reg)[N2]) {
   constexpr int H = N2 / 2;
   float2 ea[H], eb[H];
+  if (EXT) {
 #pragma unroll
-  for (int m = 0; m < H; ++m) {
-    ea[m] = __ldg(reinterpret_cast<const float2*>(rowA) + t + N1 * m);
-    eb[m] = __ldg(reinterpret_cast<const float2*>(rowB) + t + N1 * m);
+    for (int m = 0; m < H; ++m) {
+      const int s = 6 * (t + N1 * m);
+      ea[m] = make_float2(__ldg(rowA + s), __ldg(rowA + s + 3));
+      eb[m] = make_float2(__ldg(rowB + s), __ldg(rowB + s + 3));
+    }
+  } else {
+#pragma unroll
+    for (int m = 0; m < H; ++m) {
+      ea[m] = __ldg(reinterpret_cast<const float2*>(rowA) + t + N1 * m);
+      eb[m] = __ldg(reinterpret_cast<const float2*>(rowB) + t + N1 * m);
+    }
   }
 #pragma unroll
   for (int m = 0; m < H; ++m) reg[m] = make_float2(ea[m].x, eb[m].x);
@@ -274,7 +284,7 @@ __device__ __forceinline__ bool plane_item(const Job& J, int r, int& l, int& idx
 
 // DCT-II along x (rows, from global memory) then y (columns of the shared plane, to global
 // memory) of the z-plane `in` (n x n floats) into `out`.
-template <int N1, int N2>
+template <int N1, int N2, bool EXT>
 __device__ void plane_fwd(const Level& lv, const float* __restrict__ in, float* __restrict__ out, float* plane,
                           float2* scr) {
   constexpr int n = N1 * N2, GB = PL_THREADS / N1;
@@ -285,7 +295,8 @@ __device__ void plane_fwd(const Level& lv, const float* __restrict__ in, float* 
   // multiple of 32), and N1 = 1 has no warp-collective step
   for (int p = gi; p < n / 2; p += GB) {  // x-lines: rows 2p, 2p + 1
     float2 reg[N2];
-    load_fwd_rows<N1, N2>(in + (2 * p) * n, in + (2 * p + 1) * n, t, reg);
+    constexpr int es = EXT ? 3 * n : n;  // floats from row to row
+    load_fwd_rows<N1, N2, EXT>(in + (2 * p) * es, in + (2 * p + 1) * es, t, reg);
     fft2<N1, N2, false>(reg, sc, t, lv.tw);
     float XA[N2], XB[N2];
     dct2_post<N1, N2>(reg, t, lbase, lv.tw4, XA, XB);
@@ -311,6 +322,8 @@ __device__ void plane_fwd(const Level& lv, const float* __restrict__ in, float* 
   __syncthreads();
 }
 
+// EXT (both passes): a caller's gradient in, its preconditioned form out, [n^3][3] each
+template <bool EXT>
 __global__ void __launch_bounds__(PL_THREADS, 2) k_sobp(const Plan* __restrict__ P) {
   extern __shared__ float smem[];
   const int nj = P->n_jobs;
@@ -325,23 +338,24 @@ __global__ void __launch_bounds__(PL_THREADS, 2) k_sobp(const Plan* __restrict__
     const int n = lv.n, n3 = lv.n3;
     const int q = idx / J.C, c = idx - J.C * q;  // z-plane, channel
     if (n == 1) {  // no transform: copy g to tmp (the scale is 1)
-      if (threadIdx.x == 0) lv.tmp[c] = lv.g[c];
+      if (threadIdx.x == 0) lv.tmp[c] = EXT ? J.ext_in[c] : lv.g[c];
       continue;
     }
     // the gradient lives on the vertices near the data: a z-plane without an active vertex
     // stays zero, and pass B reads it as zero without loading it
     if (lv.zmask && !__ldg(lv.zmask + q)) continue;
     const size_t off = (size_t)c * n3 + (size_t)q * n * n;
+    const float* in = EXT ? J.ext_in + 3 * (size_t)q * n * n + c : lv.g + off;
     float* plane = smem;
     float2* scr = reinterpret_cast<float2*>(smem + ((plane_floats(n) + 1) & ~1));
     switch (n) {
-      case 2: plane_fwd<1, 2>(lv, lv.g + off, lv.tmp + off, plane, scr); break;
-      case 4: plane_fwd<1, 4>(lv, lv.g + off, lv.tmp + off, plane, scr); break;
-      case 8: plane_fwd<1, 8>(lv, lv.g + off, lv.tmp + off, plane, scr); break;
-      case 16: plane_fwd<1, 16>(lv, lv.g + off, lv.tmp + off, plane, scr); break;
-      case 32: plane_fwd<4, 8>(lv, lv.g + off, lv.tmp + off, plane, scr); break;
-      case 64: plane_fwd<8, 8>(lv, lv.g + off, lv.tmp + off, plane, scr); break;
-      default: plane_fwd<8, 16>(lv, lv.g + off, lv.tmp + off, plane, scr); break;
+      case 2: plane_fwd<1, 2, EXT>(lv, in, lv.tmp + off, plane, scr); break;
+      case 4: plane_fwd<1, 4, EXT>(lv, in, lv.tmp + off, plane, scr); break;
+      case 8: plane_fwd<1, 8, EXT>(lv, in, lv.tmp + off, plane, scr); break;
+      case 16: plane_fwd<1, 16, EXT>(lv, in, lv.tmp + off, plane, scr); break;
+      case 32: plane_fwd<4, 8, EXT>(lv, in, lv.tmp + off, plane, scr); break;
+      case 64: plane_fwd<8, 8, EXT>(lv, in, lv.tmp + off, plane, scr); break;
+      default: plane_fwd<8, 16, EXT>(lv, in, lv.tmp + off, plane, scr); break;
     }
   }
 }
@@ -462,7 +476,7 @@ __device__ __forceinline__ void column_solve(float* __restrict__ t, const float*
 
 // an item is COLS_PER_ITEM consecutive columns (col = y n + x) of one channel of one level
 __device__ __forceinline__ bool column_item(const Job& J, int r, int& l, int& c, int& col0) {
-  for (l = 0; l < J.L; ++l) {
+  for (l = J.L - 1; l >= 0; --l) {  // the finest level first: its columns take longest
     const int n = J.lev[l].n;
     if (tile_level(n)) continue;
     const int per = (n * n + COLS_PER_ITEM - 1) / COLS_PER_ITEM;
@@ -537,7 +551,7 @@ __global__ void __launch_bounds__(COL_THREADS, 4) k_sobz(const Plan* __restrict_
 // Inverse DCT along y (columns, from global memory) then x (rows of the shared plane) of
 // z-plane q, channel c; the preconditioned gradient goes back to tmp (coalesced pairs of
 // neighbouring columns) for the Adam kernel.
-template <int N1, int N2>
+template <int N1, int N2, bool EXT>
 __device__ void plane_inv(const Job& J, const Level& lv, int c, int q, float* plane, float2* scr) {
   constexpr int n = N1 * N2, GB = PL_THREADS / N1, H = N2 / 2;
   const int gi = threadIdx.x / N1, t = threadIdx.x % N1;
@@ -586,6 +600,18 @@ __device__ void plane_inv(const Job& J, const Level& lv, int c, int q, float* pl
       gb[h] = make_float2(reg[idx].y, o.y);
     }
     const size_t rowA = poff + (size_t)(2 * p) * n, rowB = rowA + n;
+    if (EXT) {  // a caller's [n^3][3] array
+      float* ea = J.ext_out + 3 * rowA + c;
+      float* eb = J.ext_out + 3 * rowB + c;
+#pragma unroll
+      for (int h = 0; h < H; ++h) {
+        ea[3 * xs[h]] = ga[h].x;
+        ea[3 * xs[h] + 3] = ga[h].y;
+        eb[3 * xs[h]] = gb[h].x;
+        eb[3 * xs[h] + 3] = gb[h].y;
+      }
+      continue;
+    }
 #pragma unroll
     for (int h = 0; h < H; ++h) {
       *reinterpret_cast<float2*>(out + rowA + xs[h]) = ga[h];
@@ -595,6 +621,7 @@ __device__ void plane_inv(const Job& J, const Level& lv, int c, int q, float* pl
   __syncthreads();
 }
 
+template <bool EXT>
 __global__ void __launch_bounds__(PL_THREADS, 2) k_sobp_inv(const Plan* __restrict__ P) {
   extern __shared__ float smem[];
   const int nj = P->n_jobs;
@@ -608,17 +635,20 @@ __global__ void __launch_bounds__(PL_THREADS, 2) k_sobp_inv(const Plan* __restri
     const Level& lv = J.lev[l];
     const int n = lv.n;
     const int q = idx / J.C, c = idx - J.C * q;
-    if (n == 1) continue;  // tmp already holds the preconditioned gradient (the operator is 1)
+    if (n == 1) {  // tmp already holds the preconditioned gradient (the operator is 1)
+      if (EXT && threadIdx.x == 0) J.ext_out[c] = lv.tmp[c];
+      continue;
+    }
     float* plane = smem;
     float2* scr = reinterpret_cast<float2*>(smem + ((plane_floats(n) + 1) & ~1));
     switch (n) {
-      case 2: plane_inv<1, 2>(J, lv, c, q, plane, scr); break;
-      case 4: plane_inv<1, 4>(J, lv, c, q, plane, scr); break;
-      case 8: plane_inv<1, 8>(J, lv, c, q, plane, scr); break;
-      case 16: plane_inv<1, 16>(J, lv, c, q, plane, scr); break;
-      case 32: plane_inv<4, 8>(J, lv, c, q, plane, scr); break;
-      case 64: plane_inv<8, 8>(J, lv, c, q, plane, scr); break;
-      default: plane_inv<8, 16>(J, lv, c, q, plane, scr); break;
+      case 2: plane_inv<1, 2, EXT>(J, lv, c, q, plane, scr); break;
+      case 4: plane_inv<1, 4, EXT>(J, lv, c, q, plane, scr); break;
+      case 8: plane_inv<1, 8, EXT>(J, lv, c, q, plane, scr); break;
+      case 16: plane_inv<1, 16, EXT>(J, lv, c, q, plane, scr); break;
+      case 32: plane_inv<4, 8, EXT>(J, lv, c, q, plane, scr); break;
+      case 64: plane_inv<8, 8, EXT>(J, lv, c, q, plane, scr); break;
+      default: plane_inv<8, 16, EXT>(J, lv, c, q, plane, scr); break;
     }
   }
 }
@@ -747,17 +777,27 @@ int plane_smem_max(int nmax) {
 
 void sobolev_plane_configure() {
   const int smem = plane_smem_max(128);
-  cudaFuncSetAttribute(k_sobp, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-  cudaFuncSetAttribute(k_sobp_inv, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  cudaFuncSetAttribute(k_sobp<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  cudaFuncSetAttribute(k_sobp<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  cudaFuncSetAttribute(k_sobp_inv<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  cudaFuncSetAttribute(k_sobp_inv<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
 }
 
-// part: 0 xy-forward, 1 z solve, 2 xy-inverse, 3 Adam, -1 all four
-void launch_sobolev_plane(const Plan* P, int grid, int nmax, cudaStream_t s, int part) {
+// part: 0 xy-forward, 1 z solve, 2 xy-inverse, 3 Adam; ext: on a caller's gradient (no Adam)
+void launch_sobolev_plane(const Plan* P, int grid, int nmax, cudaStream_t s, int part, bool ext) {
   const int smem = plane_smem_max(nmax);
-  if (part < 0 || part == 0) k_sobp<<<grid, PL_THREADS, smem, s>>>(P);
-  if (part < 0 || part == 1) k_sobz<<<grid * 3, COL_THREADS, 0, s>>>(P);
-  if (part < 0 || part == 2) k_sobp_inv<<<grid, PL_THREADS, smem, s>>>(P);
-  if (part < 0 || part == 3) k_adam<<<grid * 8, 256, 0, s>>>(P);
+  switch (part) {
+    case 0:
+      if (ext) k_sobp<true><<<grid, PL_THREADS, smem, s>>>(P);
+      else k_sobp<false><<<grid, PL_THREADS, smem, s>>>(P);
+      break;
+    case 1: k_sobz<<<grid * 3, COL_THREADS, 0, s>>>(P); break;
+    case 2:
+      if (ext) k_sobp_inv<true><<<grid, PL_THREADS, smem, s>>>(P);
+      else k_sobp_inv<false><<<grid, PL_THREADS, smem, s>>>(P);
+      break;
+    case 3: k_adam<<<grid * 8, 256, 0, s>>>(P); break;
+  }
 }
 
 }  // namespace pdg

@@ -15,10 +15,9 @@ namespace pdg {
 
 constexpr int STATIC_MAX_RES = PDG_STATIC_MAX_RES;
 constexpr size_t STATIC_N3 = (size_t)STATIC_MAX_RES * STATIC_MAX_RES * STATIC_MAX_RES;
-// layout: g (SoA, 3 n^3 floats) | tmp (3 n^3) | z-solve pivots ((n/2 + 1) n^2) | mu (n) | tw (n float2) | tw4 (n float2) |
+// layout: tmp (3 n^3 floats) | z-solve pivots ((n/2 + 1) n^2) | mu (n) | tw (n float2) | tw4 (n float2) |
 //         n_active (int) + bias (2 floats, read by the pass even when it skips Adam) | pivot flag | job | plan
-constexpr size_t SO_G = 0;
-constexpr size_t SO_TMP = SO_G + 3 * STATIC_N3 * sizeof(float);
+constexpr size_t SO_TMP = 0;
 constexpr size_t SO_PIV = SO_TMP + 3 * STATIC_N3 * sizeof(float);
 constexpr size_t SO_MU =
     SO_PIV + (size_t)(STATIC_MAX_RES / 2 + 1) * STATIC_MAX_RES * STATIC_MAX_RES * sizeof(float);
@@ -79,7 +78,7 @@ bool on_current_device(const void* p) {
 // one-level job that stops at the preconditioned gradient, and its plan into the scratch
 // array.  Everything comes in as kernel arguments, so the call copies nothing from host
 // memory.  One block.
-__global__ void k_static_setup(unsigned char* base, int n, int lg, float lam) {
+__global__ void k_static_setup(unsigned char* base, int n, int lg, float lam, const float* g, float* out) {
   float* mu = reinterpret_cast<float*>(base + SO_MU);
   float2* tw = reinterpret_cast<float2*>(base + SO_TW);
   float2* tw4 = reinterpret_cast<float2*>(base + SO_TW4);
@@ -109,7 +108,8 @@ __global__ void k_static_setup(unsigned char* base, int n, int lg, float lam) {
     lv.lg = lg;
     lv.n3 = n * n * n;
     lv.lam = lam;
-    lv.g = reinterpret_cast<float*>(base + SO_G);
+    J.ext_in = g;
+    J.ext_out = out;
     lv.tmp = reinterpret_cast<float*>(base + SO_TMP);
     lv.piv = reinterpret_cast<float*>(base + SO_PIV);
     lv.piv_slow = reinterpret_cast<int*>(base + SO_SLOW);
@@ -144,23 +144,18 @@ extern "C" pdg_status pdg_precondition_static(int res, float lambda, const float
   if (st != PDG_OK) return st;
   cudaStream_t s = (cudaStream_t)cuda_stream;
   const int n = res;
-  const int n3 = n * n * n;
   int lg = 0;
   while ((1 << lg) < n) ++lg;
-  k_static_setup<<<1, 256, 0, s>>>(base, n, lg, lambda);
-  float* lv_g = reinterpret_cast<float*>(base + SO_G);
-  float* lv_tmp = reinterpret_cast<float*>(base + SO_TMP);
+  k_static_setup<<<1, 256, 0, s>>>(base, n, lg, lambda, g, out);
   launch_sobz_pivots(reinterpret_cast<float*>(base + SO_PIV), reinterpret_cast<int*>(base + SO_SLOW),
                      reinterpret_cast<const float*>(base + SO_MU), n, lambda, s);
   Plan* dP = reinterpret_cast<Plan*>(base + SO_PLAN);
-  launch_aos_to_soa(g, lv_g, n3, s);
   launch_plan(dP, s);
   int sms = 1, dev = 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   const int per_sm = (227 * 1024) / plane_smem_max(n) < 8 ? (227 * 1024) / plane_smem_max(n) : 8;
-  launch_sobolev_plane(dP, sms * (per_sm > 0 ? per_sm : 1), n, s);
-  launch_soa_to_aos(lv_tmp, out, n3, s);
+  for (int part = 0; part < 3; ++part) launch_sobolev_plane(dP, sms * (per_sm > 0 ? per_sm : 1), n, s, part, true);  // no Adam
   return cudaGetLastError() == cudaSuccess ? PDG_OK : PDG_ERR_CUDA;
 }
 

@@ -24,7 +24,7 @@ void launch_adjoint(const Plan* P, int grid, cudaStream_t s);
 enum YzPass { YZ_FWD = 0, YZ_Z, YZ_INV };
 void launch_sobolev_x(const Plan* P, int sms, int nmax, bool fwd, cudaStream_t s);
 void launch_sobolev_yz(const Plan* P, int sms, int nmax, int pass, cudaStream_t s);
-void launch_sobolev_plane(const Plan* P, int grid, int nmax, cudaStream_t s, int part = -1);
+void launch_sobolev_plane(const Plan* P, int grid, int nmax, cudaStream_t s, int part, bool ext);
 void launch_loss(const Plan* P, int grid, cudaStream_t s);
 
 // per frame / per call (one job)

@@ -47,6 +47,7 @@ struct Shape {
   int sms = 1;
   int nmax = 1;   // largest level resolution
   int nline = 0;  // largest resolution among the levels the line path preconditions (0: none)
+  bool ext = false;  // the preconditioner on a caller's gradient
   int nodes = 0, supers = 0;  // interpolation, upper boxes
   int nnf = 0, nnr = 0;       // searches: warps of 32 queries, of the moving points and of the targets
 
@@ -425,7 +426,7 @@ void launch_stage(int i, const Plan* plan, const Shape& sh, cudaStream_t s, int 
     case S_ADAM: {
       const int ps = plane_smem_max(sh.nmax);
       const int per_sm = std::max(1, std::min(8, (227 * 1024) / ps));
-      launch_sobolev_plane(plan, sms * per_sm, sh.nmax, s, i - S_SOB_XY_FWD);
+      launch_sobolev_plane(plan, sms * per_sm, sh.nmax, s, i - S_SOB_XY_FWD, sh.ext);
       break;
     }
     case S_SOB_256:
@@ -1140,8 +1141,7 @@ pdg_status pdg_precondition(pdg_ctx* c, int level, const float* g, float* out, v
   if (!direct_g) CU(c, cudaMemcpyAsync(tmp, g, bytes, is_device_ptr(g) ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice, s));
   const float* gin = direct_g ? g : tmp;
   float* gout = direct_out ? out : tmp;
-  const bool line = line_size(lv.n) > 0;  // its x passes read and write [n^3][3] themselves
-  if (!line) launch_aos_to_soa(gin, lv.g, lv.n3, s);
+  const bool line = line_size(lv.n) > 0;
   // a one-level copy of the job that stores the preconditioned gradient instead of Adam
   Job oj = c->h;
   oj.L = 1;
@@ -1151,19 +1151,16 @@ pdg_status pdg_precondition(pdg_ctx* c, int level, const float* g, float* out, v
   oj.precondition = 1;
   oj.keep_pgrad = 1;
   oj.no_adam = 1;
-  oj.ext_in = line ? gin : nullptr;
-  oj.ext_out = line ? gout : nullptr;
+  oj.ext_in = gin;  // the passes read and write [n^3][3] themselves
+  oj.ext_out = gout;
   launch_op_plan(oj, c->op_job, c->op_plan, s);
   Shape sh;
   sh.sms = c->sms;
   sh.add_level(lv.n);
+  sh.ext = true;
   if (line) launch_stage(S_SOB_256, c->op_plan, sh, s);
   else
     for (int i = S_SOB_XY_FWD; i <= S_SOB_XY_INV; ++i) launch_stage(i, c->op_plan, sh, s);
-  if (!line) {
-    launch_soa_to_aos(lv.tmp, gout, lv.n3, s);
-    CU(c, cudaMemsetAsync(lv.g, 0, bytes, s));
-  }
   CU(c, cudaGetLastError());
   const pdg_status st = direct_out ? PDG_OK : copy_out(c, out, tmp, bytes, s);
   if (tmp) cudaFreeAsync(tmp, s);
