@@ -541,9 +541,9 @@ void launch_interp(const Plan* P, int grid, cudaStream_t s, int bump) { k_interp
 void launch_boxes(const Plan* P, int grid, cudaStream_t s) { k_boxes<<<grid, 64, 0, s>>>(P); }
 void launch_iso_edges(const Plan* P, int grid, cudaStream_t s) { k_iso_edges<<<grid, 256, 0, s>>>(P); }
 void launch_assemble(const Plan* P, int grid, cudaStream_t s) { k_assemble<<<grid, 256, 0, s>>>(P); }
-void launch_loss(const Plan* P, int grid, cudaStream_t s) {
-  k_loss_chunks<<<grid, 256, 0, s>>>(P);
-  k_loss_final<<<MAXJ, 256, 0, s>>>(P);
+void launch_loss(const Plan* P, int chunks, int jobs, cudaStream_t s) {
+  k_loss_chunks<<<chunks, 256, 0, s>>>(P);
+  k_loss_final<<<jobs, 256, 0, s>>>(P);
 }
 
 void launch_pack4(const float* in, float4* out, int n, cudaStream_t s) {
@@ -579,13 +579,15 @@ void launch_soa_to_aos(const float* in, float* out, int n3, cudaStream_t s, int 
   k_soa_to_aos<<<blocks_for(n3, 256), 256, 0, s>>>(in, out, n3, C);
 }
 
-// level values [n3][C] <-> the float4 arrays of a level (theta; theta_t holds channels 3..5)
-__global__ void k_pack_theta(const float* __restrict__ in, float4* __restrict__ th, float4* __restrict__ tht, int n3,
-                             int C) {
+// level values [n3][C] <-> the float4 arrays of a level (theta; theta_t holds channels 3..5); packing
+// also clears the level's Adam moments
+__global__ void k_pack_theta(const float* __restrict__ in, float4* __restrict__ th, float4* __restrict__ tht,
+                             float* __restrict__ m, float* __restrict__ v, int n3, int C) {
   for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n3; i += gridDim.x * blockDim.x) {
     const float* r = in + (size_t)C * i;
     th[i] = make_float4(r[0], r[1], r[2], 0.f);
     if (C == 6) tht[i] = make_float4(r[3], r[4], r[5], 0.f);
+    for (int c = 0; c < C; ++c) m[(size_t)c * n3 + i] = v[(size_t)c * n3 + i] = 0.f;
   }
 }
 __global__ void k_unpack_theta(const float4* __restrict__ th, const float4* __restrict__ tht, float* __restrict__ out,
@@ -600,8 +602,8 @@ __global__ void k_unpack_theta(const float4* __restrict__ th, const float4* __re
     }
   }
 }
-void launch_pack_theta(const float* in, float4* th, float4* tht, int n3, int C, cudaStream_t s) {
-  k_pack_theta<<<blocks_for(n3, 256), 256, 0, s>>>(in, th, tht, n3, C);
+void launch_pack_theta(const float* in, float4* th, float4* tht, float* m, float* v, int n3, int C, cudaStream_t s) {
+  k_pack_theta<<<blocks_for(n3, 256), 256, 0, s>>>(in, th, tht, m, v, n3, C);
 }
 void launch_unpack_theta(const float4* th, const float4* tht, float* out, int n3, int C, cudaStream_t s) {
   k_unpack_theta<<<blocks_for(n3, 256), 256, 0, s>>>(th, tht, out, n3, C);

@@ -791,12 +791,12 @@ void launch_sobolev_plane(const Plan* P, int grid, int nmax, cudaStream_t s, int
       if (ext) k_sobp<true><<<grid, PL_THREADS, smem, s>>>(P);
       else k_sobp<false><<<grid, PL_THREADS, smem, s>>>(P);
       break;
-    case 1: k_sobz<<<grid * 3, COL_THREADS, 0, s>>>(P); break;
+    case 1: k_sobz<<<grid, COL_THREADS, 0, s>>>(P); break;
     case 2:
       if (ext) k_sobp_inv<true><<<grid, PL_THREADS, smem, s>>>(P);
       else k_sobp_inv<false><<<grid, PL_THREADS, smem, s>>>(P);
       break;
-    case 3: k_adam<<<grid * 8, 256, 0, s>>>(P); break;
+    case 3: k_adam<<<grid, 256, 0, s>>>(P); break;
   }
 }
 

@@ -242,9 +242,8 @@ void sobolev_x_configure() {
   cudaFuncSetAttribute(k_sob_x<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
 }
 
-void launch_sobolev_x(const Plan* P, int sms, int nmax, bool fwd, cudaStream_t s) {
+void launch_sobolev_x(const Plan* P, int grid, int nmax, bool fwd, cudaStream_t s) {
   const int smem = x_smem_max(nmax);
-  const int grid = sms * 3 * 4;
   if (fwd) k_sob_x<true><<<grid, X_THREADS, smem, s>>>(P);
   else k_sob_x<false><<<grid, X_THREADS, smem, s>>>(P);
 }

@@ -190,9 +190,8 @@ void sobolev_yz_configure() {
   cudaFuncSetAttribute(k_sob_yz<YZ_INV>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
 }
 
-void launch_sobolev_yz(const Plan* P, int sms, int nmax, int pass, cudaStream_t s) {
+void launch_sobolev_yz(const Plan* P, int grid, int nmax, int pass, cudaStream_t s) {
   const int smem = yz_smem_max(nmax);
-  const int grid = sms * 4 * 4;
   if (pass == YZ_FWD) k_sob_yz<YZ_FWD><<<grid, YZ_THREADS, smem, s>>>(P);
   else if (pass == YZ_Z) k_sob_yz<YZ_Z><<<grid, YZ_THREADS, smem, s>>>(P);
   else k_sob_yz<YZ_INV><<<grid, YZ_THREADS, smem, s>>>(P);

@@ -151,11 +151,10 @@ extern "C" pdg_status pdg_precondition_static(int res, float lambda, const float
                      reinterpret_cast<const float*>(base + SO_MU), n, lambda, s);
   Plan* dP = reinterpret_cast<Plan*>(base + SO_PLAN);
   launch_plan(dP, s);
-  int sms = 1, dev = 0;
-  cudaGetDevice(&dev);
-  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  const int per_sm = (227 * 1024) / plane_smem_max(n) < 8 ? (227 * 1024) / plane_smem_max(n) : 8;
-  for (int part = 0; part < 3; ++part) launch_sobolev_plane(dP, sms * (per_sm > 0 ? per_sm : 1), n, s, part, true);  // no Adam
+  // a block per plane and channel, 64 columns of a channel to a block
+  launch_sobolev_plane(dP, 3 * n, n, s, 0, true);
+  launch_sobolev_plane(dP, 3 * ((n * n + 63) / 64), n, s, 1, true);
+  launch_sobolev_plane(dP, 3 * n, n, s, 2, true);
   return cudaGetLastError() == cudaSuccess ? PDG_OK : PDG_ERR_CUDA;
 }
 

@@ -22,10 +22,10 @@ void launch_adjoint_rows(const Plan* P, int grid, cudaStream_t s);
 void launch_adjoint(const Plan* P, int grid, cudaStream_t s);
 // line path (256 and sizes with a factor 3); nmax: the largest level it takes in the plan
 enum YzPass { YZ_FWD = 0, YZ_Z, YZ_INV };
-void launch_sobolev_x(const Plan* P, int sms, int nmax, bool fwd, cudaStream_t s);
-void launch_sobolev_yz(const Plan* P, int sms, int nmax, int pass, cudaStream_t s);
+void launch_sobolev_x(const Plan* P, int grid, int nmax, bool fwd, cudaStream_t s);
+void launch_sobolev_yz(const Plan* P, int grid, int nmax, int pass, cudaStream_t s);
 void launch_sobolev_plane(const Plan* P, int grid, int nmax, cudaStream_t s, int part, bool ext);
-void launch_loss(const Plan* P, int grid, cudaStream_t s);
+void launch_loss(const Plan* P, int chunks, int jobs, cudaStream_t s);
 
 // per frame / per call (one job)
 void launch_pack4(const float* in, float4* out, int n, cudaStream_t s);
@@ -78,7 +78,7 @@ cudaError_t launch_mesh_solve(MeshSolve a, float emax, int sms, cudaStream_t s);
 
 // misc conversions
 void launch_soa_to_aos(const float* in, float* out, int n3, cudaStream_t s, int C = 3);
-void launch_pack_theta(const float* in, float4* th, float4* tht, int n3, int C, cudaStream_t s);
+void launch_pack_theta(const float* in, float4* th, float4* tht, float* m, float* v, int n3, int C, cudaStream_t s);
 void launch_unpack_theta(const float4* th, const float4* tht, float* out, int n3, int C, cudaStream_t s);
 void launch_aos_to_float4(const float* in, float4* out, int n, cudaStream_t s);
 void launch_copy_int(const int* in, int* out, int n, cudaStream_t s);

@@ -45,54 +45,95 @@ int line_size(int n) { return tile_level(n) ? n : 0; }
 // still costs its launch: 4864 of them about 4 us.
 struct Shape {
   int sms = 1;
-  int nmax = 1;   // largest level resolution
-  int nline = 0;  // largest resolution among the levels the line path preconditions (0: none)
+  int nmax = 1;      // largest level resolution
+  int nline = 0;     // largest resolution among the levels the line path preconditions (0: none)
   bool ext = false;  // the preconditioner on a caller's gradient
-  int nodes = 0, supers = 0;  // interpolation, upper boxes
-  int nnf = 0, nnr = 0;       // searches: warps of 32 queries, of the moving points and of the targets
+  enum Work {
+    NODES, SUPERS,  // interpolation, upper boxes
+    NNF, NNR,       // searches: warps of 32 queries, of the moving points and of the targets
+    POINTS, EDGES, LOSS, JOBS,
+    ROWS, ADJ,          // adjoint: blocks of long rows, blocks of warp groups
+    PLANES, COLS, ADAM,  // plane path
+    XT, YZ,              // line path
+    N_WORK
+  };
+  long w[N_WORK] = {};
 
-  // Lanes per query of the searches: 8 while that leaves no more than 32 warps per SM (a warp's own
-  // latency counts), else 2 (see k_nn.cu)
-  int nn_sub() const { return nnf + 2 * nnr < 4 * sms ? 8 : 2; }
-  int nn_grid(int warps) const { return std::max(1, std::min((warps * nn_sub() + 3) / 4, 32 * sms)); }
-
-  static void cap(int& v, long add, long most) { v = (int)std::min(v + add, most); }
-  // V, N points in the two moving sets, M targets
-  void add_points(long V, long N, long M) {
+  // V, N points in the two moving sets, M targets, E edges
+  void add_points(long V, long N, long M, long E) {
     const long vn = (V + NODE - 1) / NODE, pn = (N + NODE - 1) / NODE;
-    cap(nodes, vn + pn, 8L * sms);
-    cap(supers, ((vn + 31) / 32 + (pn + 31) / 32 + 1) / 2, sms);
-    cap(nnf, (V + 31) / 32 + (N + 31) / 32, 128L * sms);
-    cap(nnr, (M + 31) / 32, 128L * sms);
+    w[NODES] += vn + pn;
+    w[SUPERS] += (vn + 31) / 32 + (pn + 31) / 32;
+    w[NNF] += (V + 31) / 32 + (N + 31) / 32;
+    w[NNR] += (M + 31) / 32;
+    w[POINTS] += V + N;
+    w[EDGES] += E;
+    w[LOSS] += (V + N + (N > 0 ? 2 : 1) * M + E + LOSS_CHUNK - 1) / LOSS_CHUNK;
+    w[JOBS] += 1;
   }
-  void add_level(int n) {
-    nmax = std::max(nmax, n);
-    nline = std::max(nline, line_size(n));
+  // a level of n vertices per axis, C channels, Q points
+  void add_level(long n, long C, long Q) {
+    nmax = std::max(nmax, (int)n);
+    nline = std::max(nline, line_size((int)n));
+    // rows (active vertices) of at most 8 Q entries: a block each from 512 entries on average, else
+    // warps of up to 32 rows with at least half their lanes' entries
+    const long rows = std::min(n * n * n, 8 * Q);
+    w[ROWS] += std::min(rows, 8 * Q / 512 + 1);
+    w[ADJ] += (8 * Q / 256 + rows / 32 + 1 + 7) / 8;
+    if (line_size((int)n)) {
+      w[XT] += C / 3 * x_tiles((int)n);
+      w[YZ] += C * yz_tiles((int)n);
+    } else {
+      w[PLANES] += C * n;
+      w[COLS] += C * ((n * n + 63) / 64);
+      w[ADAM] += (n * n * n + 3) / 4;
+    }
   }
   void add(const Shape& o) {  // a batch's member
     sms = o.sms;
     nmax = std::max(nmax, o.nmax);
     nline = std::max(nline, o.nline);
-    cap(nodes, o.nodes, 8L * sms);
-    cap(supers, o.supers, sms);
-    cap(nnf, o.nnf, 128L * sms);
-    cap(nnr, o.nnr, 128L * sms);
+    for (int i = 0; i < N_WORK; ++i) w[i] += o.w[i];
   }
-  // componentwise maximum; true if it grew
-  bool grow(const Shape& o) {
-    bool g = false;
-    auto m = [&](int& a, int b) {
-      g = g || b > a;
-      a = std::max(a, b);
-    };
-    m(sms, o.sms);
-    m(nmax, o.nmax);
-    m(nline, o.nline);
-    m(nodes, o.nodes);
-    m(supers, o.supers);
-    m(nnf, o.nnf);
-    m(nnr, o.nnr);
-    return g;
+  // makes this cover `o` too; true if a launch of this shape would have had fewer blocks than one of
+  // `o` (or too little shared memory)
+  bool cover(const Shape& o) {
+    bool more = o.nmax > nmax || o.nline > nline || sms != o.sms;
+    for (int i = 0; i < N_WORK; ++i) more = more || blocks(i) < o.blocks(i);
+    if (!more) return false;
+    sms = o.sms;
+    nmax = std::max(nmax, o.nmax);
+    nline = std::max(nline, o.nline);
+    for (int i = 0; i < N_WORK; ++i) w[i] = std::max(w[i], o.w[i]);
+    return true;
+  }
+
+  // Lanes per query of the searches: 8 while that leaves no more than 32 warps per SM (a warp's own
+  // latency counts), else 2 (see k_nn.cu)
+  int nn_sub() const { return w[NNF] + 2 * w[NNR] < 4 * sms ? 8 : 2; }
+  int plane_blocks_per_sm() const { return std::max(1, std::min(8, (227 * 1024) / plane_smem_max(nmax))); }
+
+  // blocks of a launch: what the work fills, at most the number beyond which blocks only queue
+  int blocks(int i) const {
+    long n = w[i], most = 8L * sms;
+    switch (i) {
+      case NODES: break;
+      case SUPERS: n = (n + 1) / 2, most = sms; break;
+      case NNF:
+      case NNR: n = (n * nn_sub() + 3) / 4, most = 32L * sms; break;
+      case POINTS:
+      case EDGES: n = (n + 255) / 256; break;
+      case LOSS: most = 2L * sms; break;
+      case JOBS: most = MAXJ; break;
+      case ROWS: break;
+      case ADJ: most = 16L * sms; break;
+      case PLANES: most = (long)sms * plane_blocks_per_sm(); break;
+      case COLS: most = 3L * sms * plane_blocks_per_sm(); break;
+      case ADAM: n = (n + 255) / 256, most = 8L * sms * plane_blocks_per_sm(); break;
+      case XT: most = 12L * sms; break;
+      case YZ: most = 16L * sms; break;
+    }
+    return (int)std::max(1L, std::min(n, most));
   }
 };
 
@@ -145,17 +186,23 @@ bool is_device_ptr(const void* p) {
   return a.type == cudaMemoryTypeDevice || a.type == cudaMemoryTypeManaged;
 }
 
-// the streams of a step's capture
+// The side streams of a step (and the main one of its capture) and the events that tie them to the
+// main stream.
 struct Streams {
   cudaStream_t s[3] = {};
+  cudaEvent_t ev[7] = {};
   bool create() {
     for (auto& x : s)
       if (cudaStreamCreateWithFlags(&x, cudaStreamNonBlocking) != cudaSuccess) return false;
+    for (auto& x : ev)
+      if (cudaEventCreateWithFlags(&x, cudaEventDisableTiming) != cudaSuccess) return false;
     return true;
   }
   void destroy() {
     for (auto& x : s)
       if (x) cudaStreamDestroy(x);
+    for (auto& x : ev)
+      if (x) cudaEventDestroy(x);
   }
 };
 
@@ -408,84 +455,81 @@ enum StageIndex {
 // step, 2: evaluation); count: the nearest-neighbour instances that count candidates and
 // exact ties.  The plan's item prefixes must be current (refresh_plan).
 void launch_stage(int i, const Plan* plan, const Shape& sh, cudaStream_t s, int bump = 1, bool count = false) {
-  const int sms = sh.sms;
-  const int grid = sms * 8;
+  const bool planes = sh.w[Shape::PLANES] > 0;
   switch (i) {
-    case S_INTERP: launch_interp(plan, sh.nodes, s, bump); break;
-    case S_BOXES: launch_boxes(plan, sh.supers, s); break;
-    case S_NN: launch_nn(plan, sh.nn_grid(sh.nnf), s, -1, sh.nn_sub(), count); break;
-    case S_NN_REV0: launch_nn(plan, sh.nn_grid(sh.nnr), s, 0, sh.nn_sub(), count); break;
-    case S_NN_REV1: launch_nn(plan, sh.nn_grid(sh.nnr), s, 1, sh.nn_sub(), count); break;
-    case S_ISO: launch_iso_edges(plan, grid, s); break;
-    case S_ASSEMBLE: launch_assemble(plan, grid, s); break;
-    case S_ADJOINT_ROWS: launch_adjoint_rows(plan, grid, s); break;
-    case S_ADJOINT: launch_adjoint(plan, grid * 2, s); break;
+    case S_INTERP: launch_interp(plan, sh.blocks(Shape::NODES), s, bump); break;
+    case S_BOXES: launch_boxes(plan, sh.blocks(Shape::SUPERS), s); break;
+    case S_NN: launch_nn(plan, sh.blocks(Shape::NNF), s, -1, sh.nn_sub(), count); break;
+    case S_NN_REV0: launch_nn(plan, sh.blocks(Shape::NNR), s, 0, sh.nn_sub(), count); break;
+    case S_NN_REV1: launch_nn(plan, sh.blocks(Shape::NNR), s, 1, sh.nn_sub(), count); break;
+    case S_ISO: launch_iso_edges(plan, sh.blocks(Shape::EDGES), s); break;
+    case S_ASSEMBLE: launch_assemble(plan, sh.blocks(Shape::POINTS), s); break;
+    case S_ADJOINT_ROWS: launch_adjoint_rows(plan, sh.blocks(Shape::ROWS), s); break;
+    case S_ADJOINT: launch_adjoint(plan, sh.blocks(Shape::ADJ), s); break;
     case S_SOB_XY_FWD:
-    case S_SOB_Z:
     case S_SOB_XY_INV:
-    case S_ADAM: {
-      const int ps = plane_smem_max(sh.nmax);
-      const int per_sm = std::max(1, std::min(8, (227 * 1024) / ps));
-      launch_sobolev_plane(plan, sms * per_sm, sh.nmax, s, i - S_SOB_XY_FWD, sh.ext);
+      if (planes) launch_sobolev_plane(plan, sh.blocks(Shape::PLANES), sh.nmax, s, i - S_SOB_XY_FWD, sh.ext);
       break;
-    }
+    case S_SOB_Z:
+      if (planes) launch_sobolev_plane(plan, sh.blocks(Shape::COLS), sh.nmax, s, i - S_SOB_XY_FWD, sh.ext);
+      break;
+    case S_ADAM:
+      if (planes) launch_sobolev_plane(plan, sh.blocks(Shape::ADAM), sh.nmax, s, i - S_SOB_XY_FWD, sh.ext);
+      break;
     case S_SOB_256:
       if (sh.nline == 0) break;
-      launch_sobolev_x(plan, sms, sh.nline, true, s);
-      for (int p = YZ_FWD; p <= YZ_INV; ++p) launch_sobolev_yz(plan, sms, sh.nline, p, s);
-      launch_sobolev_x(plan, sms, sh.nline, false, s);
+      launch_sobolev_x(plan, sh.blocks(Shape::XT), sh.nline, true, s);
+      for (int p = YZ_FWD; p <= YZ_INV; ++p) launch_sobolev_yz(plan, sh.blocks(Shape::YZ), sh.nline, p, s);
+      launch_sobolev_x(plan, sh.blocks(Shape::XT), sh.nline, false, s);
       break;
-    case S_LOSS: launch_loss(plan, sms * 2, s); break;
+    case S_LOSS: launch_loss(plan, sh.blocks(Shape::LOSS), sh.blocks(Shape::JOBS), s); break;
   }
 }
-constexpr int ST_SOB_FIRST = S_SOB_XY_FWD, ST_SOB_LAST = S_SOB_256;  // preconditioner and Adam stages
 
-// Captures one step.  Branches: the searches of the moving points (in the target tree, which needs
-// no boxes of this step) and the isometry beside the moving trees' upper boxes and the targets'
-// searches, one per moving set; the two adjoint kernels beside each other; the loss reduction beside
-// the adjoint and the preconditioner (nothing downstream reads it).
+// One step on `main` (launched, or captured into a graph), or with eval only the loss and its
+// gradients.  Branches: the searches of the moving points (in the target tree, which needs no boxes
+// of this step) and the isometry beside the moving trees' upper boxes and the targets' searches, one
+// per moving set; the two adjoint kernels beside each other; the loss reduction beside the adjoint
+// and the preconditioner (nothing downstream reads it).  All of it ends on `main`.
+void launch_step(const Plan* plan, const Shape& sh, const Streams& st, cudaStream_t main, bool count, bool eval) {
+  const cudaStream_t side = st.s[1], side2 = st.s[2];
+  int n_ev = 0;
+  auto after = [&](cudaStream_t to, cudaStream_t from) {  // `to` goes on after what `from` holds now
+    cudaEventRecord(st.ev[n_ev], from);
+    cudaStreamWaitEvent(to, st.ev[n_ev++], 0);
+  };
+  launch_stage(S_INTERP, plan, sh, main, eval ? 2 : 1);  // starts the step of every job
+  after(side, main);
+  launch_stage(S_BOXES, plan, sh, side);
+  after(side2, side);
+  launch_stage(S_NN_REV0, plan, sh, side, 1, count);
+  launch_stage(S_NN_REV1, plan, sh, side2, 1, count);
+  launch_stage(S_NN, plan, sh, main, 1, count);
+  launch_stage(S_ISO, plan, sh, main);
+  after(main, side);
+  after(main, side2);
+  launch_stage(S_ASSEMBLE, plan, sh, main);
+  after(side, main);
+  launch_stage(S_ADJOINT_ROWS, plan, sh, side);
+  launch_stage(S_ADJOINT, plan, sh, main);
+  after(main, side);
+  launch_stage(S_LOSS, plan, sh, side);
+  if (!eval)
+    for (int i = S_SOB_XY_FWD; i <= S_SOB_256; ++i) launch_stage(i, plan, sh, main);  // preconditioner, Adam
+  after(main, side);
+}
+
 pdg_status capture_step(pdg_ctx* c, const Plan* plan, const Shape& sh, const Streams& st, cudaGraphExec_t* out,
                         std::string* err, int* n_kernels = nullptr) {
-  const cudaStream_t cap = st.s[0], cap2 = st.s[1], cap3 = st.s[2];
+  const cudaStream_t cap = st.s[0];
   cudaGraph_t g = nullptr;
-  cudaEvent_t ev[7] = {};
-  for (auto& e : ev)
-    if (cudaEventCreateWithFlags(&e, cudaEventDisableTiming) != cudaSuccess) {
-      *err = "cudaEventCreate failed";
-      return PDG_ERR_CUDA;
-    }
   cudaError_t e = cudaStreamBeginCapture(cap, cudaStreamCaptureModeThreadLocal);
   if (e != cudaSuccess) {
     *err = std::string("cudaStreamBeginCapture: ") + cudaGetErrorString(e);
-    for (auto& x : ev) cudaEventDestroy(x);
     return PDG_ERR_CUDA;
   }
-  const bool count = c && c->h.count_nn;  // a batch graph never counts
-  int n_ev = 0;
-  auto after = [&](cudaStream_t to, cudaStream_t from) {  // `to` goes on after what `from` holds now
-    cudaEventRecord(ev[n_ev], from);
-    cudaStreamWaitEvent(to, ev[n_ev++], 0);
-  };
-  launch_stage(S_INTERP, plan, sh, cap);  // starts the step of every job
-  after(cap2, cap);
-  launch_stage(S_BOXES, plan, sh, cap2);
-  after(cap3, cap2);
-  launch_stage(S_NN_REV0, plan, sh, cap2, 1, count);
-  launch_stage(S_NN_REV1, plan, sh, cap3, 1, count);
-  launch_stage(S_NN, plan, sh, cap, 1, count);
-  launch_stage(S_ISO, plan, sh, cap);
-  after(cap, cap2);
-  after(cap, cap3);
-  launch_stage(S_ASSEMBLE, plan, sh, cap);
-  after(cap2, cap);
-  launch_stage(S_ADJOINT_ROWS, plan, sh, cap2);
-  launch_stage(S_ADJOINT, plan, sh, cap);
-  after(cap, cap2);
-  launch_stage(S_LOSS, plan, sh, cap2);
-  for (int i = S_SOB_XY_FWD; i <= S_SOB_256; ++i) launch_stage(i, plan, sh, cap);  // preconditioner, Adam
-  after(cap, cap2);
+  launch_step(plan, sh, st, cap, c && c->h.count_nn, false);  // a batch graph never counts
   e = cudaStreamEndCapture(cap, &g);
-  for (auto& x : ev) cudaEventDestroy(x);
   if (e != cudaSuccess) {
     *err = std::string("cudaStreamEndCapture: ") + cudaGetErrorString(e);
     if (g) cudaGraphDestroy(g);
@@ -598,7 +642,7 @@ pdg_status pdg_create(const pdg_config* cfg, const float* template_xyz, int n_ve
   if (cudaGetDevice(&c->dev) != cudaSuccess) return bail(PDG_ERR_CUDA);
   cudaDeviceGetAttribute(&c->sms, cudaDevAttrMultiProcessorCount, c->dev);
   c->shape.sms = c->sms;
-  c->shape.add_points(n_verts, max_pts, max_pts);
+  c->shape.add_points(n_verts, max_pts, max_pts, n_edges);
   sobolev_x_configure();
   sobolev_yz_configure();
   sobolev_plane_configure();
@@ -716,7 +760,7 @@ pdg_status pdg_create(const pdg_config* cfg, const float* template_xyz, int n_ve
     lv.ent = (int2*)P(o.ent);
     lv.n_active = (int*)P(o.n_active);
     lv.csum = (int*)P(o.csum);
-    c->shape.add_level(n);
+    c->shape.add_level(n, J.C, c->Qmax);
     mu.resize(n);
     tw.resize(n);
     tw4.resize(n);
@@ -1102,9 +1146,7 @@ pdg_status pdg_write_theta(pdg_ctx* c, int level, const float* theta, void* cuda
     CU(c, cudaMemcpyAsync(tmp, theta, bytes, cudaMemcpyHostToDevice, s));
     src = tmp;
   }
-  launch_pack_theta(src, lv.theta, lv.theta_t, lv.n3, C, s);
-  CU(c, cudaMemsetAsync(lv.m, 0, C * sizeof(float) * lv.n3, s));
-  CU(c, cudaMemsetAsync(lv.v, 0, C * sizeof(float) * lv.n3, s));
+  launch_pack_theta(src, lv.theta, lv.theta_t, lv.m, lv.v, lv.n3, C, s);
   if (tmp) {
     CU(c, cudaFreeAsync(tmp, s));
     CU(c, cudaStreamSynchronize(s));
@@ -1117,8 +1159,7 @@ pdg_status pdg_eval(pdg_ctx* c, double* loss, void* cuda_stream) {
   if (!c->in_frame) return c->fail(PDG_ERR_STATE, "pdg_eval outside a frame");
   cudaStream_t s = (cudaStream_t)cuda_stream;
   TRY(refresh_plan(c, s));
-  for (int i = 0; i < N_STAGES; ++i)  // no preconditioner, no Adam, no step count
-    if (i < ST_SOB_FIRST || i > ST_SOB_LAST) launch_stage(i, c->dplan, c->shape, s, 2, c->h.count_nn != 0);
+  launch_step(c->dplan, c->shape, c->cap, s, c->h.count_nn != 0, true);  // no preconditioner, no Adam, no step count
   CU(c, cudaGetLastError());
   if (loss) {
     CU(c, cudaMemcpyAsync(loss, c->h.loss, 4 * sizeof(double), cudaMemcpyDeviceToHost, s));
@@ -1156,7 +1197,7 @@ pdg_status pdg_precondition(pdg_ctx* c, int level, const float* g, float* out, v
   launch_op_plan(oj, c->op_job, c->op_plan, s);
   Shape sh;
   sh.sms = c->sms;
-  sh.add_level(lv.n);
+  sh.add_level(lv.n, 3, 0);
   sh.ext = true;
   if (line) launch_stage(S_SOB_256, c->op_plan, sh, s);
   else
@@ -1246,7 +1287,7 @@ pdg_status pdg_fit_mesh(pdg_ctx* c, const float* p0_xyz, int n_p0, int n_steps, 
   CU(c, cudaMemcpyAsync(c->coef, coef.data(), sizeof(float2) * coef.size(), cudaMemcpyHostToDevice, s));
   Shape sh;
   sh.sms = c->sms;
-  sh.add_points(V, 0, n_p0);
+  sh.add_points(V, 0, n_p0, 0);
   for (int k = 1; k <= n_steps; ++k) {
     launch_mesh_points(c->op_job, V, s);
     for (int i = S_BOXES; i <= S_NN_REV0; ++i) launch_stage(i, c->op_plan, sh, s);
@@ -1360,7 +1401,7 @@ pdg_status pdg_batch_step(pdg_batch* b, int n_steps, void* cuda_stream) {
     for (size_t i = 0; i < b->members.size(); ++i) b->gens[i] = b->members[i]->frame_gen;
   }
   Shape need = b->graph_shape;
-  if (need.grow(sh) || !b->gexec) {
+  if (need.cover(sh) || !b->gexec) {
     if (b->gexec) cudaGraphExecDestroy(b->gexec);
     b->gexec = nullptr;
     if (cudaStreamSynchronize(s) != cudaSuccess) return PDG_ERR_CUDA;
