@@ -12,102 +12,88 @@
 
 namespace pdg {
 
-// corners of point p in level lv: flat vertex ids and trilinear weights (Eq. 1)
-__device__ __forceinline__ int corners(const Job& J, const Level& lv, float px, float py, float pz, int vid[8],
-                                       float w[8]) {
+// A point's cell in a level (Eq. 1): its first corner and the fractional coordinates
+__device__ __forceinline__ int level_cell(const Job& J, const Level& lv, const float4& x, float& fx, float& fy,
+                                          float& fz) {
   const int n = lv.n;
-  if (n == 1) {
-    vid[0] = 0;
-    w[0] = 1.f;
-    return 1;
-  }
+  fx = fy = fz = 0.f;
+  if (n == 1) return 0;
   int ix, iy, iz;
-  float fx, fy, fz;
-  grid_coord(px, J.lo[0], lv.sc_hi[0], lv.sc_lo[0], n, ix, fx);
-  grid_coord(py, J.lo[1], lv.sc_hi[1], lv.sc_lo[1], n, iy, fy);
-  grid_coord(pz, J.lo[2], lv.sc_hi[2], lv.sc_lo[2], n, iz, fz);
-  const int b = (iz * n + iy) * n + ix;
-#pragma unroll
-  for (int c = 0; c < 8; ++c) {
-    const int dx = c & 1, dy = (c >> 1) & 1, dz = c >> 2;
-    vid[c] = b + dx + dy * n + dz * n * n;
-    w[c] = (dx ? fx : 1.f - fx) * (dy ? fy : 1.f - fy) * (dz ? fz : 1.f - fz);
-  }
-  return 8;
+  grid_coord(x.x, J.lo[0], lv.sc_hi[0], lv.sc_lo[0], n, ix, fx);
+  grid_coord(x.y, J.lo[1], lv.sc_hi[1], lv.sc_lo[1], n, iy, fy);
+  grid_coord(x.z, J.lo[2], lv.sc_hi[2], lv.sc_lo[2], n, iz, fz);
+  return (iz * n + iy) * n + ix;
 }
 
-__global__ void k_csr_count(Job* __restrict__ Jp) {
+__device__ __forceinline__ int corner_offset(int c, int n) { return (c & 1) + ((c >> 1) & 1) * n + (c >> 2) * n * n; }
+
+// Lanes of the warp whose points share a cell: the group's leader does one atomic per corner for all
+// of them.  Points come in slot order, so on coarse levels a whole warp is often one group; with an
+// atomic per point and corner, the rows of a 16^3 level took hundreds of them one after another.
+struct CellGroup {
+  int leader, rank, size;
+};
+__device__ __forceinline__ CellGroup cell_group(int cell) {
+  const unsigned m = __match_any_sync(0xffffffffu, cell);
+  const int lane = threadIdx.x & 31;
+  return CellGroup{__ffs(m) - 1, __popc(m & ((1u << lane) - 1u)), __popc(m)};
+}
+
+// entry counts of every level's vertices (and cleared z-plane marks); slots: a multiple of 32
+__global__ void __launch_bounds__(256) k_csr_count(Job* __restrict__ Jp, int slots) {
   const Job& J = *Jp;
-  for (int p = blockIdx.x * blockDim.x + threadIdx.x; p < J.Q; p += gridDim.x * blockDim.x) {
-    const float4 x = J.x[p];
+  const int i0 = blockIdx.x * blockDim.x + threadIdx.x, step = gridDim.x * blockDim.x;
+  for (int l = 0; l < J.L; ++l)
+    for (int z = i0; z < J.lev[l].n; z += step) J.lev[l].zmask[z] = 0;
+  for (int i = i0; i < slots; i += step) {  // warp-uniform
+    const float4 x = J.xs[i];
+    const bool in = __float_as_int(x.w) >= 0;
     for (int l = 0; l < J.L; ++l) {
-      int vid[8];
-      float w[8];
-      const int K = corners(J, J.lev[l], x.x, x.y, x.z, vid, w);
-      for (int c = 0; c < K; ++c) atomicAdd(&J.lev[l].cnt[vid[c]], 1);
+      const Level& lv = J.lev[l];
+      float fx, fy, fz;
+      const int cell = level_cell(J, lv, x, fx, fy, fz);
+      const CellGroup g = cell_group(in ? cell : -1);
+      if (!in || g.rank) continue;
+      for (int c = 0; c < (lv.n == 1 ? 1 : 8); ++c) atomicAdd(&lv.cnt[cell + corner_offset(c, lv.n)], g.size);
     }
   }
 }
 
-__global__ void k_csr_fill(Job* __restrict__ Jp) {
+__global__ void __launch_bounds__(256) k_csr_fill(Job* __restrict__ Jp, int slots) {
   const Job& J = *Jp;
   const float invL = 1.f / (float)J.L;
-  for (int p = blockIdx.x * blockDim.x + threadIdx.x; p < J.Q; p += gridDim.x * blockDim.x) {
-    const float4 x = J.x[p];
+  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < slots; i += gridDim.x * blockDim.x) {  // warp-uniform
+    const float4 x = J.xs[i];
+    const int p = __float_as_int(x.w);
     for (int l = 0; l < J.L; ++l) {
       const Level& lv = J.lev[l];
-      int vid[8];
-      float w[8];
-      const int K = corners(J, lv, x.x, x.y, x.z, vid, w);
-      for (int c = 0; c < K; ++c) {
-        const int pos = lv.rowptr[vid[c]] + atomicSub(&lv.cnt[vid[c]], 1) - 1;
-        lv.ent[pos] = make_int2(p, __float_as_int(w[c] * invL));
+      float fx, fy, fz;
+      const int cell = level_cell(J, lv, x, fx, fy, fz);
+      const CellGroup g = cell_group(p >= 0 ? cell : -1);
+      const int K = lv.n == 1 ? 1 : 8;
+      int first[8];
+#pragma unroll
+      for (int c = 0; c < 8; ++c) {  // the group's range in each row (counts return to zero)
+        const int v = cell + corner_offset(c, lv.n);
+        first[c] = c < K && p >= 0 && g.rank == 0 ? lv.rowptr[v] + atomicSub(&lv.cnt[v], g.size) - g.size : 0;
+      }
+#pragma unroll
+      for (int c = 0; c < 8; ++c) {
+        const int pos = __shfl_sync(0xffffffffu, first[c], g.leader) + g.rank;
+        const float w = (c & 1 ? fx : 1.f - fx) * ((c >> 1) & 1 ? fy : 1.f - fy) * (c >> 2 ? fz : 1.f - fz);
+        if (c < K && p >= 0) lv.ent[pos] = make_int2(p, __float_as_int(w * invL));
       }
     }
   }
 }
 
-__global__ void k_csr_flags(Job* __restrict__ Jp, int l) {
-  const Level& lv = Jp->lev[l];
-  for (int v = blockIdx.x * blockDim.x + threadIdx.x; v < lv.n3; v += gridDim.x * blockDim.x)
-    lv.flag[v] = lv.rowptr[v + 1] > lv.rowptr[v] ? 1 : 0;
-}
-
-__global__ void k_csr_compact(Job* __restrict__ Jp, int l) {
-  const Level& lv = Jp->lev[l];
-  for (int v = blockIdx.x * blockDim.x + threadIdx.x; v < lv.n3; v += gridDim.x * blockDim.x) {
-    if (lv.rowptr[v + 1] > lv.rowptr[v]) {
-      const int i = lv.flag[v];
-      lv.act_v[i] = v;
-      lv.act_ptr[i] = lv.rowptr[v];
-    }
-    if (v == 0) {
-      const int na = lv.flag[lv.n3];
-      *lv.n_active = na;
-      lv.act_ptr[na] = lv.rowptr[lv.n3];
-    }
-  }
-}
-
-
+// after launch_tree_build (the points' slot order)
 void launch_csr_build(Job* J, const Job& hJ, cudaStream_t s) {
-  const int grid = max(1, min((hJ.Q + 255) / 256, 4096));
-  k_csr_count<<<grid, 256, 0, s>>>(J);
-  for (int l = 0; l < hJ.L; ++l) {
-    const Level& lv = hJ.lev[l];
-    ScanSeg seg{lv.cnt, lv.rowptr, lv.n3, lv.csum};
-    launch_scan_segments(&seg, 1, nullptr, nullptr, s);
-  }
-  k_csr_fill<<<grid, 256, 0, s>>>(J);
-  for (int l = 0; l < hJ.L; ++l) {
-    const Level& lv = hJ.lev[l];
-    const int g2 = max(1, min((lv.n3 + 255) / 256, 4096));
-    k_csr_flags<<<g2, 256, 0, s>>>(J, l);
-    ScanSeg seg{lv.flag, lv.flag, lv.n3, lv.csum};
-    launch_scan_segments(&seg, 1, nullptr, nullptr, s);
-    k_csr_compact<<<g2, 256, 0, s>>>(J, l);
-  }
-  launch_zmask(J, hJ, s);
+  const int slots = ((hJ.V + NODE - 1) / NODE + (hJ.N + NODE - 1) / NODE) * NODE;
+  const int grid = min(slots / 256, 4096);
+  k_csr_count<<<grid, 256, 0, s>>>(J, slots);
+  launch_csr_scan(J, hJ, s);
+  k_csr_fill<<<grid, 256, 0, s>>>(J, slots);
 }
 
 // ------------------------------------------------------------------------------ per step

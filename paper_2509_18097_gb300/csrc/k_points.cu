@@ -97,12 +97,12 @@ __global__ void k_plan(Plan* P) {
   }
 }
 
-// the job record (by value, in the launch's arguments) and the plan that holds it alone
+// the job record (by value, in the launch's arguments) and, if given, the plan that holds it alone
 __global__ void k_op_job(const __grid_constant__ Job job, Job* dJ, Plan* dP) {
   const unsigned* src = reinterpret_cast<const unsigned*>(&job);
   unsigned* dst = reinterpret_cast<unsigned*>(dJ);
   for (int i = threadIdx.x; i < (int)(sizeof(Job) / 4); i += blockDim.x) dst[i] = src[i];
-  if (threadIdx.x == 0) {
+  if (dP && threadIdx.x == 0) {
     dP->n_jobs = 1;
     dP->jobs[0] = dJ;
   }
@@ -444,20 +444,43 @@ __global__ void k_frame_points(Job* J) {
   }
 }
 
-// Tree builds (per frame): cell keys and counts, scatter of the indices into slot order
-__global__ void k_tgt_keys(Job* J) {
-  for (int p = blockIdx.x * blockDim.x + threadIdx.x; p < J->M; p += gridDim.x * blockDim.x) {
-    const float4 t = J->tgt4[p];
-    const int key = cell_key(J->tgt, t.x, t.y, t.z, 0);
-    J->tgt.keys[p] = key;
-    atomicAdd(&J->tgt.hist[key], 1);
+// Tree builds (per frame), both trees in each launch: cell keys and counts, scatter of the indices into
+// slot order.  i < M: target i; else moving point i - M.
+__global__ void k_tree_keys(Job* J) {
+  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < J->M + J->Q; i += gridDim.x * blockDim.x) {
+    const bool t = i < J->M;
+    const int p = t ? i : i - J->M;
+    const float4 x = t ? J->tgt4[p] : J->x[p];
+    const Tree& T = t ? J->tgt : J->mov;
+    const int key = cell_key(T, x.x, x.y, x.z, t || p < J->V ? 0 : 1);
+    T.keys[p] = key;
+    atomicAdd(&T.hist[key], 1);
   }
 }
 
-__global__ void k_tgt_scatter(Job* J) {
-  for (int p = blockIdx.x * blockDim.x + threadIdx.x; p < J->M; p += gridDim.x * blockDim.x) {
-    const int key = J->tgt.keys[p];
-    J->tgt.perm[J->tgt.off[key] + atomicSub(&J->tgt.hist[key], 1) - 1] = p;
+__global__ void k_tree_scatter(Job* J) {
+  const SetRange r0 = mov_set(*J, 0), r1 = mov_set(*J, 1);
+  const int pad0 = r0.nodes * NODE - r0.n, pad1 = r1.nodes * NODE - r1.n;
+  const int M = J->M, Q = J->Q;
+  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < M + Q + pad0 + pad1; i += gridDim.x * blockDim.x) {
+    if (i < M + Q) {
+      const bool t = i < M;
+      const int p = t ? i : i - M;
+      const Tree& T = t ? J->tgt : J->mov;
+      const int key = T.keys[p];
+      const int pos = T.off[key] + atomicSub(&T.hist[key], 1) - 1;
+      const int slot = t || p < J->V ? pos : r1.slot0 + pos - J->V;
+      T.perm[slot] = p;
+      if (!t) {
+        const float4 x = J->x[p];
+        J->xs[slot] = make_float4(x.x, x.y, x.z, __int_as_float(p));
+      }
+    } else {  // padding of the moving sets' last nodes
+      const int k = i - M - Q;
+      const int slot = k < pad0 ? r0.n + k : r1.slot0 + r1.n + k - pad0;
+      J->xs[slot] = make_float4(0.f, 0.f, 0.f, __int_as_float(-1));
+      J->mov.perm[slot] = -1;
+    }
   }
 }
 
@@ -476,34 +499,6 @@ __global__ void __launch_bounds__(NODE) k_tgt_nodes(Job* J) {
 __global__ void __launch_bounds__(32) k_tgt_boxes(Job* J) {
   const SetRange r = set_range(0, 0, J->M);
   for (int s = blockIdx.x; s < r.supers; s += gridDim.x) super_box(J->tgt, r, s);
-}
-
-__global__ void k_mov_keys(Job* J) {
-  for (int p = blockIdx.x * blockDim.x + threadIdx.x; p < J->Q; p += gridDim.x * blockDim.x) {
-    const float4 x = J->x[p];
-    const int key = cell_key(J->mov, x.x, x.y, x.z, p < J->V ? 0 : 1);
-    J->mov.keys[p] = key;
-    atomicAdd(&J->mov.hist[key], 1);
-  }
-}
-
-__global__ void k_mov_scatter(Job* J) {
-  const SetRange r0 = mov_set(*J, 0), r1 = mov_set(*J, 1);
-  const int i0 = blockIdx.x * blockDim.x + threadIdx.x, step = gridDim.x * blockDim.x;
-  for (int p = i0; p < J->Q; p += step) {
-    const int key = J->mov.keys[p];
-    const int pos = J->mov.off[key] + atomicSub(&J->mov.hist[key], 1) - 1;
-    const int slot = p < J->V ? pos : r1.slot0 + pos - J->V;
-    const float4 x = J->x[p];
-    J->xs[slot] = make_float4(x.x, x.y, x.z, __int_as_float(p));
-    J->mov.perm[slot] = p;
-  }
-  const int pad0 = r0.nodes * NODE - r0.n, pad1 = r1.nodes * NODE - r1.n;
-  for (int i = i0; i < pad0 + pad1; i += step) {
-    const int slot = i < pad0 ? r0.n + i : r1.slot0 + r1.n + i - pad0;
-    J->xs[slot] = make_float4(0.f, 0.f, 0.f, __int_as_float(-1));
-    J->mov.perm[slot] = -1;
-  }
 }
 
 // frame end: X_t = M(T_t(X_{t-1})) X_{t-1} with the final grids (Sec. 3.3)
@@ -532,8 +527,11 @@ __global__ void k_deform(const Job* __restrict__ J, const float* __restrict__ in
 static inline int blocks_for(int n, int threads) { return max(1, min((n + threads - 1) / threads, 4096)); }
 
 void launch_plan(Plan* P, cudaStream_t s) { k_plan<<<1, 256, 0, s>>>(P); }
-void launch_op_plan(const Job& job, Job* dJ, Plan* dP, cudaStream_t s) {
+void launch_job(const Job& job, Job* dJ, cudaStream_t s) {
   static_assert(sizeof(Job) % 4 == 0, "copied word by word");
+  k_op_job<<<1, 256, 0, s>>>(job, dJ, nullptr);
+}
+void launch_op_plan(const Job& job, Job* dJ, Plan* dP, cudaStream_t s) {
   k_op_job<<<1, 256, 0, s>>>(job, dJ, dP);
   launch_plan(dP, s);
 }
@@ -617,23 +615,17 @@ void launch_copy_int(const int* in, int* out, int n, cudaStream_t s) {
   k_copy_int<<<blocks_for(n, 256), 256, 0, s>>>(in, out, n);
 }
 
-// target tree of the frame: keys + counts, exclusive scan, scatter, boxes
-void launch_tgt_build(Job* J, const Job& hJ, cudaStream_t s) {
-  k_tgt_keys<<<blocks_for(hJ.M, 256), 256, 0, s>>>(J);
-  ScanSeg seg{hJ.tgt.hist, hJ.tgt.off, 1 << (3 * hJ.tgt.bits), hJ.tgt.csum};
-  launch_scan_segments(&seg, 1, nullptr, nullptr, s);
-  k_tgt_scatter<<<blocks_for(hJ.M, 256), 256, 0, s>>>(J);
+// both trees of the frame: keys + counts, exclusive scans, scatter; the targets' points and boxes (the
+// moving points' come with the interpolation)
+void launch_tree_build(Job* J, const Job& hJ, cudaStream_t s) {
+  const int n = hJ.M + hJ.Q;
+  k_tree_keys<<<blocks_for(n, 256), 256, 0, s>>>(J);
+  launch_scan(ScanSeg{hJ.tgt.hist, hJ.tgt.off, 1 << (3 * hJ.tgt.bits), hJ.tgt.csum},
+              ScanSeg{hJ.mov.hist, hJ.mov.off, 2 << (3 * hJ.mov.bits), hJ.mov.csum}, s);
+  k_tree_scatter<<<blocks_for(n + 2 * NODE, 256), 256, 0, s>>>(J);
   const SetRange r = set_range(0, 0, hJ.M);
   k_tgt_nodes<<<min(r.nodes, 4096), NODE, 0, s>>>(J);
   k_tgt_boxes<<<min(r.supers, 4096), 32, 0, s>>>(J);
-}
-
-// slot order of the moving sets for the frame (from x)
-void launch_mov_build(Job* J, const Job& hJ, cudaStream_t s) {
-  k_mov_keys<<<blocks_for(hJ.Q, 256), 256, 0, s>>>(J);
-  ScanSeg seg{hJ.mov.hist, hJ.mov.off, 2 << (3 * hJ.mov.bits), hJ.mov.csum};
-  launch_scan_segments(&seg, 1, nullptr, nullptr, s);
-  k_mov_scatter<<<blocks_for(hJ.Q, 256), 256, 0, s>>>(J);
 }
 
 }  // namespace pdg

@@ -747,27 +747,6 @@ __global__ void __launch_bounds__(256) k_adam(const Plan* __restrict__ P) {
   }
 }
 
-// ------------------------------------------------------------------------------ per frame
-
-// zmask[z] = 1 for the z-planes of a level that hold an active vertex (per frame)
-__global__ void k_zmask(Job* __restrict__ Jp, int l) {
-  const Level& lv = Jp->lev[l];
-  const int na = *lv.n_active;
-  const int n2 = lv.n * lv.n;
-  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < na; i += gridDim.x * blockDim.x)
-    lv.zmask[lv.act_v[i] / n2] = 1;
-}
-
-void launch_zmask(Job* J, const Job& hJ, cudaStream_t s) {
-  for (int l = 0; l < hJ.L; ++l) {
-    const Level& lv = hJ.lev[l];
-    if (!lv.zmask) continue;
-    cudaMemsetAsync(lv.zmask, 0, sizeof(int) * lv.n, s);
-    const int grid = lv.n3 / 256 + 1 < 1024 ? lv.n3 / 256 + 1 : 1024;
-    k_zmask<<<grid, 256, 0, s>>>(J, l);
-  }
-}
-
 // largest shared memory a plane pass needs over the levels n <= nmax it may meet
 int plane_smem_max(int nmax) {
   int m = 0;

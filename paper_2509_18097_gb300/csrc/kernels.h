@@ -9,7 +9,9 @@ namespace pdg {
 
 // per step (plan-driven; `grid` = blocks of the persistent launch)
 void launch_plan(Plan* P, cudaStream_t s);
-// a record and a plan for one job, from the launch's arguments (nothing is copied from host memory)
+// a job's record, and with it a plan for it alone, from the launch's arguments (nothing is copied from
+// host memory)
+void launch_job(const Job& job, Job* dJ, cudaStream_t s);
 void launch_op_plan(const Job& job, Job* dJ, Plan* dP, cudaStream_t s);
 void launch_interp(const Plan* P, int grid, cudaStream_t s, int bump);
 void launch_boxes(const Plan* P, int grid, cudaStream_t s);
@@ -32,22 +34,21 @@ void launch_pack4(const float* in, float4* out, int n, cudaStream_t s);
 void launch_unpack4(const float4* in, float* out, int n, cudaStream_t s);
 void launch_check_finite(const float* in, int n, int* flag, cudaStream_t s);
 void launch_frame_points(Job* J, int Q, int E, cudaStream_t s);
-void launch_tgt_build(Job* J, const Job& hJ, cudaStream_t s);
-void launch_mov_build(Job* J, const Job& hJ, cudaStream_t s);
+void launch_tree_build(Job* J, const Job& hJ, cudaStream_t s);
 void launch_nn_seed(Job* J, const Job& hJ, cudaStream_t s);
 void launch_csr_build(Job* J, const Job& hJ, cudaStream_t s);
 void launch_end_frame(Job* J, int V, cudaStream_t s);
 void launch_deform(const Job* J, const float* in, float* out, int n, cudaStream_t s);
 
-// generic exclusive scans over explicit segments (per-frame structures)
+// exclusive scans of two arrays
 struct ScanSeg {
   const int* in;
   int* out;   // [len + 1]
   int len;
   int* csum;  // [ceil(len / SCAN_CHUNK)]
 };
-void launch_scan_segments(const ScanSeg* hsegs, int nseg, ScanSeg* dsegs_scratch, int* dpre_scratch,
-                          cudaStream_t s);
+void launch_scan(const ScanSeg& a, const ScanSeg& b, cudaStream_t s);
+void launch_csr_scan(const Job* J, const Job& hJ, cudaStream_t s);
 
 void sobolev_x_configure();
 void sobolev_yz_configure();
@@ -55,7 +56,6 @@ void sobolev_plane_configure();
 int plane_smem_bytes(int n);
 int plane_smem_max(int nmax);
 void launch_aos_to_soa(const float* in, float* out, int n3, cudaStream_t s, int C = 3);
-void launch_zmask(Job* J, const Job& hJ, cudaStream_t s);
 void launch_sobz_pivots(float* piv, int* slow, const float* mu, int n, float lam, cudaStream_t s);
 
 // template-mesh fit (k_mesh.cu)

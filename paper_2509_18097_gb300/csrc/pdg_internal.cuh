@@ -61,12 +61,11 @@ struct Level {
   // point -> vertex interpolation lists, built once per frame (x is fixed in a frame)
   int* cnt;       // [n3] per-vertex entry counts (zero between builds)
   int* rowptr;    // [n3 + 1]
-  int* flag;      // [n3 + 1] active-vertex flags, then their exclusive prefix
   int* act_v;     // [cap] active vertices (ascending)
   int* act_ptr;   // [cap + 1] entry range of each active vertex
   int2* ent;      // [8 Q] entries: (point, bits of the trilinear weight / L)
   int* n_active;  // device scalar
-  int* csum;      // scan scratch
+  unsigned long long* csum;  // scan scratch
   int adj_lg;     // adjoint: log2 of the lanes per row, 6 = a block per row (set by the plan kernel)
 };
 

@@ -283,7 +283,7 @@ struct Layout {
   size_t total = 0;
   size_t job, plan, flag, stage, op_job, op_plan;
   struct Lv {
-    size_t theta, theta_t, m, v, g, tmp, zmask, piv, piv_slow, mu, tw, twm, tw4, cnt, rowptr, flag, act_v, act_ptr, ent, n_active,
+    size_t theta, theta_t, m, v, g, tmp, zmask, piv, piv_slow, mu, tw, twm, tw4, cnt, rowptr, act_v, act_ptr, ent, n_active,
         csum;
     int cap;
   } lv[MAXL];
@@ -329,12 +329,11 @@ Layout make_layout(const pdg_config& c, int V, int E, int max_pts) {
     v.tw4 = a.take<float2>(n);
     v.cnt = a.take<int>(n3);
     v.rowptr = a.take<int>(n3 + 1);
-    v.flag = a.take<int>(n3 + 1);
     v.act_v = a.take<int>(v.cap);
     v.act_ptr = a.take<int>(v.cap + 1);
     v.ent = a.take<int2>(8 * (size_t)Q);
     v.n_active = a.take<int>(1);
-    v.csum = a.take<int>((n3 + 1) / SCAN_CHUNK + 2);
+    v.csum = a.take<unsigned long long>((n3 + 1) / SCAN_CHUNK + 2);
   }
   L.x = a.take<float4>(Q);
   L.y = a.take<float4>(Q);
@@ -434,7 +433,8 @@ pdg_status load_points(pdg_ctx* c, const float* xyz, int n, float4* dst, cudaStr
 // plan kernel writes into the device record (each level's adjoint lanes per row), so the
 // plan of the context, and of any batch holding it, is recomputed before the next step.
 pdg_status upload_job(pdg_ctx* c, cudaStream_t s) {
-  CU(c, cudaMemcpyAsync(c->dJ, &c->h, sizeof(Job), cudaMemcpyHostToDevice, s));
+  launch_job(c->h, c->dJ, s);
+  CU(c, cudaGetLastError());
   c->plan_stale = true;
   ++c->frame_gen;
   return PDG_OK;
@@ -754,12 +754,11 @@ pdg_status pdg_create(const pdg_config* cfg, const float* template_xyz, int n_ve
     lv.tw4 = (float2*)P(o.tw4);
     lv.cnt = (int*)P(o.cnt);
     lv.rowptr = (int*)P(o.rowptr);
-    lv.flag = (int*)P(o.flag);
     lv.act_v = (int*)P(o.act_v);
     lv.act_ptr = (int*)P(o.act_ptr);
     lv.ent = (int2*)P(o.ent);
     lv.n_active = (int*)P(o.n_active);
-    lv.csum = (int*)P(o.csum);
+    lv.csum = (unsigned long long*)P(o.csum);
     c->shape.add_level(n, J.C, c->Qmax);
     mu.resize(n);
     tw.resize(n);
@@ -900,21 +899,15 @@ pdg_status pdg_begin_frame(pdg_ctx* c, const float* target_xyz, int n_tgt, void*
   J.Q = J.V + J.N;
   TRY(upload_job(c, s));
   launch_frame_points(c->dJ, J.Q, J.E, s);
+  // A level's theta, theta_t, m, v and g follow one another in the arena (see make_layout), as do the
+  // step count, bias corrections, losses and status: one clearing each.
   for (int l = 0; l < J.L; ++l) {
     const Level& lv = J.lev[l];
-    if (!c->cfg.warm_start) {
-      CU(c, cudaMemsetAsync(lv.theta, 0, sizeof(float4) * lv.n3, s));
-      if (lv.theta_t) CU(c, cudaMemsetAsync(lv.theta_t, 0, sizeof(float4) * lv.n3, s));
-    }
-    CU(c, cudaMemsetAsync(lv.m, 0, sizeof(float) * J.C * lv.n3, s));
-    CU(c, cudaMemsetAsync(lv.v, 0, sizeof(float) * J.C * lv.n3, s));
-    CU(c, cudaMemsetAsync(lv.g, 0, sizeof(float) * J.C * lv.n3, s));
+    char* from = c->cfg.warm_start ? (char*)lv.m : (char*)lv.theta;
+    CU(c, cudaMemsetAsync(from, 0, (char*)(lv.g + (size_t)J.C * lv.n3) - from, s));
   }
-  CU(c, cudaMemsetAsync(J.step, 0, sizeof(int), s));
-  CU(c, cudaMemsetAsync(J.status, 0, sizeof(int), s));
-  CU(c, cudaMemsetAsync(J.loss, 0, 4 * sizeof(double), s));
-  launch_tgt_build(c->dJ, J, s);
-  launch_mov_build(c->dJ, J, s);
+  CU(c, cudaMemsetAsync(J.step, 0, (char*)(J.status + 1) - (char*)J.step, s));
+  launch_tree_build(c->dJ, J, s);
   launch_nn_seed(c->dJ, J, s);
   launch_csr_build(c->dJ, J, s);
   CU(c, cudaGetLastError());
@@ -1249,8 +1242,7 @@ pdg_status pdg_fit_mesh(pdg_ctx* c, const float* p0_xyz, int n_p0, int n_steps, 
   CU(c, cudaMemsetAsync(am, 0, 2 * sizeof(float4) * (size_t)V, s));
   CU(c, cudaMemsetAsync(J.loss, 0, 4 * sizeof(double), s));
   CU(c, cudaMemsetAsync(J.status, 0, sizeof(int), s));
-  launch_tgt_build(c->op_job, mj, s);
-  launch_mov_build(c->op_job, mj, s);
+  launch_tree_build(c->op_job, mj, s);
   launch_nn_seed(c->op_job, mj, s);
   // Chebyshev interval: the Laplacian's eigenvalues lie in [0, 2 max degree] (Gershgorin), so
   // those of I + lambda L in [1, emax]; iterations for a relative error below 1e-7 in exact
