@@ -266,9 +266,12 @@ __device__ __forceinline__ void dct3_pre(const float2 (&X)[N2], int t, int lbase
 }
 
 // maps a plane item of a job to (level, index); C n items per level (plane major, then
-// channel), only the plane-path levels (powers of two up to 128) take part
+// channel), only the plane-path levels (powers of two up to 128) take part, the finest first: its
+// planes take longest, and with a block per item the short ones fill the SMs that are done.  (Two
+// blocks per SM that loop over the items, coarsest level first: A 34.8, C 61.1 us with the 6-D payload
+// on 16^3..128^3; so: 26.6 and 57.3; with 3 channels C 35.7 and 31.6.)
 __device__ __forceinline__ bool plane_item(const Job& J, int r, int& l, int& idx) {
-  for (l = 0; l < J.L; ++l) {
+  for (l = J.L - 1; l >= 0; --l) {
     const int n = J.lev[l].n;
     if (tile_level(n)) continue;
     if (r < J.C * n) {

@@ -201,15 +201,15 @@ __global__ void __launch_bounds__(X_THREADS, 3) k_sob_x(const Plan* __restrict__
     const Job& J = *P->jobs[j];
     if (FWD && !J.precondition) continue;
     int t = it - P->pre[ST_XTILE][j];
-    int l = 0, per = 0;
-    for (; l < J.L; ++l) {
+    int l = J.L - 1, per = 0;
+    for (; l >= 0; --l) {
       const int n = J.lev[l].n;
       if (!tile_level(n)) continue;
       per = x_tiles(n);
       if (t < J.C / 3 * per) break;
       t -= J.C / 3 * per;
     }
-    if (l >= J.L) continue;
+    if (l < 0) continue;
     const Level& lv = J.lev[l];
     const int h = t / per;
     const int tile = t - h * per;

@@ -150,15 +150,15 @@ __global__ void __launch_bounds__(YZ_THREADS, 4) k_sob_yz(const Plan* __restrict
     const Job& J = *P->jobs[j];
     if (!J.precondition) continue;
     int t = it - P->pre[ST_TILE][j];
-    int l = 0, per = 0;
-    for (; l < J.L; ++l) {
+    int l = J.L - 1, per = 0;
+    for (; l >= 0; --l) {
       const int n = J.lev[l].n;
       if (!tile_level(n)) continue;
       per = yz_tiles(n);
       if (t < J.C * per) break;
       t -= J.C * per;
     }
-    if (l >= J.L) continue;
+    if (l < 0) continue;
     const Level& lv = J.lev[l];
     const int c = t / per;
     const int tile = t - c * per;

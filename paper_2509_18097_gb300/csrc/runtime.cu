@@ -127,11 +127,11 @@ struct Shape {
       case JOBS: most = MAXJ; break;
       case ROWS: break;
       case ADJ: most = 16L * sms; break;
-      case PLANES: most = (long)sms * plane_blocks_per_sm(); break;
-      case COLS: most = 3L * sms * plane_blocks_per_sm(); break;
+      case PLANES: most = 16L * sms; break;
+      case COLS: most = 32L * sms; break;
       case ADAM: n = (n + 255) / 256, most = 8L * sms * plane_blocks_per_sm(); break;
-      case XT: most = 12L * sms; break;
-      case YZ: most = 16L * sms; break;
+      case XT:
+      case YZ: most = 256L * sms; break;
     }
     return (int)std::max(1L, std::min(n, most));
   }
