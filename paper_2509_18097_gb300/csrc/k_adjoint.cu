@@ -1,7 +1,7 @@
 // Adjoint of the multi-level trilinear evaluation (chain rule of Eq. 1):
 //   dLoss/dTheta_l[v] = (1/L) sum_{p : v is a corner of p in level l} w_{l,v}(x_p) dLoss/dy_p.
 // The query points x are fixed for a whole frame, so the per-level point -> vertex lists
-// (point id, weight / L) are built once per frame by a counting sort keyed by vertex, and
+// (the point's slot, weight / L) are built once per frame by a counting sort keyed by vertex, and
 // compacted to the vertices that some point touches.  Each step then gathers every active
 // vertex's row (with the Cayley payload, both the dLoss/dz and the dLoss/dt halves).  A row is summed in 64-bit fixed point with a scale chosen from the step's
 // bound on |dLoss/dy| (taken in the assembly kernel): integer addition is associative, so
@@ -81,7 +81,7 @@ __global__ void __launch_bounds__(256) k_csr_fill(Job* __restrict__ Jp, int slot
       for (int c = 0; c < 8; ++c) {
         const int pos = __shfl_sync(0xffffffffu, first[c], g.leader) + g.rank;
         const float w = (c & 1 ? fx : 1.f - fx) * ((c >> 1) & 1 ? fy : 1.f - fy) * (c >> 2 ? fz : 1.f - fz);
-        if (c < K && p >= 0) lv.ent[pos] = make_int2(p, __float_as_int(w * invL));
+        if (c < K && p >= 0) lv.ent[pos] = make_int2(i, __float_as_int(w * invL));
       }
     }
   }
@@ -98,6 +98,11 @@ void launch_csr_build(Job* J, const Job& hJ, cudaStream_t s) {
 
 // ------------------------------------------------------------------------------ per step
 
+// What bounds it: the entries stream from DRAM (38 MB a step at 100k points, 6 us at the copy rate) and
+// the gathers wait on L2.  The point gradients are gathered in slot order, so the points of a cell, which
+// are neighbours in a row, share cache lines: 26.6 + 24.4 us for the two launches at 100k points
+// (28.8 + 26.6 in the points' own order, one after another; side by side they overlap).
+//
 // All levels of all jobs in two launches, side by side in the step.  Rows are summed by groups of
 // 2^adj_lg lanes, set by the plan kernel from the level's mean row length (a few dozen
 // entries per row on 128^3, thousands on 16^3): 32 >> adj_lg rows per warp (k_adjoint), or a whole
@@ -229,7 +234,7 @@ __device__ __forceinline__ void block_row(const Job& J, const Level& lv, int i, 
                                           float isc, long long (*red)[8]) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   RowAcc A;
-  if (live) row_sum<C>(lv, J.gy, J.gz, __ldg(lv.act_ptr + i) + threadIdx.x, __ldg(lv.act_ptr + i + 1), 256, sc, A);
+  if (live) row_sum<C>(lv, J.gys, J.gz, __ldg(lv.act_ptr + i) + threadIdx.x, __ldg(lv.act_ptr + i + 1), 256, sc, A);
   group_sum<C>(A, 32);
   if (lane == 0) {
     red[0][warp] = A.a0; red[1][warp] = A.a1; red[2][warp] = A.a2;
@@ -258,7 +263,7 @@ __device__ __forceinline__ void group_row(const Job& J, const Level& lv, int r, 
   const int lpr = 1 << lg;
   const int sub = lane & (lpr - 1);
   RowAcc A;
-  if (r < na && live) row_sum<C>(lv, J.gy, J.gz, __ldg(lv.act_ptr + r) + sub, __ldg(lv.act_ptr + r + 1), lpr, sc, A);
+  if (r < na && live) row_sum<C>(lv, J.gys, J.gz, __ldg(lv.act_ptr + r) + sub, __ldg(lv.act_ptr + r + 1), lpr, sc, A);
   group_sum<C>(A, lpr);
   if (sub == 0 && r < na) store_row<C>(lv, r, finite, isc, A);
 }

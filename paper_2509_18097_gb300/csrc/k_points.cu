@@ -300,23 +300,35 @@ __global__ void k_assemble(const Plan* __restrict__ P) {
     g.z += wr * from_fx(J.acc[3 * p + 2]);
     if (p < J.V && J.w_iso != 0.f) {
       float ix = 0.f, iy = 0.f, iz = 0.f;
-      for (int k = J.v2e_ptr[p]; k < J.v2e_ptr[p + 1]; ++k) {
-        const int ent = J.v2e[k];
-        const float4 d = J.edge_d[ent >> 1];
-        if (ent & 1) { ix -= d.x; iy -= d.y; iz -= d.z; }
-        else { ix += d.x; iy += d.y; iz += d.z; }
+      const int k1 = J.v2e_ptr[p + 1];
+      for (int k = J.v2e_ptr[p]; k < k1; k += 8) {  // 8 edges at a time, loads before sums
+        int ent[8];
+        float4 d[8];
+#pragma unroll
+        for (int u = 0; u < 8; ++u) ent[u] = k + u < k1 ? __ldg(J.v2e + k + u) : -1;
+#pragma unroll
+        for (int u = 0; u < 8; ++u)
+          if (ent[u] >= 0) d[u] = __ldg(J.edge_d + (ent[u] >> 1));
+#pragma unroll
+        for (int u = 0; u < 8; ++u) {
+          if (ent[u] < 0) break;
+          if (ent[u] & 1) { ix -= d[u].x; iy -= d[u].y; iz -= d[u].z; }
+          else { ix += d[u].x; iy += d[u].y; iz += d[u].z; }
+        }
       }
       g.x += J.w_iso * ix;
       g.y += J.w_iso * iy;
       g.z += J.w_iso * iz;
     }
     J.gy[p] = g;
+    const int slot = J.slot_of[p];
+    J.gys[slot] = g;
     float gm = fmaxf(fabsf(g.x), fmaxf(fabsf(g.y), fabsf(g.z)));
     if (J.C == 6) {  // the point's gradient with respect to its averaged Cayley z
       const float4 z4 = J.zq[p], u4 = J.uq[p];
       const float3 gzv = cayley_grad_z(make_float3(z4.x, z4.y, z4.z), make_float3(u4.x, u4.y, u4.z),
                                        make_float3(g.x, g.y, g.z));
-      J.gz[p] = make_float4(gzv.x, gzv.y, gzv.z, 0.f);
+      J.gz[slot] = make_float4(gzv.x, gzv.y, gzv.z, 0.f);
       gm = fmaxf(gm, fmaxf(fabsf(gzv.x), fmaxf(fabsf(gzv.y), fabsf(gzv.z))));
     }
     // running bound on the point gradients of the job (order-independent max, one atomic per
@@ -474,6 +486,7 @@ __global__ void k_tree_scatter(Job* J) {
       if (!t) {
         const float4 x = J->x[p];
         J->xs[slot] = make_float4(x.x, x.y, x.z, __int_as_float(p));
+        J->slot_of[p] = slot;
       }
     } else {  // padding of the moving sets' last nodes
       const int k = i - M - Q;

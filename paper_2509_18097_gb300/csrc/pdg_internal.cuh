@@ -63,7 +63,7 @@ struct Level {
   int* rowptr;    // [n3 + 1]
   int* act_v;     // [cap] active vertices (ascending)
   int* act_ptr;   // [cap + 1] entry range of each active vertex
-  int2* ent;      // [8 Q] entries: (point, bits of the trilinear weight / L)
+  int2* ent;      // [8 Q] entries: (slot of the point, bits of the trilinear weight / L)
   int* n_active;  // device scalar
   unsigned long long* csum;  // scan scratch
   int adj_lg;     // adjoint: log2 of the lanes per row, 6 = a block per row (set by the plan kernel)
@@ -85,9 +85,10 @@ struct Job {
   float4* gfwd;            // [Q] forward Chamfer gradient
   long long* acc;          // [Q][3] reverse Chamfer sums, fixed point (2^-40)
   float4* gy;              // [Q] dLoss/dy (= dLoss/dt with the Cayley payload)
+  float4* gys;             // [slots of mov] the same in slot order, which the adjoint gathers from
   float4* zq;              // [Q] Cayley payload: the point's averaged z (null otherwise)
   float4* uq;              // [Q] Cayley payload: u = (I - Z)^{-1} x, so that R(z) x = 2 u - x
-  float4* gz;              // [Q] Cayley payload: dLoss/dz of the point
+  float4* gz;              // [slots of mov] Cayley payload: dLoss/dz of the point, in slot order
   float* loss_fwd;         // [Q] phi(d^2) of each forward query
   float* loss_rev;         // [2 max_pts] phi(d^2) of each reverse query (set 0 then set 1)
   float* loss_iso;         // [E] |r_e|
@@ -103,6 +104,7 @@ struct Job {
   float4* verts4;          // [V] current deformed template X_{t-1}
   Tree tgt;                // target points, built per frame
   Tree mov;                // two sets (template, source): order of the frame's x, boxes of the step's y
+  int* slot_of;            // [Q] slot of a point
   float4* xs;              // [slots of mov] undeformed point and its index (bits) in slot order
   float* loss_part;        // [loss chunks][5] partial sums
   unsigned* gmax;          // max |dLoss/dy| component of the step (float bits; sets the adjoint's fixed-point scale)

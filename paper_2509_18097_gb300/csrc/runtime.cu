@@ -293,7 +293,7 @@ struct Layout {
     size_t hist, off, keys, csum, perm, pts, lbox, nbox, sbox;
     int bits;
   } tgt, mov;
-  size_t xs, step, bias, loss, status, loss_part, gmax, counters;
+  size_t xs, slot_of, gys, step, bias, loss, status, loss_part, gmax, counters;
   size_t nbr, coef, bar;
   size_t mesh;  // template-mesh fit: 7 float4 [V] arrays (gradient copy, solves, Adam moments)
 };
@@ -341,7 +341,10 @@ Layout make_layout(const pdg_config& c, int V, int E, int max_pts) {
   L.gy = a.take<float4>(Q);
   L.zq = a.take<float4>(C == 6 ? Q : 1);
   L.uq = a.take<float4>(C == 6 ? Q : 1);
-  L.gz = a.take<float4>(C == 6 ? Q : 1);
+  const int vn = (V + NODE - 1) / NODE, pn = (max_pts + NODE - 1) / NODE;
+  const size_t slots = (size_t)(vn + pn) * NODE;
+  L.gz = a.take<float4>(C == 6 ? slots : 1);
+  L.gys = a.take<float4>(slots);
   L.acc = a.take<long long>(3 * (size_t)Q);
   L.loss_fwd = a.take<float>(Q);
   L.loss_rev = a.take<float>(2 * (size_t)max_pts);
@@ -369,10 +372,10 @@ Layout make_layout(const pdg_config& c, int V, int E, int max_pts) {
     t.nbox = a.take<float4>((size_t)nodes * 2);
     t.sbox = a.take<float4>(((size_t)nodes / 32 + 2) * 2);
   };
-  const int vn = (V + NODE - 1) / NODE, pn = (max_pts + NODE - 1) / NODE;
   tree(L.tgt, 1, max_pts, max_pts, pn);
   tree(L.mov, 2, std::max(V, max_pts), Q, vn + pn);
-  L.xs = a.take<float4>((size_t)(vn + pn) * NODE);
+  L.xs = a.take<float4>(slots);
+  L.slot_of = a.take<int>(Q);
   L.loss_part = a.take<float>(5 * ((Q + 2 * (size_t)max_pts + std::max(E, 1)) / LOSS_CHUNK + 2));
   L.step = a.take<int>(1);
   L.bias = a.take<float>(2);
@@ -824,6 +827,8 @@ pdg_status pdg_create(const pdg_config* cfg, const float* template_xyz, int n_ve
   tree_init(J.tgt, L.tgt);
   tree_init(J.mov, L.mov);
   J.xs = (float4*)P(L.xs);
+  J.slot_of = (int*)P(L.slot_of);
+  J.gys = (float4*)P(L.gys);
   J.loss_part = (float*)P(L.loss_part);
   J.step = (int*)P(L.step);
   J.bias = (float*)P(L.bias);
