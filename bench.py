@@ -392,8 +392,8 @@ def run_mesh_fit(B, ctx, state0, p0, stream, iters=50):
     B.pdg_load_state(ctx, state0)
     return {"iterations": iters, "ms_per_iteration": ms, "iterations_per_s": 1000.0 / ms,
             "loss_last": st.cd_mesh, "lambda": B.MESH_LAMBDA, "lr": B.MESH_LR,
-            "note": "eager launches: the step's Chamfer kernels on the vertices, two Chebyshev solves "
-                    "of (I + lambda L) (135 one-kernel iterations each at max degree 6), Adam"}
+            "note": "the step's Chamfer kernels on the vertices, then two Chebyshev solves of "
+                    "(I + lambda L) (135 iterations each at max degree 6) and Adam in one cooperative launch"}
 
 
 def main():

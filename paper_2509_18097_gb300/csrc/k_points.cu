@@ -82,7 +82,6 @@ __global__ void k_plan(Plan* P) {
     cnt[ST_PLANE][j] = J->C * p3;
     cnt[ST_COL][j] = cols;
     cnt[ST_ADAM][j] = ad;
-    cnt[ST_JOB][j] = 1;
     cnt[ST_LOSSCH][j] = (J->Q + nrs * J->M + J->E + LOSS_CHUNK - 1) / LOSS_CHUNK;
   }
   __syncthreads();
@@ -574,17 +573,10 @@ void launch_deform(const Job* J, const float* in, float* out, int n, cudaStream_
   k_deform<<<blocks_for(n, 256), 256, 0, s>>>(J, in, out, n);
 }
 
-// channel-planar [C][n3] <-> interleaved [n3][C]
+// channel-planar [C][n3] -> interleaved [n3][C]
 __global__ void k_soa_to_aos(const float* __restrict__ in, float* __restrict__ out, int n3, int C) {
   for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n3; i += gridDim.x * blockDim.x)
     for (int c = 0; c < C; ++c) out[(size_t)C * i + c] = in[(size_t)c * n3 + i];
-}
-__global__ void k_aos_to_soa(const float* __restrict__ in, float* __restrict__ out, int n3, int C) {
-  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n3; i += gridDim.x * blockDim.x)
-    for (int c = 0; c < C; ++c) out[(size_t)c * n3 + i] = in[(size_t)C * i + c];
-}
-void launch_aos_to_soa(const float* in, float* out, int n3, cudaStream_t s, int C) {
-  k_aos_to_soa<<<blocks_for(n3, 256), 256, 0, s>>>(in, out, n3, C);
 }
 void launch_soa_to_aos(const float* in, float* out, int n3, cudaStream_t s, int C) {
   k_soa_to_aos<<<blocks_for(n3, 256), 256, 0, s>>>(in, out, n3, C);
@@ -618,14 +610,6 @@ void launch_pack_theta(const float* in, float4* th, float4* tht, float* m, float
 }
 void launch_unpack_theta(const float4* th, const float4* tht, float* out, int n3, int C, cudaStream_t s) {
   k_unpack_theta<<<blocks_for(n3, 256), 256, 0, s>>>(th, tht, out, n3, C);
-}
-
-__global__ void k_copy_int(const int* __restrict__ in, int* __restrict__ out, int n) {
-  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) out[i] = in[i];
-}
-void launch_aos_to_float4(const float* in, float4* out, int n, cudaStream_t s) { launch_pack4(in, out, n, s); }
-void launch_copy_int(const int* in, int* out, int n, cudaStream_t s) {
-  k_copy_int<<<blocks_for(n, 256), 256, 0, s>>>(in, out, n);
 }
 
 // both trees of the frame: keys + counts, exclusive scans, scatter; the targets' points and boxes (the

@@ -78,7 +78,7 @@ bool on_current_device(const void* p) {
 // one-level job that stops at the preconditioned gradient, and its plan into the scratch
 // array.  Everything comes in as kernel arguments, so the call copies nothing from host
 // memory.  One block.
-__global__ void k_static_setup(unsigned char* base, int n, int lg, float lam, const float* g, float* out) {
+__global__ void k_static_setup(unsigned char* base, int n, float lam, const float* g, float* out) {
   float* mu = reinterpret_cast<float*>(base + SO_MU);
   float2* tw = reinterpret_cast<float2*>(base + SO_TW);
   float2* tw4 = reinterpret_cast<float2*>(base + SO_TW4);
@@ -105,7 +105,6 @@ __global__ void k_static_setup(unsigned char* base, int n, int lg, float lam, co
     J.no_adam = 1;
     Level& lv = J.lev[0];
     lv.n = n;
-    lv.lg = lg;
     lv.n3 = n * n * n;
     lv.lam = lam;
     J.ext_in = g;
@@ -144,9 +143,7 @@ extern "C" pdg_status pdg_precondition_static(int res, float lambda, const float
   if (st != PDG_OK) return st;
   cudaStream_t s = (cudaStream_t)cuda_stream;
   const int n = res;
-  int lg = 0;
-  while ((1 << lg) < n) ++lg;
-  k_static_setup<<<1, 256, 0, s>>>(base, n, lg, lambda, g, out);
+  k_static_setup<<<1, 256, 0, s>>>(base, n, lambda, g, out);
   launch_sobz_pivots(reinterpret_cast<float*>(base + SO_PIV), reinterpret_cast<int*>(base + SO_SLOW),
                      reinterpret_cast<const float*>(base + SO_MU), n, lambda, s);
   Plan* dP = reinterpret_cast<Plan*>(base + SO_PLAN);

@@ -55,7 +55,6 @@ void sobolev_yz_configure();
 void sobolev_plane_configure();
 int plane_smem_bytes(int n);
 int plane_smem_max(int nmax);
-void launch_aos_to_soa(const float* in, float* out, int n3, cudaStream_t s, int C = 3);
 void launch_sobz_pivots(float* piv, int* slow, const float* mu, int n, float lam, cudaStream_t s);
 
 // template-mesh fit (k_mesh.cu)
@@ -80,7 +79,5 @@ cudaError_t launch_mesh_solve(MeshSolve a, float emax, int sms, cudaStream_t s);
 void launch_soa_to_aos(const float* in, float* out, int n3, cudaStream_t s, int C = 3);
 void launch_pack_theta(const float* in, float4* th, float4* tht, float* m, float* v, int n3, int C, cudaStream_t s);
 void launch_unpack_theta(const float4* th, const float4* tht, float* out, int n3, int C, cudaStream_t s);
-void launch_aos_to_float4(const float* in, float4* out, int n, cudaStream_t s);
-void launch_copy_int(const int* in, int* out, int n, cudaStream_t s);
 
 }  // namespace pdg

@@ -39,8 +39,7 @@ struct Tree {
 };
 
 struct Level {
-  int n;       // vertices per axis (1 or a power of two)
-  int lg;      // log2(n)
+  int n;       // vertices per axis: 1 or 2^a 3^b
   int n3;      // n^3
   float sc_hi[3], sc_lo[3];  // (n - 1) / (hi - lo) per axis as a float pair (hi + lo)
   float lr;    // learning rate of the level (already x0.1 without preconditioning)
@@ -122,7 +121,7 @@ struct Job {
 
 enum Counter { CNT_NN_CANDIDATES = 0, CNT_NN_TIES = 1 };
 
-enum Stage { ST_Q = 0, ST_NODE, ST_SUPER, ST_NNF, ST_NNR, ST_E, ST_ADJ, ST_TILE, ST_JOB, ST_ADJROW, ST_LOSSCH, ST_PLANE, ST_COL, ST_ADAM, ST_XTILE, NSTAGE };
+enum Stage { ST_Q = 0, ST_NODE, ST_SUPER, ST_NNF, ST_NNR, ST_E, ST_ADJ, ST_TILE, ST_ADJROW, ST_LOSSCH, ST_PLANE, ST_COL, ST_ADAM, ST_XTILE, NSTAGE };
 
 struct Plan {
   int n_jobs;

@@ -145,12 +145,6 @@ bool valid_res(int n) {
   return n == 1;
 }
 
-int ilog2(int n) {
-  int l = 0;
-  while ((1 << l) < n) ++l;
-  return l;
-}
-
 // Test hook: the next `g_fail_allocs` device allocations of the library report failure.
 std::atomic<int> g_fail_allocs{0};
 
@@ -733,7 +727,6 @@ pdg_status pdg_create(const pdg_config* cfg, const float* template_xyz, int n_ve
     const auto& o = L.lv[l];
     const int n = cfg->res[l];
     lv.n = n;
-    lv.lg = (n & (n - 1)) == 0 ? ilog2(n) : -1;
     lv.n3 = n * n * n;
     lv.lr = (float)(cfg->lr0 * std::pow((double)cfg->lr_growth, l) * (cfg->precondition ? 1.0 : 0.1));
     lv.lam = (float)(cfg->lambda0 * std::pow((double)cfg->lambda_growth, l));
