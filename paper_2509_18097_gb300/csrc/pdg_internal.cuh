@@ -133,8 +133,8 @@ struct Plan {
 // ------------------------------------------------------------------------------ helpers
 
 // Which preconditioner path takes a level of n vertices per axis: powers of two up to 128
-// (and n = 1) take the shared-memory plane path, 256 and the sizes with a factor 3 the
-// line path.
+// (and n = 1) take the shared-memory plane path, 256 (whose plane does not fit) and the sizes with a
+// factor 3 the line path.  Levels 16^3..128^3 together, with Adam: 125 us by planes, 177 us by lines.
 __host__ __device__ __forceinline__ bool tile_level(int n) { return n > 128 || (n & (n - 1)) != 0; }
 
 // Line path: sizes, line pairs of a y or z tile, x-lines (per channel) of an x tile.  A stage
