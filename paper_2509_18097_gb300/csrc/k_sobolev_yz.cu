@@ -87,8 +87,8 @@ __device__ __forceinline__ void yz_tile(const Level& lv, float* t, int tile, flo
   // the inverse's input
   float ma = 0.f, mb = 0.f;
   if (PASS == YZ_Z) {  // the tile's lines are (kx, ky) columns, ky n + kx (padding wraps into range)
-    ma = 1.f + lv.lam * (__ldg(lv.mu + l.a % n) + __ldg(lv.mu + l.a / n % n));
-    mb = 1.f + lv.lam * (__ldg(lv.mu + l.b % n) + __ldg(lv.mu + l.b / n % n));
+    ma = __ldg(lv.mu + l.a % n) + __ldg(lv.mu + l.a / n % n);
+    mb = __ldg(lv.mu + l.b % n) + __ldg(lv.mu + l.b / n % n);
   }
   const float lam = lv.lam, inv_n3 = 1.f / ((float)n * n * n);
 #pragma unroll 1
@@ -108,12 +108,11 @@ __device__ __forceinline__ void yz_tile(const Level& lv, float* t, int tile, flo
       if (two) l.store(nq, xn);
     } else {
       if (PASS == YZ_Z) {
-        // 1 / d^2 of both lines from one division: 1 / da = db / (da db)
+        // a division per line: one shared by both, 1 / da = db / (da db), rounds more often, and its
+        // products leave the range of float (NaN) long before 1 / da^2 does
         auto scale = [&](float m, float2 x) {
-          const float da = fmaf(lam, m, ma), db = fmaf(lam, m, mb);
-          const float r = 1.f / (da * db);
-          const float ia = r * db, ib = r * da;
-          return make_float2(x.x * (ia * ia * inv_n3), x.y * (ib * ib * inv_n3));
+          const float da = fmaf(lam, ma + m, 1.f), db = fmaf(lam, mb + m, 1.f);
+          return make_float2(x.x * (inv_n3 / (da * da)), x.y * (inv_n3 / (db * db)));
         };
         xq = scale(__ldg(lv.mu + q), xq);
         xn = q ? scale(__ldg(lv.mu + nq), xn) : make_float2(0.f, 0.f);

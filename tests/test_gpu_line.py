@@ -33,6 +33,25 @@ def test_random_gradient_matches_eigenbasis(n):
     H.check_close(f"n={n}", out, ref)
 
 
+@pytest.mark.parametrize("lam", [1e20, 1e38])
+@pytest.mark.parametrize("n", [6, 27, 96])
+def test_largest_lambdas_leave_the_mean(n, lam):
+    """Any finite lambda is accepted.  The operator then keeps the constant mode alone (the next factor,
+    (1 + lambda mu)^-2, is below 1e-34), whatever the intermediate products overflow to.  Tolerance as
+    above: the gradient's mean is 1, its deviation 0.1, so the result is as large as the terms."""
+    from paper_2509_18097_gb300 import binding as B
+
+    r = np.random.Generator(np.random.PCG64(n))
+    g = (1.0 + 0.1 * r.standard_normal((n**3, 3))).astype(np.float32)
+    ctx = ctx_for(B, n, lam0=lam)
+    try:
+        out = B.pdg_precondition(ctx, 0, g, np.empty_like(g))
+    finally:
+        B.pdg_destroy(ctx)
+    assert np.isfinite(out).all()
+    H.check_close(f"n={n} lambda={lam}", out, np.broadcast_to(g.astype(np.float64).mean(0), out.shape))
+
+
 @pytest.mark.parametrize("res", [(27, 54), (48, 81)])
 def test_planes_without_active_vertices(res):
     """A frame whose points lie in a thin slab after one that filled the domain: what the first
