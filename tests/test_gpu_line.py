@@ -33,6 +33,22 @@ def test_random_gradient_matches_eigenbasis(n):
     H.check_close(f"n={n}", out, ref)
 
 
+@pytest.mark.parametrize("n,before", [(36, 2.640e-7), (108, 3.193e-7), (162, 3.353e-7), (216, 3.481e-7)])
+def test_error_no_larger_than_before_the_register_transforms(n, before):
+    """Relative RMS error against FP64 of a white gradient; `before`: that of the Stockham transforms in
+    shared memory, which the register transforms replaced, on the same input."""
+    from paper_2509_18097_gb300 import binding as B
+
+    g = np.random.Generator(np.random.PCG64(1000 + n)).standard_normal((n**3, 3)).astype(np.float32)
+    ctx = ctx_for(B, n, lam0=0.25)
+    try:
+        out = B.pdg_precondition(ctx, 0, g, np.empty_like(g))
+    finally:
+        B.pdg_destroy(ctx)
+    ref = O.sobolev_precondition_spectral(g.reshape(n, n, n, 3).astype(np.float64), 0.25).reshape(-1, 3)
+    assert np.sqrt(((out - ref) ** 2).mean() / (ref**2).mean()) <= before
+
+
 @pytest.mark.parametrize("lam", [1e20, 1e38])
 @pytest.mark.parametrize("n", [6, 27, 96])
 def test_largest_lambdas_leave_the_mean(n, lam):
