@@ -243,6 +243,9 @@ const char* pdg_last_error(const pdg_ctx* ctx);
 pdg_status pdg_batch_create(int max_jobs, pdg_batch** out);
 pdg_status pdg_batch_set(pdg_batch* b, pdg_ctx* const* ctxs, int n_jobs);
 pdg_status pdg_batch_step(pdg_batch* b, int n_steps, void* cuda_stream);
+/* Times the batch has captured its step graph: at the first step, and when a membership needs
+ * more blocks or larger levels than any before it (a smaller one never does).  No GPU work. */
+pdg_status pdg_batch_graph_captures(const pdg_batch* b, int* out);
 void pdg_batch_destroy(pdg_batch* b);
 
 /* ---- checkpoint / resume (between frames) ------------------------------------------- */

@@ -100,6 +100,7 @@ _SIGS = {
     "pdg_batch_create": (C.c_int, [C.c_int, C.POINTER(C.c_void_p)]),
     "pdg_batch_set": (C.c_int, [C.c_void_p, C.POINTER(C.c_void_p), C.c_int]),
     "pdg_batch_step": (C.c_int, [C.c_void_p, C.c_int, C.c_void_p]),
+    "pdg_batch_graph_captures": (C.c_int, [C.c_void_p, C.POINTER(C.c_int)]),
     "pdg_batch_destroy": (None, [C.c_void_p]),
     "pdg_state_bytes": (C.c_size_t, [C.c_void_p]),
     "pdg_save_state": (C.c_int, [C.c_void_p, C.c_void_p, C.c_size_t, C.c_void_p]),
@@ -370,6 +371,13 @@ def pdg_batch_set(batch, ctxs):
 
 def pdg_batch_step(batch, n_steps: int = 1, stream=None):
     _check(load().pdg_batch_step(batch, int(n_steps), _stream(stream)))
+
+
+def pdg_batch_graph_captures(batch) -> int:
+    """Times the batch has captured its step graph."""
+    out = C.c_int(0)
+    _check(load().pdg_batch_graph_captures(batch, C.byref(out)))
+    return int(out.value)
 
 
 def pdg_batch_destroy(batch):

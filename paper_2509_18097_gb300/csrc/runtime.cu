@@ -95,17 +95,20 @@ struct Shape {
     nline = std::max(nline, o.nline);
     for (int i = 0; i < N_WORK; ++i) w[i] += o.w[i];
   }
-  // makes this cover `o` too; true if a launch of this shape would have had fewer blocks than one of
-  // `o` (or too little shared memory)
-  bool cover(const Shape& o) {
-    bool more = o.nmax > nmax || o.nline > nline || sms != o.sms;
-    for (int i = 0; i < N_WORK; ++i) more = more || blocks(i) < o.blocks(i);
-    if (!more) return false;
-    sms = o.sms;
+  // makes this cover `o` too: the larger of both in every quantity, so once covered, `o` changes nothing
+  void cover(const Shape& o) {
+    sms = std::max(sms, o.sms);
     nmax = std::max(nmax, o.nmax);
     nline = std::max(nline, o.nline);
     for (int i = 0; i < N_WORK; ++i) w[i] = std::max(w[i], o.w[i]);
-    return true;
+  }
+  // whether a step of this shape launches what one of `o` does.  (blocks() alone does not order shapes:
+  // a small one has more lanes per query, a larger nmax a smaller cap.)
+  bool same_launches(const Shape& o) const {
+    bool same = sms == o.sms && nmax == o.nmax && nline == o.nline && nn_sub() == o.nn_sub() &&
+                (w[PLANES] > 0) == (o.w[PLANES] > 0);
+    for (int i = 0; i < N_WORK; ++i) same = same && blocks(i) == o.blocks(i);
+    return same;
   }
 
   // Lanes per query of the searches: 8 while that leaves no more than 32 warps per SM (a warp's own
@@ -255,7 +258,8 @@ struct pdg_batch {
   std::vector<unsigned long long> gens;  // members' frame_gen when dplan's prefixes were computed
   Streams cap;  // of the capture
   cudaGraphExec_t gexec = nullptr;
-  Shape graph_shape;  // what gexec was captured for
+  Shape graph_shape;  // what gexec covers
+  int captures = 0;
   bool dirty = true;  // membership changed since the last upload of the job table
   std::string err;
 };
@@ -1390,18 +1394,28 @@ pdg_status pdg_batch_step(pdg_batch* b, int n_steps, void* cuda_stream) {
     b->gens.resize(b->members.size());
     for (size_t i = 0; i < b->members.size(); ++i) b->gens[i] = b->members[i]->frame_gen;
   }
+  // the graph is captured for the largest of every quantity so far: again only when that grows past
+  // what its launches have
   Shape need = b->graph_shape;
-  if (need.cover(sh) || !b->gexec) {
+  need.cover(sh);
+  if (!b->gexec || !need.same_launches(b->graph_shape)) {
     if (b->gexec) cudaGraphExecDestroy(b->gexec);
     b->gexec = nullptr;
     if (cudaStreamSynchronize(s) != cudaSuccess) return PDG_ERR_CUDA;
     const pdg_status st = capture_step(nullptr, b->dplan, need, b->cap, &b->gexec, &b->err);
     if (st != PDG_OK) return st;
-    b->graph_shape = need;
+    ++b->captures;
   }
+  b->graph_shape = need;
   for (int i = 0; i < n_steps; ++i)
     if (cudaGraphLaunch(b->gexec, s) != cudaSuccess) return PDG_ERR_CUDA;
   for (auto* c : b->members) c->steps_in_frame += n_steps;
+  return PDG_OK;
+}
+
+pdg_status pdg_batch_graph_captures(const pdg_batch* b, int* out) {
+  if (!b || !out) return PDG_ERR_INVALID;
+  *out = b->captures;
   return PDG_OK;
 }
 

@@ -92,6 +92,41 @@ def test_batch_membership_changes():
     B.pdg_batch_destroy(b)
 
 
+def test_draining_batch_keeps_its_graph():
+    """A batch captured for many members serves fewer of them with the same graph.  Three sequences of
+    2562 vertices and 2500 points search with fewer lanes per query than one does, so the one alone would
+    ask for more blocks than the graph has; a member of finer levels leaves less room per SM for Adam."""
+    from paper_2509_18097_gb300 import binding as B
+
+    ws = [job(20 + i, sub=4, n_src=2500, n_tgt=2500, res=(8, 16, 32)) for i in range(3)]
+    ws.append(job(23, sub=1, n_src=300, n_tgt=300, res=(8, 128)))
+    ref = [solo(B, w, 9) for w in ws[:1]]
+    ctxs = [make(B, w) for w in ws]
+    b = B.pdg_batch_create(4)
+
+    def step(members, n=1):
+        B.pdg_batch_set(b, members)
+        for _ in range(n):
+            B.pdg_batch_step(b, 1)
+        return B.pdg_batch_graph_captures(b)
+
+    try:
+        assert B.pdg_batch_graph_captures(b) == 0
+        assert step(ctxs[:3]) == 1
+        assert step(ctxs[:1], 3) == 1
+        assert step(ctxs[:3], 1) == 1
+        assert step(ctxs[3:]) == 2  # a larger level
+        assert step(ctxs[:1], 3) == 2
+        assert step(ctxs[:3]) == 2
+        s = snapshot(B, ctxs[0], ws[0])
+        for k in ref[0]:
+            assert np.array_equal(s[k], ref[0][k]), k
+    finally:
+        for c in ctxs:
+            B.pdg_destroy(c)
+        B.pdg_batch_destroy(b)
+
+
 def seq_set(n_seq=4, n_frames=3):
     seqs = []
     for i in range(n_seq):
