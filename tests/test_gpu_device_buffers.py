@@ -75,3 +75,32 @@ def test_grid_loss_same_on_host_and_device_grids():
     assert got[0][0] == got[1][0]
     for a, b in zip(got[0][1:], got[1][1:]):
         assert np.array_equal(a, b)
+
+
+@pytest.mark.parametrize("dev", ["cpu", "cuda"])
+def test_grid_loss_may_be_changed_in_place(dev):
+    import torch
+
+    from paper_2509_18097_gb300 import binding as B
+    from paper_2509_18097_gb300.autograd import grid_loss
+
+    w = small_sphere(seed=73, n_src=300, n_tgt=200)
+    ctx = B.pdg_create(B.pdg_config_default(res=w.res), w.template, w.edges, w.source, max_pts=300)
+    try:
+        B.pdg_begin_frame(ctx, w.target)
+        th = [torch.tensor(t, device=dev, requires_grad=True) for t in w.thetas]
+        grid_loss(ctx, th).backward()
+        plain = [t.grad.clone() for t in th]
+        for t in th:
+            t.grad = None
+        loss = grid_loss(ctx, th)
+        before = loss.item()
+        loss *= 2.0
+        loss += sum((t.double() ** 2).sum() for t in th)
+        loss.backward()
+        assert loss.item() == 2.0 * before + sum((t.detach().double() ** 2).sum() for t in th).item()
+        for t, g in zip(th, plain):  # the regulariser's part is 2 theta; both sums in FP32
+            d = (t.grad - (2.0 * g + 2.0 * t.detach())).abs().max()
+            assert d <= 2.0**-22 * (2.0 * g.abs().max() + 2.0 * t.detach().abs().max())
+    finally:
+        B.pdg_destroy(ctx)
