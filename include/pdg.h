@@ -210,7 +210,9 @@ pdg_status pdg_precondition(pdg_ctx* ctx, int level, const float* g, float* out,
  * max_pts: PDG_ERR_BUDGET).  Between frames only (PDG_ERR_STATE inside
  * a frame); the source cloud and the grids are untouched.  stats (may be NULL): loss_total =
  * cd_mesh = L_mesh of the last iteration (before its update).  Synchronises `cuda_stream`.
- * PDG_ERR_NONFINITE if a loss was NaN/Inf (the vertices are then as the fit left them). */
+ * PDG_ERR_NONFINITE if a loss was NaN/Inf (the vertices are then as the fit left them).
+ * PDG_ERR_TIMEOUT if a wait inside the solves ran out (each is bounded to about half a second):
+ * the vertices are then as they were before the call. */
 pdg_status pdg_fit_mesh(pdg_ctx* ctx, const float* p0_xyz, int n_p0, int n_steps, float lambda, float lr,
                         pdg_fit_stats* stats, void* cuda_stream);
 
@@ -230,6 +232,12 @@ pdg_status pdg_set_debug(pdg_ctx* ctx, int flags);
  * the failing call frees whatever it had already taken.  n <= 0 turns the hook off.
  * Process-wide; no GPU work. */
 void pdg_debug_fail_allocations(int n);
+
+/* Test hook: the waits of this context's mesh solves give up after `looks` looks at the barrier's
+ * count instead of the usual 2^20 (0: the usual), so that callers can exercise their
+ * PDG_ERR_TIMEOUT path: with 1, a block that is not the last to arrive gives up at once.  looks < 0:
+ * PDG_ERR_INVALID.  No GPU work. */
+pdg_status pdg_debug_mesh_wait(pdg_ctx* ctx, int looks);
 
 void pdg_destroy(pdg_ctx* ctx);
 const char* pdg_status_string(pdg_status s);

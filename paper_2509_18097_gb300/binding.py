@@ -95,6 +95,7 @@ _SIGS = {
     "pdg_step_kernel_count": (C.c_int, [C.c_void_p, C.POINTER(C.c_int)]),
     "pdg_destroy": (None, [C.c_void_p]),
     "pdg_debug_fail_allocations": (None, [C.c_int]),
+    "pdg_debug_mesh_wait": (C.c_int, [C.c_void_p, C.c_int]),
     "pdg_status_string": (C.c_char_p, [C.c_int]),
     "pdg_last_error": (C.c_char_p, [C.c_void_p]),
     "pdg_batch_create": (C.c_int, [C.c_int, C.POINTER(C.c_void_p)]),
@@ -320,6 +321,11 @@ def pdg_set_debug(ctx, keep_pgrad: bool = True, count_nn: bool = False):
 def pdg_debug_fail_allocations(n: int):
     """Test hook: the library's next n device allocations fail (PDG_ERR_OOM)."""
     load().pdg_debug_fail_allocations(int(n))
+
+
+def pdg_debug_mesh_wait(ctx, looks: int):
+    """Test hook: the mesh solves of this context give up after `looks` looks at a barrier (0: the usual)."""
+    _check(load().pdg_debug_mesh_wait(ctx, int(looks)), ctx)
 
 
 def pdg_profile_stages() -> int:

@@ -109,18 +109,18 @@ __global__ void k_mesh_adam(float4* __restrict__ x, const float4* __restrict__ g
 // us; 1024 threads a block (half the blocks, 64 registers): 3.4 us; 384 threads: the same.
 constexpr int MS_THREADS = 512;
 
-// All blocks of the grid (co-resident: cooperative launch).  False after about half a second of
-// waiting: the kernel then gives up and the caller reports it.
-__device__ __forceinline__ bool grid_barrier(unsigned* count, unsigned target, int* err) {
+// All blocks of the grid (co-resident: cooperative launch).  False after `limit` looks at the count
+// (MESH_WAIT: about half a second): the kernel then gives up and the caller reports it.
+__device__ __forceinline__ bool grid_barrier(unsigned* count, unsigned target, int limit, int* err) {
   __shared__ int ok;
   __syncthreads();
   if (threadIdx.x == 0) {
     asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(count) : "memory");
     unsigned seen = 0;
-    int spins = 0;
+    int looks = 0;
     do {
       asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(seen) : "l"(count) : "memory");
-    } while (seen < target && ++spins < (1 << 20));
+    } while (seen < target && ++looks < limit);
     ok = seen >= target;
     if (!ok) atomicExch(err, 1);
   }
@@ -138,6 +138,8 @@ __global__ void __launch_bounds__(MS_THREADS) k_mesh_solve(const MeshSolve a) {
   unsigned phase = 0;
   float4* din = a.d0;
   float4* dout = a.d1;
+  // some block gave up: leave the vertices as they are (the whole block decides alike)
+  if (__syncthreads_or(*reinterpret_cast<volatile int*>(a.err))) return;
 #pragma unroll
   for (int k = 0; k < K; ++k) {
     const int i = base + k * MS_THREADS;
@@ -162,7 +164,7 @@ __global__ void __launch_bounds__(MS_THREADS) k_mesh_solve(const MeshSolve a) {
       }
       if (i < V) din[i] = make_float4(d[k][0], d[k][1], d[k][2], 0.f);
     }
-    if (!grid_barrier(a.bar, ++phase * gridDim.x, a.err)) return;
+    if (!grid_barrier(a.bar, ++phase * gridDim.x, a.wait, a.err)) return;
     for (int it = 0; it < a.iters; ++it) {
       const float2 co = __ldg(a.coef + it);
 #pragma unroll
@@ -197,7 +199,7 @@ __global__ void __launch_bounds__(MS_THREADS) k_mesh_solve(const MeshSolve a) {
       float4* t = din;
       din = dout;
       dout = t;
-      if (it + 1 < a.iters && !grid_barrier(a.bar, ++phase * gridDim.x, a.err)) return;
+      if (it + 1 < a.iters && !grid_barrier(a.bar, ++phase * gridDim.x, a.wait, a.err)) return;
     }
   }
 #pragma unroll

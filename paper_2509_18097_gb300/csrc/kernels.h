@@ -58,6 +58,7 @@ int plane_smem_max(int nmax);
 void launch_sobz_pivots(float* piv, int* slow, const float* mu, int n, float lam, cudaStream_t s);
 
 // template-mesh fit (k_mesh.cu)
+constexpr int MESH_WAIT = 1 << 20;  // looks at a grid barrier: about half a second
 void launch_mesh_points(Job* J, int V, cudaStream_t s);
 // (I + lambda L)^{-2} b by two Chebyshev solves, then Adam on x
 struct MeshSolve {
@@ -68,6 +69,7 @@ struct MeshSolve {
   float4 *x, *m, *v;
   float2* coef;          // [iters] constants of the recurrence (mesh_coef)
   unsigned* bar;         // grid barrier
+  int wait;              // looks at the barrier before a block gives up
   int* err;              // set when the barrier's wait ran out
   int V, iters;
   float lam, inv_theta, lr, b1, b2, eps, bias1, ibias2;

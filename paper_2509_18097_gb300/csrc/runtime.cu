@@ -227,6 +227,7 @@ struct pdg_ctx {
   float2* coef = nullptr;  // [MESH_ITERS_MAX] constants of the solves
   unsigned* bar = nullptr; // grid barrier of the solves, and their error flag
   int max_degree = 0;      // largest vertex degree of the mesh (bounds the Laplacian's spectrum)
+  int mesh_wait = MESH_WAIT;  // looks at a barrier of the solves before they give up
   bool mesh_valid = false; // a template-mesh fit has run (PDG_BUF_MESH_* readable)
   float* stage = nullptr;  // [stage_pts][3] staging of host inputs
   int stage_pts = 0;
@@ -1268,6 +1269,7 @@ pdg_status pdg_fit_mesh(pdg_ctx* c, const float* p0_xyz, int n_p0, int n_steps, 
   ms.coef = c->coef;
   ms.bar = c->bar;
   ms.err = reinterpret_cast<int*>(c->bar + 1);
+  ms.wait = c->mesh_wait;
   ms.V = V;
   ms.iters = iters;
   ms.lam = lambda;
@@ -1292,14 +1294,19 @@ pdg_status pdg_fit_mesh(pdg_ctx* c, const float* p0_xyz, int n_p0, int n_steps, 
     ms.ibias2 = (float)(1.0 / std::sqrt(1.0 - std::pow((double)J.beta2, k)));
     CU(c, launch_mesh_solve(ms, (float)emax, c->sms, s));
   }
-  CU(c, cudaMemcpyAsync(J.verts4, J.x, sizeof(float4) * V, cudaMemcpyDeviceToDevice, s));
   double loss[4];
   int status = 0, gave_up = 0;
   CU(c, cudaMemcpyAsync(loss, J.loss, sizeof(loss), cudaMemcpyDeviceToHost, s));
   CU(c, cudaMemcpyAsync(&status, J.status, sizeof(int), cudaMemcpyDeviceToHost, s));
   CU(c, cudaMemcpyAsync(&gave_up, ms.err, sizeof(int), cudaMemcpyDeviceToHost, s));
   CU(c, cudaStreamSynchronize(s));
-  c->mesh_valid = n_steps > 0;
+  // Blocks give up one by one: some of the failing iteration may have updated their vertices.  The
+  // template then stays as it was before the call.
+  if (!gave_up) {
+    CU(c, cudaMemcpyAsync(J.verts4, J.x, sizeof(float4) * V, cudaMemcpyDeviceToDevice, s));
+    CU(c, cudaStreamSynchronize(s));
+  }
+  c->mesh_valid = n_steps > 0 && !gave_up;
   c->plan_stale = true;  // the frame plan is recomputed at the next frame
   const pdg_status st = gave_up ? PDG_ERR_TIMEOUT : status ? PDG_ERR_NONFINITE : PDG_OK;
   if (stats) {
@@ -1317,6 +1324,12 @@ pdg_status pdg_fit_mesh(pdg_ctx* c, const float* p0_xyz, int n_p0, int n_steps, 
 }
 
 // ------------------------------------------------------------------------------ batching
+
+pdg_status pdg_debug_mesh_wait(pdg_ctx* c, int looks) {
+  if (!c || looks < 0) return PDG_ERR_INVALID;
+  c->mesh_wait = looks ? looks : MESH_WAIT;
+  return PDG_OK;
+}
 
 void pdg_debug_fail_allocations(int n) { g_fail_allocs.store(n > 0 ? n : 0); }
 

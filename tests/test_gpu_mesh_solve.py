@@ -29,3 +29,31 @@ def test_hub_and_isolated_vertices():
     v = synth.torus_points(r, 60).astype(np.float32)
     e = np.stack([np.zeros(40, np.int32), np.arange(1, 41, dtype=np.int32)], 1)  # vertices 41..59 have no edge
     M.check_one_step(v, e, cloud(300))
+
+
+def test_wait_that_runs_out_is_a_status_and_leaves_the_template():
+    """40 blocks meet at 270 barriers an iteration; with one look each, the first to arrive gives up."""
+    from paper_2509_18097_gb300 import binding as B
+
+    v, _, e = synth.torus_mesh(200, 100)
+    p0 = cloud()
+    X = lambda c: B.pdg_get_vertices(c, np.empty((len(v), 3), np.float32))  # noqa: E731
+    ctx, fresh = M.make_ctx(B, v, e, p0), M.make_ctx(B, v, e, p0)
+    try:
+        before = X(ctx)
+        B.pdg_debug_mesh_wait(ctx, 1)
+        with pytest.raises(B.PdgError) as ei:
+            B.pdg_fit_mesh(ctx, p0, 3)
+        assert ei.value.status == B.ERR_TIMEOUT
+        assert np.array_equal(X(ctx), before)
+        with pytest.raises(B.PdgError) as ei:
+            B.pdg_read(ctx, B.BUF_MESH_PGRAD, 0, np.empty((len(v), 3), np.float32))
+        assert ei.value.status == B.ERR_STATE
+        B.pdg_debug_mesh_wait(ctx, 0)  # and the context works as before
+        a, b = B.pdg_fit_mesh(ctx, p0, 3), B.pdg_fit_mesh(fresh, p0, 3)
+        assert a.loss_total == b.loss_total
+        assert np.array_equal(X(ctx), X(fresh))
+        assert not np.array_equal(X(ctx), before)
+    finally:
+        B.pdg_destroy(ctx)
+        B.pdg_destroy(fresh)
