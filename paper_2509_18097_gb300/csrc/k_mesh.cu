@@ -106,7 +106,9 @@ __global__ void k_mesh_adam(float4* __restrict__ x, const float4* __restrict__ g
 // the grid's blocks (at most one per SM) after each write; a vertex's neighbours are loaded together.
 // What bounds it: the latency of the barrier and of one gather from L2, 1.9 us an iteration on 50 412
 // vertices (a launch per iteration: 6.5 us, 270 of them).  Neighbours loaded one after another: 2.65
-// us; 1024 threads a block (half the blocks, 64 registers): 3.4 us; 384 threads: the same.
+// us; 1024 threads a block (half the blocks, 64 registers): 3.4 us; 384 threads: the same.  A vertex of
+// 518 edges on 50 400 vertices: 40 us an iteration (its later neighbours one after another: 82; a launch
+// per iteration: 96).
 constexpr int MS_THREADS = 512;
 
 // All blocks of the grid (co-resident: cooperative launch).  False after `limit` looks at the count
@@ -182,11 +184,21 @@ __global__ void __launch_bounds__(MS_THREADS) k_mesh_solve(const MeshSolve a) {
             l[1] += d[k][1] - dj[e].y;
             l[2] += d[k][2] - dj[e].z;
           }
-        for (int e = p0[k] + NB; e < p1[k]; ++e) {
-          const float4 t = __ldcg(din + __ldg(a.nbr + e));
-          l[0] += d[k][0] - t.x;
-          l[1] += d[k][1] - t.y;
-          l[2] += d[k][2] - t.z;
+#pragma unroll 1
+        for (int e0 = p0[k] + NB; e0 < p1[k]; e0 += NB) {  // the others, as many at a time
+          int id[NB];
+#pragma unroll
+          for (int e = 0; e < NB; ++e) id[e] = e0 + e < p1[k] ? __ldg(a.nbr + e0 + e) : -1;
+#pragma unroll
+          for (int e = 0; e < NB; ++e)
+            if (id[e] >= 0) dj[e] = __ldcg(din + id[e]);
+#pragma unroll
+          for (int e = 0; e < NB; ++e)
+            if (id[e] >= 0) {
+              l[0] += d[k][0] - dj[e].x;
+              l[1] += d[k][1] - dj[e].y;
+              l[2] += d[k][2] - dj[e].z;
+            }
         }
 #pragma unroll
         for (int c = 0; c < 3; ++c) {
@@ -236,9 +248,13 @@ static void launch_cheb_solve(const MeshSolve& a, const float4* b, float4* h, do
   }
 }
 
-// vertices per thread of the one-launch form: the fewest that leave at most a block per SM (0: the
-// mesh is too large for it)
-static int mesh_solve_k(int V, int sms) {
+// Vertices per thread of the one-launch form: the fewest that leave at most a block per SM (0: the
+// mesh is too large for it, or has a vertex of so many edges that the others' wait at the barrier
+// could run out while its thread walks them: 0.08 us an edge, so 4096 take 0.3 ms of about 500, where
+// a launch per iteration takes 0.5).
+constexpr int MS_DEGREE = 4096;
+static int mesh_solve_k(int V, int degree, int sms) {
+  if (degree > MS_DEGREE) return 0;
   for (int k = 1; k <= 4; k *= 2)
     if ((V + MS_THREADS * k - 1) / (MS_THREADS * k) <= sms) return k;
   return 0;
@@ -269,7 +285,7 @@ cudaError_t launch_mesh_solve(MeshSolve a, float emax, int sms, cudaStream_t s) 
   // Chebyshev constants for the interval [1, emax] (theta its centre, delta its half-width)
   const double theta = 0.5 * (emax + 1.0), delta = 0.5 * (emax - 1.0);
   a.inv_theta = (float)(1.0 / theta);
-  const int k = mesh_solve_k(a.V, sms);
+  const int k = mesh_solve_k(a.V, a.degree, sms);
   if (k == 0) {
     launch_cheb_solve(a, a.b, a.h, theta, delta, s);
     launch_cheb_solve(a, a.h, a.pg, theta, delta, s);

@@ -72,6 +72,7 @@ struct MeshSolve {
   int wait;              // looks at the barrier before a block gives up
   int* err;              // set when the barrier's wait ran out
   int V, iters;
+  int degree;            // largest of a vertex
   float lam, inv_theta, lr, b1, b2, eps, bias1, ibias2;
 };
 void mesh_coef(std::vector<float2>& coef, int iters, float emax);

@@ -1272,6 +1272,7 @@ pdg_status pdg_fit_mesh(pdg_ctx* c, const float* p0_xyz, int n_p0, int n_steps, 
   ms.wait = c->mesh_wait;
   ms.V = V;
   ms.iters = iters;
+  ms.degree = c->max_degree;
   ms.lam = lambda;
   ms.lr = lr;
   ms.b1 = J.beta1;

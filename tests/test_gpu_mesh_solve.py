@@ -57,3 +57,30 @@ def test_wait_that_runs_out_is_a_status_and_leaves_the_template():
     finally:
         B.pdg_destroy(ctx)
         B.pdg_destroy(fresh)
+
+
+def star(degree):
+    r = np.random.Generator(np.random.PCG64(7))
+    v = synth.torus_points(r, degree + 1).astype(np.float32)
+    return v, np.stack([np.zeros(degree, np.int32), np.arange(1, degree + 1, dtype=np.int32)], 1)
+
+
+@pytest.mark.parametrize("degree", [4096, 4097])
+def test_vertex_with_thousands_of_edges(degree):
+    """Either side of the line beyond which a vertex's edges take longer than the others should wait.
+    The hub's FP32 sum of its edges rounds by sqrt(degree) 6e-8 = 4e-6 of itself, a part of the result's
+    scale after the solve: inside check_one_step's 1e-5."""
+    v, e = star(degree)
+    M.check_one_step(v, e, cloud(500), lam=0.01)
+
+
+def test_no_wait_beside_a_vertex_with_thousands_of_edges():
+    from paper_2509_18097_gb300 import binding as B
+
+    v, e = star(4097)
+    ctx = M.make_ctx(B, v, e, cloud(500))
+    try:
+        B.pdg_debug_mesh_wait(ctx, 1)  # any wait would run out
+        assert B.pdg_fit_mesh(ctx, cloud(500), 1, 0.01).status == B.OK
+    finally:
+        B.pdg_destroy(ctx)
