@@ -239,6 +239,11 @@ void pdg_debug_fail_allocations(int n);
  * PDG_ERR_INVALID.  No GPU work. */
 pdg_status pdg_debug_mesh_wait(pdg_ctx* ctx, int looks);
 
+/* Test hook: the next n cooperative launches of this context's mesh solves count as refused by the
+ * device (as where it gives the process fewer SMs than it has); the solves then take a launch per
+ * iteration, as meshes too large for one launch do.  n <= 0 turns the hook off.  No GPU work. */
+pdg_status pdg_debug_mesh_refuse(pdg_ctx* ctx, int n);
+
 void pdg_destroy(pdg_ctx* ctx);
 const char* pdg_status_string(pdg_status s);
 const char* pdg_last_error(const pdg_ctx* ctx);

@@ -96,6 +96,7 @@ _SIGS = {
     "pdg_destroy": (None, [C.c_void_p]),
     "pdg_debug_fail_allocations": (None, [C.c_int]),
     "pdg_debug_mesh_wait": (C.c_int, [C.c_void_p, C.c_int]),
+    "pdg_debug_mesh_refuse": (C.c_int, [C.c_void_p, C.c_int]),
     "pdg_status_string": (C.c_char_p, [C.c_int]),
     "pdg_last_error": (C.c_char_p, [C.c_void_p]),
     "pdg_batch_create": (C.c_int, [C.c_int, C.POINTER(C.c_void_p)]),
@@ -326,6 +327,11 @@ def pdg_debug_fail_allocations(n: int):
 def pdg_debug_mesh_wait(ctx, looks: int):
     """Test hook: the mesh solves of this context give up after `looks` looks at a barrier (0: the usual)."""
     _check(load().pdg_debug_mesh_wait(ctx, int(looks)), ctx)
+
+
+def pdg_debug_mesh_refuse(ctx, n: int):
+    """Test hook: the next n cooperative launches of this context's mesh solves count as refused."""
+    _check(load().pdg_debug_mesh_refuse(ctx, int(n)), ctx)
 
 
 def pdg_profile_stages() -> int:

@@ -267,6 +267,11 @@ static cudaError_t launch_mesh_coop(MeshSolve a, cudaStream_t s) {
                                      dim3(MS_THREADS), args, 0, s);
 }
 
+// the device will not hold the grid at once (fewer SMs for this context than the device has)
+static bool coop_refused(cudaError_t e) {
+  return e == cudaErrorCooperativeLaunchTooLarge || e == cudaErrorNotSupported || e == cudaErrorLaunchOutOfResources;
+}
+
 // the constants of the recurrence, c1 and c2 of each iteration (lambda = 0: A = I, one iteration)
 void mesh_coef(std::vector<float2>& coef, int iters, float emax) {
   const double theta = 0.5 * (emax + 1.0), delta = 0.5 * (emax - 1.0);
@@ -281,21 +286,26 @@ void mesh_coef(std::vector<float2>& coef, int iters, float emax) {
   }
 }
 
-cudaError_t launch_mesh_solve(MeshSolve a, float emax, int sms, cudaStream_t s) {
+cudaError_t launch_mesh_solve(MeshSolve a, float emax, int sms, int& refuse, cudaStream_t s) {
   // Chebyshev constants for the interval [1, emax] (theta its centre, delta its half-width)
   const double theta = 0.5 * (emax + 1.0), delta = 0.5 * (emax - 1.0);
   a.inv_theta = (float)(1.0 / theta);
   const int k = mesh_solve_k(a.V, a.degree, sms);
-  if (k == 0) {
-    launch_cheb_solve(a, a.b, a.h, theta, delta, s);
-    launch_cheb_solve(a, a.h, a.pg, theta, delta, s);
-    k_mesh_adam<<<mesh_blocks(a.V), 256, 0, s>>>(a.x, a.pg, a.m, a.v, a.V, a.lr, a.b1, a.b2, a.eps, a.bias1, a.ibias2);
-    return cudaGetLastError();
+  if (k > 0) {
+    cudaError_t e = cudaErrorCooperativeLaunchTooLarge;
+    if (refuse > 0) {
+      --refuse;
+    } else {
+      cudaMemsetAsync(a.bar, 0, sizeof(unsigned), s);
+      e = k == 1 ? launch_mesh_coop<1>(a, s) : k == 2 ? launch_mesh_coop<2>(a, s) : launch_mesh_coop<4>(a, s);
+    }
+    if (!coop_refused(e)) return e;
+    cudaGetLastError();
   }
-  cudaMemsetAsync(a.bar, 0, sizeof(unsigned), s);
-  return k == 1   ? launch_mesh_coop<1>(a, s)
-         : k == 2 ? launch_mesh_coop<2>(a, s)
-                  : launch_mesh_coop<4>(a, s);
+  launch_cheb_solve(a, a.b, a.h, theta, delta, s);
+  launch_cheb_solve(a, a.h, a.pg, theta, delta, s);
+  k_mesh_adam<<<mesh_blocks(a.V), 256, 0, s>>>(a.x, a.pg, a.m, a.v, a.V, a.lr, a.b1, a.b2, a.eps, a.bias1, a.ibias2);
+  return cudaGetLastError();
 }
 
 }  // namespace pdg

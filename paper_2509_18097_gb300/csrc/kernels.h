@@ -76,7 +76,8 @@ struct MeshSolve {
   float lam, inv_theta, lr, b1, b2, eps, bias1, ibias2;
 };
 void mesh_coef(std::vector<float2>& coef, int iters, float emax);
-cudaError_t launch_mesh_solve(MeshSolve a, float emax, int sms, cudaStream_t s);
+// refuse: cooperative launches still to be taken as refused (test hook)
+cudaError_t launch_mesh_solve(MeshSolve a, float emax, int sms, int& refuse, cudaStream_t s);
 
 // misc conversions
 void launch_soa_to_aos(const float* in, float* out, int n3, cudaStream_t s, int C = 3);

@@ -228,6 +228,7 @@ struct pdg_ctx {
   unsigned* bar = nullptr; // grid barrier of the solves, and their error flag
   int max_degree = 0;      // largest vertex degree of the mesh (bounds the Laplacian's spectrum)
   int mesh_wait = MESH_WAIT;  // looks at a barrier of the solves before they give up
+  int mesh_refuse = 0;        // cooperative launches of the solves still to be taken as refused
   bool mesh_valid = false; // a template-mesh fit has run (PDG_BUF_MESH_* readable)
   float* stage = nullptr;  // [stage_pts][3] staging of host inputs
   int stage_pts = 0;
@@ -1293,7 +1294,7 @@ pdg_status pdg_fit_mesh(pdg_ctx* c, const float* p0_xyz, int n_p0, int n_steps, 
     // (I + lambda L)^{-2} dL/dX by two solves, then Adam on the vertices
     ms.bias1 = (float)(1.0 / (1.0 - std::pow((double)J.beta1, k)));
     ms.ibias2 = (float)(1.0 / std::sqrt(1.0 - std::pow((double)J.beta2, k)));
-    CU(c, launch_mesh_solve(ms, (float)emax, c->sms, s));
+    CU(c, launch_mesh_solve(ms, (float)emax, c->sms, c->mesh_refuse, s));
   }
   double loss[4];
   int status = 0, gave_up = 0;
@@ -1329,6 +1330,12 @@ pdg_status pdg_fit_mesh(pdg_ctx* c, const float* p0_xyz, int n_p0, int n_steps, 
 pdg_status pdg_debug_mesh_wait(pdg_ctx* c, int looks) {
   if (!c || looks < 0) return PDG_ERR_INVALID;
   c->mesh_wait = looks ? looks : MESH_WAIT;
+  return PDG_OK;
+}
+
+pdg_status pdg_debug_mesh_refuse(pdg_ctx* c, int n) {
+  if (!c) return PDG_ERR_INVALID;
+  c->mesh_refuse = std::max(n, 0);
   return PDG_OK;
 }
 

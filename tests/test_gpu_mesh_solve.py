@@ -84,3 +84,34 @@ def test_no_wait_beside_a_vertex_with_thousands_of_edges():
         assert B.pdg_fit_mesh(ctx, cloud(500), 1, 0.01).status == B.OK
     finally:
         B.pdg_destroy(ctx)
+
+
+def test_refused_cooperative_launch_takes_the_other_form(monkeypatch):
+    """The first iteration refused, and each of a fit's: against the oracle and, over several
+    iterations, within Adam's steps of the one-launch fit (both solve to 1e-7; the sign of a gradient
+    component within rounding of zero may differ, 2 lr a step)."""
+    from paper_2509_18097_gb300 import binding as B
+
+    make = M.make_ctx
+
+    def refusing(*args, **kw):
+        ctx = make(*args, **kw)
+        B.pdg_debug_mesh_refuse(ctx, 1)
+        return ctx
+
+    v, _, e = synth.torus_mesh(60, 30)
+    with monkeypatch.context() as m:
+        m.setattr(M, "make_ctx", refusing)
+        M.check_one_step(v, e, cloud())
+    got = []
+    for n in (0, 2, 5):
+        ctx = make(B, v, e, cloud())
+        try:
+            B.pdg_debug_mesh_refuse(ctx, n)
+            st = B.pdg_fit_mesh(ctx, cloud(), 5)
+            got.append((st.cd_mesh, B.pdg_get_vertices(ctx, np.empty((len(v), 3), np.float32))))
+        finally:
+            B.pdg_destroy(ctx)
+    for loss, x in got[1:]:
+        assert abs(loss - got[0][0]) <= 1e-5 * got[0][0]
+        assert np.abs(x - got[0][1]).max() <= 5 * 2 * M.LR
