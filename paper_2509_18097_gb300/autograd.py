@@ -29,8 +29,8 @@ class GridLoss(torch.autograd.Function):
         dev0 = thetas[0].device
         if dev0.type == "cuda":  # the loss stays on the device: nothing waits for the evaluation
             B.pdg_eval_async(handle)
-            # a tensor of its own: a view made in here could not be changed in place by the caller
-            loss = B.pdg_read(handle, B.BUF_LOSS, 0, torch.empty(4, dtype=torch.float64, device=dev0))[0].clone()
+            # cut to the total in place: a view made in here could not be changed in place by the caller
+            loss = B.pdg_read(handle, B.BUF_LOSS, 0, torch.empty(4, dtype=torch.float64, device=dev0)).resize_(())
         else:
             loss = torch.tensor(B.pdg_eval(handle)[0], dtype=torch.float64, device=dev0)
         grads = []
