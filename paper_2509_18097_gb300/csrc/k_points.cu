@@ -68,7 +68,7 @@ __global__ void k_plan(Plan* P) {
       else aw += (na + (32 >> lg) - 1) >> (5 - lg);
       if (tile_level(J->lev[l].n)) {
         t += J->C * yz_tiles(J->lev[l].n);
-        xt += J->C / 3 * x_tiles(J->lev[l].n);
+        xt += x_tiles(J->lev[l].n);
       } else {
         p3 += J->lev[l].n;
         cols += J->C * ((J->lev[l].n * J->lev[l].n + 63) / 64);  // blocks of 64 columns (two threads each)

@@ -718,7 +718,6 @@ __global__ void __launch_bounds__(256) k_adam(const Plan* __restrict__ P) {
   for (int it = blockIdx.x * blockDim.x + threadIdx.x; it < total; it += gridDim.x * blockDim.x) {
     const int j = find_job(P->pre[ST_ADAM], nj, it);
     const Job& J = *P->jobs[j];
-    if (J.no_adam) continue;
     int l, q;
     if (!adam_item(J, it - P->pre[ST_ADAM][j], l, q)) continue;
     const Level& lv = J.lev[l];

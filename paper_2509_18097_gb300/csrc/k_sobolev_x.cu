@@ -42,9 +42,9 @@ __device__ __forceinline__ void line_load(const float* __restrict__ src, bool in
 
 constexpr int x_smem(int n) { return n * (3 * (x_lines(n) / 2) + 1) * 8; }
 
-// x forward on channels 3 h .. 3 h + 2
+// x forward
 template <int n>
-__device__ __forceinline__ void x_fwd(const Job& J, const Level& lv, int h, int tile, float2* smem, int2 zr) {
+__device__ __forceinline__ void x_fwd(const Job& J, const Level& lv, int tile, float2* smem, int2 zr) {
   using L = XT<n>;
   constexpr int P = L::P, S = L::S, STEP = L::STEP, XL = L::XL, nl = L::nl, N1 = Fac<n>::N1, N2 = Fac<n>::N2;
   const int r0 = tile * XL, tid = thread_here(), lane = tid & 31, warp = tid >> 5;
@@ -60,7 +60,7 @@ __device__ __forceinline__ void x_fwd(const Job& J, const Level& lv, int h, int 
       line_load<3 * n>(src + (size_t)l * 3 * n, r0 + l < nl, lane,
                        [&](int i, float x) { f[L::at(i / 3, i - i / 3 * 3, l)] = x; });
   } else {
-    const float* src = lv.g + (size_t)(3 * h) * lv.n3 + (size_t)r0 * n;
+    const float* src = lv.g + (size_t)r0 * n;
 #pragma unroll 1
     for (int r = warp; r < 3 * XL; r += X_WARPS) {  // a warp per line
       const int c = r / XL, l = r - c * XL;
@@ -89,7 +89,7 @@ __device__ __forceinline__ void x_fwd(const Job& J, const Level& lv, int h, int 
     if (q && 2 * q != n) sm[nq * S] = xn;
   }
   __syncthreads();
-  float* dst = lv.tmp + (size_t)(3 * h) * lv.n3 + (size_t)r0 * n;
+  float* dst = lv.tmp + (size_t)r0 * n;
 #pragma unroll 1
   for (int r = warp; r < 3 * XL; r += X_WARPS) {
     const int c = r / XL, l = r - c * XL;
@@ -98,18 +98,18 @@ __device__ __forceinline__ void x_fwd(const Job& J, const Level& lv, int h, int 
   }
 }
 
-// Adam (PyTorch semantics) on the tile's vertices, channels 3 h .. 3 h + 2, with the gradient in f
+// Adam (PyTorch semantics) on the tile's vertices with the gradient in f
 template <int n>
-__device__ __forceinline__ void adam_tile(const Job& J, const Level& lv, int h, int r0, int tid, const float* f) {
+__device__ __forceinline__ void adam_tile(const Job& J, const Level& lv, int r0, int tid, const float* f) {
   using L = XT<n>;
   const int cnt = min(L::XL, L::nl - r0) * n;
-  const size_t n3 = lv.n3, v0 = (size_t)(3 * h) * n3 + (size_t)r0 * n;
+  const int n3 = lv.n3, v0 = r0 * n;
   const float b1 = J.beta1, b2 = J.beta2, eps = J.eps;
   const float step = lv.lr * J.bias[0], ib2 = J.bias[1];
   const bool pre = J.precondition, keep = J.keep_pgrad && pre;
   float* mp = lv.m + v0;
   float* vp = lv.v + v0;
-  float4* th = (h ? lv.theta_t : lv.theta) + (size_t)r0 * n;
+  float4* th = lv.theta + (size_t)r0 * n;
 #pragma unroll 1
   for (int v = tid; v < cnt; v += X_THREADS) {
     const int l = v / n, e = v - l * n;
@@ -134,13 +134,13 @@ __device__ __forceinline__ void adam_tile(const Job& J, const Level& lv, int h, 
   }
 }
 
-// x inverse on channels 3 h .. 3 h + 2, then Adam (PyTorch semantics)
+// x inverse, then Adam
 template <int n>
-__device__ __forceinline__ void x_inv(const Job& J, const Level& lv, int h, int tile, float2* smem) {
+__device__ __forceinline__ void x_inv(const Job& J, const Level& lv, int tile, float2* smem) {
   using L = XT<n>;
   constexpr int P = L::P, S = L::S, STEP = L::STEP, XL = L::XL, nl = L::nl, N1 = Fac<n>::N1, N2 = Fac<n>::N2;
   const int r0 = tile * XL, tid = thread_here(), lane = tid & 31, warp = tid >> 5;
-  const size_t n3 = lv.n3, v0 = (size_t)(3 * h) * n3 + (size_t)r0 * n;
+  const size_t n3 = lv.n3, v0 = (size_t)r0 * n;
   float* f = reinterpret_cast<float*>(smem);
   if (J.precondition) {
     float2* sm = smem + tid % P;
@@ -186,10 +186,11 @@ __device__ __forceinline__ void x_inv(const Job& J, const Level& lv, int h, int 
       }
     return;
   }
-  adam_tile<n>(J, lv, h, r0, tid, f);
+  adam_tile<n>(J, lv, r0, tid, f);
 }
 
-// Items: the tiles of every line-path level of every job, per group of three channels.
+// Items: the tiles of every line-path level of every job (three channels: the Cayley payload takes
+// plane-path levels only).
 template <bool FWD>
 __global__ void __launch_bounds__(X_THREADS, 3) k_sob_x(const Plan* __restrict__ P) {
   extern __shared__ float2 smx[];
@@ -206,23 +207,21 @@ __global__ void __launch_bounds__(X_THREADS, 3) k_sob_x(const Plan* __restrict__
       const int n = J.lev[l].n;
       if (!tile_level(n)) continue;
       per = x_tiles(n);
-      if (t < J.C / 3 * per) break;
-      t -= J.C / 3 * per;
+      if (t < per) break;
+      t -= per;
     }
     if (l < 0) continue;
     const Level& lv = J.lev[l];
-    const int h = t / per;
-    const int tile = t - h * per;
     __syncthreads();  // the previous item is done with the shared arrays
     if (FWD) {
       z_range(lv, &zrange);
       __syncthreads();
     }
     switch (lv.n) {
-#define PDG_CASE(N)                                    \
-  case N:                                              \
-    if (FWD) x_fwd<N>(J, lv, h, tile, smx, zrange);      \
-    else x_inv<N>(J, lv, h, tile, smx);                \
+#define PDG_CASE(N)                           \
+  case N:                                     \
+    if (FWD) x_fwd<N>(J, lv, t, smx, zrange); \
+    else x_inv<N>(J, lv, t, smx);             \
     break;
       PDG_LINE_SIZES(PDG_CASE)
 #undef PDG_CASE

@@ -16,7 +16,7 @@ namespace pdg {
 constexpr int STATIC_MAX_RES = PDG_STATIC_MAX_RES;
 constexpr size_t STATIC_N3 = (size_t)STATIC_MAX_RES * STATIC_MAX_RES * STATIC_MAX_RES;
 // layout: tmp (3 n^3 floats) | z-solve pivots ((n/2 + 1) n^2) | mu (n) | tw (n float2) | tw4 (n float2) |
-//         n_active (int) + bias (2 floats, read by the pass even when it skips Adam) | pivot flag | job | plan
+//         n_active (int) | pivot flag (int) | job | plan
 constexpr size_t SO_TMP = 0;
 constexpr size_t SO_PIV = SO_TMP + 3 * STATIC_N3 * sizeof(float);
 constexpr size_t SO_MU =
@@ -24,8 +24,7 @@ constexpr size_t SO_MU =
 constexpr size_t SO_TW = SO_MU + STATIC_MAX_RES * sizeof(float);
 constexpr size_t SO_TW4 = SO_TW + STATIC_MAX_RES * sizeof(float2);
 constexpr size_t SO_NA = SO_TW4 + STATIC_MAX_RES * sizeof(float2);
-constexpr size_t SO_SLOW = SO_NA + 4 * sizeof(int);  // after n_active and the two bias floats
-constexpr size_t SO_BIAS = SO_NA + sizeof(int);
+constexpr size_t SO_SLOW = SO_NA + sizeof(int);
 constexpr size_t SO_JOB = (SO_SLOW + sizeof(int) + 255) & ~size_t(255);
 constexpr size_t SO_PLAN = (SO_JOB + sizeof(Job) + 255) & ~size_t(255);
 constexpr size_t SO_BYTES = (SO_PLAN + sizeof(Plan) + 255) & ~size_t(255);
@@ -101,8 +100,6 @@ __global__ void k_static_setup(unsigned char* base, int n, float lam, const floa
     J.L = 1;
     J.C = 3;
     J.precondition = 1;
-    J.keep_pgrad = 1;
-    J.no_adam = 1;
     Level& lv = J.lev[0];
     lv.n = n;
     lv.n3 = n * n * n;
@@ -117,8 +114,6 @@ __global__ void k_static_setup(unsigned char* base, int n, float lam, const floa
     lv.tw4 = tw4;
     lv.n_active = reinterpret_cast<int*>(base + SO_NA);
     *lv.n_active = 0;
-    J.bias = reinterpret_cast<float*>(base + SO_BIAS);
-    J.bias[0] = J.bias[1] = 1.f;
     Plan& P = *reinterpret_cast<Plan*>(base + SO_PLAN);
     P.n_jobs = 1;
     P.jobs[0] = &J;

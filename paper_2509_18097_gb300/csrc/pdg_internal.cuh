@@ -75,7 +75,6 @@ struct alignas(16) Job {
   float lo[3], hi[3];
   float alpha, w_mesh, w_pts, w_iso;
   int stopgrad, precondition, keep_pgrad;
-  int no_adam;             // 1: pass C stores the preconditioned gradient and skips Adam
   float beta1, beta2, eps;
   int V, N, M, E, Q;       // template verts, source pts, target pts, edges, V + N
   int max_pts;
@@ -146,19 +145,15 @@ __host__ __device__ __forceinline__ bool tile_level(int n) { return n > 128 || (
 // 16 points or fewer, but for 162, 216 (18) and 243 (27)
 __host__ __device__ constexpr int line_n1(int n) {
   return n <= 6      ? 1
-         : n == 8    ? 2
          : n <= 12   ? 3
-         : n == 16   ? 4
          : n == 18   ? 3
          : n == 24   ? 4
          : n == 27   ? 3
-         : n == 32   ? 4
          : n <= 54   ? 6
          : n <= 72   ? 8
          : n == 81   ? 9
          : n == 96   ? 8
          : n == 108  ? 9
-         : n == 128  ? 8
          : n == 144  ? 12
          : n == 162  ? 9
          : n <= 216  ? 12

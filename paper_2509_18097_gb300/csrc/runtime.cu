@@ -81,7 +81,7 @@ struct Shape {
     w[ROWS] += std::min(rows, 8 * Q / 512 + 1);
     w[ADJ] += (8 * Q / 256 + rows / 32 + 1 + 7) / 8;
     if (line_size((int)n)) {
-      w[XT] += C / 3 * x_tiles((int)n);
+      w[XT] += x_tiles((int)n);
       w[YZ] += C * yz_tiles((int)n);
     } else {
       w[PLANES] += C * n;
@@ -1180,15 +1180,13 @@ pdg_status pdg_precondition(pdg_ctx* c, int level, const float* g, float* out, v
   const float* gin = direct_g ? g : tmp;
   float* gout = direct_out ? out : tmp;
   const bool line = line_size(lv.n) > 0;
-  // a one-level copy of the job that stores the preconditioned gradient instead of Adam
+  // a one-level copy of the job, for the passes without Adam
   Job oj = c->h;
   oj.L = 1;
   oj.C = 3;  // the entry point preconditions 3 channels whatever the payload
   oj.lev[0] = lv;
   oj.lev[0].zmask = nullptr;  // a caller's gradient may be non-zero on any plane
   oj.precondition = 1;
-  oj.keep_pgrad = 1;
-  oj.no_adam = 1;
   oj.ext_in = gin;  // the passes read and write [n^3][3] themselves
   oj.ext_out = gout;
   launch_op_plan(oj, c->op_job, c->op_plan, s);
