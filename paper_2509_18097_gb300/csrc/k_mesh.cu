@@ -3,8 +3,9 @@
 // The robust Chamfer search and gradient are the step's own kernels, run on a job record
 // whose query points are the mesh vertices alone (no source set, no isometry term).  The
 // vertex gradient is then preconditioned by (I + lambda L)^{-2}, L the combinatorial graph
-// Laplacian of the mesh edges, by two Chebyshev solves (no inner products, one kernel per
-// iteration), and Adam moves the vertices.
+// Laplacian of the mesh edges, by two Chebyshev solves (no inner products), and Adam moves the
+// vertices: both in one cooperative launch (k_mesh_solve), or with a launch per Chebyshev iteration
+// where that does not fit.
 #include "kernels.h"
 
 namespace pdg {
@@ -224,9 +225,20 @@ __global__ void __launch_bounds__(MS_THREADS) k_mesh_solve(const MeshSolve a) {
   }
 }
 
+// The fitted vertices become the template, unless a solve gave up: blocks give up one by one, so some
+// of that iteration may have moved their vertices.
+__global__ void k_mesh_commit(const float4* __restrict__ x, float4* __restrict__ verts, int V, const int* __restrict__ err) {
+  if (*err) return;
+  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < V; i += gridDim.x * blockDim.x) verts[i] = x[i];
+}
+
 static inline int mesh_blocks(int n) { return max(1, min((n + 255) / 256, 4096)); }
 
 void launch_mesh_points(Job* J, int V, cudaStream_t s) { k_mesh_points<<<mesh_blocks(V), NODE, 0, s>>>(J); }
+
+void launch_mesh_commit(const MeshSolve& a, float4* verts, cudaStream_t s) {
+  k_mesh_commit<<<mesh_blocks(a.V), 256, 0, s>>>(a.x, verts, a.V, a.err);
+}
 
 static void launch_cheb_solve(const MeshSolve& a, const float4* b, float4* h, double theta, double delta, cudaStream_t s) {
   const int nb = mesh_blocks(a.V);

@@ -75,6 +75,7 @@ struct MeshSolve {
   int degree;            // largest of a vertex
   float lam, inv_theta, lr, b1, b2, eps, bias1, ibias2;
 };
+void launch_mesh_commit(const MeshSolve& a, float4* verts, cudaStream_t s);
 void mesh_coef(std::vector<float2>& coef, int iters, float emax);
 // refuse: cooperative launches still to be taken as refused (test hook)
 cudaError_t launch_mesh_solve(MeshSolve a, float emax, int sms, int& refuse, cudaStream_t s);

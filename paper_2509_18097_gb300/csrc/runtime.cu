@@ -295,7 +295,7 @@ struct Layout {
   } tgt, mov;
   size_t xs, slot_of, gys, step, bias, loss, status, loss_part, gmax, counters;
   size_t nbr, coef, bar;
-  size_t mesh;  // template-mesh fit: 7 float4 [V] arrays (gradient copy, solves, Adam moments)
+  size_t mesh;  // template-mesh fit: 7 float4 [V] arrays (solves, preconditioned gradient, Adam moments)
 };
 
 Layout make_layout(const pdg_config& c, int V, int E, int max_pts) {
@@ -1294,18 +1294,14 @@ pdg_status pdg_fit_mesh(pdg_ctx* c, const float* p0_xyz, int n_p0, int n_steps, 
     ms.ibias2 = (float)(1.0 / std::sqrt(1.0 - std::pow((double)J.beta2, k)));
     CU(c, launch_mesh_solve(ms, (float)emax, c->sms, c->mesh_refuse, s));
   }
+  launch_mesh_commit(ms, J.verts4, s);
+  CU(c, cudaGetLastError());
   double loss[4];
   int status = 0, gave_up = 0;
   CU(c, cudaMemcpyAsync(loss, J.loss, sizeof(loss), cudaMemcpyDeviceToHost, s));
   CU(c, cudaMemcpyAsync(&status, J.status, sizeof(int), cudaMemcpyDeviceToHost, s));
   CU(c, cudaMemcpyAsync(&gave_up, ms.err, sizeof(int), cudaMemcpyDeviceToHost, s));
   CU(c, cudaStreamSynchronize(s));
-  // Blocks give up one by one: some of the failing iteration may have updated their vertices.  The
-  // template then stays as it was before the call.
-  if (!gave_up) {
-    CU(c, cudaMemcpyAsync(J.verts4, J.x, sizeof(float4) * V, cudaMemcpyDeviceToDevice, s));
-    CU(c, cudaStreamSynchronize(s));
-  }
   c->mesh_valid = n_steps > 0 && !gave_up;
   c->plan_stale = true;  // the frame plan is recomputed at the next frame
   const pdg_status st = gave_up ? PDG_ERR_TIMEOUT : status ? PDG_ERR_NONFINITE : PDG_OK;
