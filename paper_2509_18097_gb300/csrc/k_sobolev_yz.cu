@@ -8,11 +8,12 @@
 // eigenvalues mu_k = 4 sin^2(pi k / 2n), so the operator is diagonal in that basis.
 //
 // What bounds them: at 256^3 a pass moves 403 MB (60 us at the copy rate) and takes 92 (y forward),
-// 143 (z) and 122 us (y inverse), at 108^3 13 to 19 us; a warp-per-line Stockham FFT in shared memory
+// 134 (z) and 121 us (y inverse), at 108^3 13 to 19 us; a warp-per-line Stockham FFT in shared memory
 // took 484, 815 and 511 us.  Neither DRAM nor a pipe is full: a block's loads, stages and stores
-// follow one another, so what counts is how many blocks overlap.  64 registers (4 blocks per SM)
-// beat 80 (98, 156, 134 us) and 48 (103, 150, 123 us).  Tiles of 32 line pairs at 32 <= n < 144 beat
-// 16 (108^3: 13, 19, 13 against 15, 22, 15 us), whose stages fill half a block.
+// follow one another, so what counts is how many blocks overlap.  64 registers (4 blocks per SM; 92,
+// 143, 122 us with the z pass of that time) beat 80 (98, 156, 134) and 48 (103, 150, 123).  Tiles of
+// 32 line pairs at 32 <= n < 144 beat 16 (108^3: 13, 19, 13 against 15, 22, 15 us), whose stages fill
+// half a block.
 #include "sobolev_line.cuh"
 
 namespace pdg {
@@ -108,11 +109,13 @@ __device__ __forceinline__ void yz_tile(const Level& lv, float* t, int tile, flo
       if (two) l.store(nq, xn);
     } else {
       if (PASS == YZ_Z) {
-        // a division per line: one shared by both, 1 / da = db / (da db), rounds more often, and its
-        // products leave the range of float (NaN) long before 1 / da^2 does
+        // A division per line: one shared by both, 1 / da = db / (da db), rounds more often, and its
+        // products leave the range of float (NaN) long before 1 / da^2 does.  __fdividef (2 ulp) leaves
+        // the preconditioner's error where an exact division has it (256^3: 3.12e-7 and 3.14e-7 RMS) and
+        // the pass at 134 instead of 147 us; past 2^126 it gives 0, as the quotient nearly is.
         auto scale = [&](float m, float2 x) {
           const float da = fmaf(lam, ma + m, 1.f), db = fmaf(lam, mb + m, 1.f);
-          return make_float2(x.x * (inv_n3 / (da * da)), x.y * (inv_n3 / (db * db)));
+          return make_float2(x.x * __fdividef(inv_n3, da * da), x.y * __fdividef(inv_n3, db * db));
         };
         xq = scale(__ldg(lv.mu + q), xq);
         xn = q ? scale(__ldg(lv.mu + nq), xn) : make_float2(0.f, 0.f);
