@@ -287,7 +287,7 @@ pdg_status pdg_load_state(pdg_ctx* ctx, const void* host_buf, size_t n, void* cu
  *    and sets the kernels' shared-memory limits; make that first call before any stream
  *    capture.
  *  - Every call uses the same array and leaves its contents behind; each call writes its
- *    tables, job record and gradient copy before reading them, so nothing carries over.
+ *    tables, job record and work buffer before reading them, so nothing carries over.
  *    Calls in one process whose work overlaps on the GPU (other streams or threads) race on
  *    the array: serialise them.  (Each process has its own copy of the array.)
  *  - Asynchronous on `cuda_stream`: every table and record is written by a kernel from its

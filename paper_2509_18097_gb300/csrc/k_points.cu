@@ -1,5 +1,5 @@
 // Point- and edge-parallel kernels of the step: the plan, multi-level trilinear
-// evaluation (Eq. 1), the moving-set cell keys, edge isometry (Sec. 3.4), gradient
+// evaluation (Eq. 1), the boxes of the moving trees, edge isometry (Sec. 3.4), gradient
 // assembly and the loss reduction; plus the per-frame set-up kernels.
 #include "kernels.h"
 

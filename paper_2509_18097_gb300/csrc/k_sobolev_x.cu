@@ -7,13 +7,13 @@
 // the loads and stores and along the pairs in the transform stages; the shared rows are padded by
 // one pair, which leaves two lanes to a bank in the former and none shared in the latter.
 //
-// What bounds them: at 256^3 the forward pass takes 74 us inside a frame (planes away from the
-// points are skipped) and 141 us on a dense gradient (403 MB, 60 us at the copy rate; shared-memory
-// wavefronts are 68% of their peak), the inverse with Adam 333 us (1.5 GB, 222 us); a warp-per-line
+// What bounds them: at 256^3 the forward pass takes 67 us inside a frame (planes away from the
+// points are skipped) and 138 us on a dense gradient (403 MB, 60 us at the copy rate; L1 and shared
+// memory are 77% busy), the inverse with Adam 328 us (1.5 GB, 222 us); a warp-per-line
 // FFT with one-channel tiles, whose update touched theta in 4-byte strides, took 500 and about 1200.
 // 56 registers (3 blocks per SM) beat 80 (147 and 162 against 141 and 145 us on a dense gradient);
-// prefetching the moments and theta to L2 before the transform (388 us) and two vertices per thread
-// at a time (338) did not help the update.
+// prefetching the moments and theta to L2 before the transform (388 us), two vertices per thread
+// at a time (338) and 64-bit indices (340) did not help the update.
 #include "sobolev_line.cuh"
 
 namespace pdg {
